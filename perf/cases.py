@@ -146,7 +146,8 @@ def _ortho(X, s, passes=2):
     """X L^{-T} with X^T M X = L L^T."""
     for _ in range(passes):
         Lc = torch.linalg.cholesky(X.T @ _mass(X, s))
-        X = torch.linalg.solve_triangular(Lc, X.T, upper=False).T.contiguous()
+        eye = torch.eye(X.shape[1], dtype=F64, device=DEV)
+        X = X @ torch.linalg.solve_triangular(Lc, eye, upper=False).T
     return X
 
 
@@ -159,10 +160,10 @@ def _block(s, seed):
 def _iterate(s, seed):
     """An M-orthonormal block as the iteration meets it: the seeded start smoothed."""
     X = _block(s, seed)
-    for _ in range(4):
+    for _ in range(2):
         for ax in range(3):
             X = _axis(X, s.N, ax, 0.5, 0.25)
-    return _ortho(X, s)
+    return _ortho(X, s, passes=1)
 
 
 def _jobs(c):
@@ -177,7 +178,8 @@ def _inputs(case, seed):
     st = {}
     if op in ("grad", "grad_of"):
         st["X"] = _iterate(s, seed)
-        st["Xt"] = _ortho(st["X"] + 0.02 * st["X"].abs().max() * _block(s, seed + 1), s)
+        st["Xt"] = _ortho(st["X"] + 0.02 * st["X"].abs().max() * _block(s, seed + 1), s,
+                          passes=1)
     elif op == "retract":
         st["X"] = _iterate(s, seed)
         st["EX"] = _gradient(s, st["X"])[1]
