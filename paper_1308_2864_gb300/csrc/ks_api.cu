@@ -198,15 +198,15 @@ static ks_status project(Problem &P, int retraction, const T *X, const T *EX, co
   const int p = P.p;
   T *G = blk<T>(P, B_G);
   KS_TRY(launch_mass_inverse<T>(P, EX, G));
-  KS_TRY(launch_gram<T>(P, EX, p, X, p, sm(P, S_S)));
+  KS_TRY(launch_gram_sym<T>(P, EX, X, sm(P, S_S)));      // E_X = H(X) X with H symmetric
   KS_TRY(launch_combine<T>(P, X, p, sm(P, S_S), nullptr, 0, nullptr, -1.0, 1.0, G, D, p));
   KS_TRY(launch_mass_dots<T>(P, D, MD, X, MX, prev, P.scal + SC_DNORM2));
   if (retraction == KS_QR) {
-    KS_TRY(launch_gram<T>(P, D, p, MD, p, sm(P, S_DMD)));
+    KS_TRY(launch_gram_sym<T>(P, D, MD, sm(P, S_DMD)));
   } else {
     KS_TRY(launch_transpose(P, sm(P, S_S), sm(P, S_A)));
-    KS_TRY(launch_gram<T>(P, EX, p, G, p, sm(P, S_B)));
-    KS_TRY(launch_gram<T>(P, X, p, MX, p, sm(P, S_O)));
+    KS_TRY(launch_gram_sym<T>(P, EX, G, sm(P, S_B)));
+    KS_TRY(launch_gram_sym<T>(P, X, MX, sm(P, S_O)));
   }
   KS_TRY(sync_scalars(P));
   tr->dnorm2 = P.scal_host[SC_DNORM2];
@@ -226,6 +226,8 @@ static ks_status retract(Problem &P, int retraction, const T *X, const T *D, dou
   const int p = P.p;
   if (retraction == KS_QR) {
     KS_TRY(launch_qr_factor(P, sm(P, S_DMD), nullptr, tau, sm(P, S_C1), sm(P, S_C2)));
+    if constexpr (sizeof(T) == 8)
+      if (update_tri_applies(P)) return launch_update_tri(P, X, D, tau, sm(P, S_C1), Xout);
     KS_TRY(launch_combine<T>(P, X, p, sm(P, S_C1), D, p, sm(P, S_C2), 1.0, 0.0, nullptr, Xout, p));
   } else {
     KS_TRY(launch_cayley_factor(P, sm(P, S_A), sm(P, S_S), sm(P, S_B), sm(P, S_O), tau,
@@ -236,28 +238,40 @@ static ks_status retract(Problem &P, int retraction, const T *X, const T *D, dou
   return KS_OK;
 }
 
-// Cholesky QR in the M inner product, `passes` times; X is updated in place
-// (tmp is an n x p scratch block, MX receives M X of the result).  The Gram
-// and the factor are FP64 in both precisions.
+// Cholesky QR in the M inner product, `passes` times, of the block `in` into X
+// (in may be X; tmp is an n x p scratch block; MX receives M X of the result
+// when final_mx is set, and is scratch otherwise).  The Gram and the factor
+// are FP64 in both precisions.
 template <typename T>
-static ks_status orthonormalize(Problem &P, T *X, T *tmp, T *MX, int passes) {
+static ks_status orthonormalize(Problem &P, const T *in, T *X, T *tmp, T *MX, int passes,
+                                bool final_mx = true) {
   const int p = P.p;
   for (int k = 0; k < passes; ++k) {
-    KS_TRY(launch_mass<T>(P, X, MX));
-    KS_TRY(launch_gram<T>(P, X, p, MX, p, sm(P, S_O)));
+    const T *src = k == 0 ? in : X;
+    KS_TRY(launch_mass<T>(P, src, MX));
+    KS_TRY(launch_gram_sym<T>(P, src, MX, sm(P, S_O)));
     KS_TRY(launch_qr_factor(P, nullptr, sm(P, S_O), 0.0, sm(P, S_C1), nullptr));
-    KS_TRY(launch_combine<T>(P, X, p, sm(P, S_C1), nullptr, 0, nullptr, 1.0, 0.0, nullptr, tmp, p));
-    KS_CUDA_TRY(cudaMemcpyAsync(X, tmp, (size_t)P.n * p * sizeof(T), cudaMemcpyDeviceToDevice,
-                                P.stream));
+    if constexpr (sizeof(T) == 8) {
+      if (update_tri_applies(P)) {
+        KS_TRY(launch_update_tri(P, src, nullptr, 0.0, sm(P, S_C1), X));
+        continue;
+      }
+    }
+    T *dst = src == X ? tmp : X;
+    KS_TRY(launch_combine<T>(P, src, p, sm(P, S_C1), nullptr, 0, nullptr, 1.0, 0.0, nullptr, dst,
+                             p));
+    if (dst != X)
+      KS_CUDA_TRY(cudaMemcpyAsync(X, tmp, (size_t)P.n * p * sizeof(T), cudaMemcpyDeviceToDevice,
+                                  P.stream));
   }
-  KS_TRY(launch_mass<T>(P, X, MX));
+  if (final_mx) KS_TRY(launch_mass<T>(P, X, MX));
   return sync_scalars(P);
 }
 
 // ||X^T M X - I||_F
 template <typename T>
 static ks_status ortho_error(Problem &P, const T *X, const T *MX, double *err) {
-  KS_TRY(launch_gram<T>(P, X, P.p, MX, P.p, sm(P, S_T)));
+  KS_TRY(launch_gram_sym<T>(P, X, MX, sm(P, S_T)));
   KS_TRY(launch_ortho_err(P, sm(P, S_T), P.scal + SC_ORTHO));
   KS_TRY(sync_scalars(P));
   *err = std::sqrt(P.scal_host[SC_ORTHO]);
@@ -329,8 +343,7 @@ static ks_status run_phase(Problem &P, const T *Xstart, T *Xend, const ks_opts &
     KS_TRY(project<T>(P, S.retraction, X(0), EX(0), MX(0), D(0), MD(0),
                       have_prev ? &prev : nullptr, &tr));
   } else {
-    KS_CUDA_TRY(cudaMemcpyAsync(X(0), Xstart, bytes, cudaMemcpyDeviceToDevice, P.stream));
-    KS_TRY(orthonormalize<T>(P, X(0), X(2), MX(0), 2));
+    KS_TRY(orthonormalize<T>(P, Xstart, X(0), X(2), MX(0), 2));
     KS_TRY(evaluate<T>(P, X(0), EX(0), MX(0), &E));
     cg_total = P.last_cg_iters;
     KS_TRY(project<T>(P, o.retraction, X(0), EX(0), MX(0), D(0), MD(0), nullptr, &tr));
@@ -411,7 +424,7 @@ static ks_status run_phase(Problem &P, const T *Xstart, T *Xend, const ks_opts &
       reortho = oerr > ortho_tol;
     }
     if (reortho) {
-      KS_TRY(orthonormalize<T>(P, X(0), X(2), MX(0), 1));
+      KS_TRY(orthonormalize<T>(P, X(0), X(0), X(2), MX(0), 1));
       KS_TRY(evaluate<T>(P, X(0), EX(0), MX(0), &E));
       cg_total += P.last_cg_iters;
     }
@@ -651,7 +664,7 @@ static ks_status rebase_split(Problem &P, int bx, int bmx, int bex, int bxp, int
   KS_TRY(launch_split_join(P, base_hi(P), base_lo(P), lower32(P, bx), xb));
   for (int pass = 0; pass < 2; ++pass) {
     KS_TRY(evaluate<double>(P, xb, w1, w2, E));
-    KS_TRY(launch_gram<double>(P, xb, p, w2, p, sm(P, S_O)));
+    KS_TRY(launch_gram_sym<double>(P, xb, w2, sm(P, S_O)));
     KS_TRY(launch_ortho_err(P, sm(P, S_O), P.scal + SC_ORTHO));
     KS_TRY(sync_scalars(P));
     if (pass == 1 || std::sqrt(P.scal_host[SC_ORTHO]) <= kSplitOrthoTol) break;
@@ -668,7 +681,7 @@ static ks_status rebase_split(Problem &P, int bx, int bmx, int bex, int bxp, int
                               cudaMemcpyDeviceToDevice, P.stream));
   // S_b = E_b^T X_b and D_b = M^{-1} E_b - X_b S_b in FP64
   KS_TRY(launch_mass_inverse<double>(P, w1, w2));
-  KS_TRY(launch_gram<double>(P, w1, p, xb, p, sm(P, S_SB)));
+  KS_TRY(launch_gram_sym<double>(P, w1, xb, sm(P, S_SB)));
   KS_TRY(launch_convert(P, w1, base_eb(P)));
   KS_TRY(launch_combine<double>(P, xb, p, sm(P, S_SB), nullptr, 0, nullptr, -1.0, 1.0, w2, w1, p));
   KS_TRY(launch_convert(P, w1, base_db(P)));
@@ -727,9 +740,7 @@ static ks_status run_phase_split(Problem &P, const double *Xstart, double *Xend,
   } else {
     // FP64 start: X_b = CholQR2(Xstart) in block ix[2], delta = 0
     double *x64 = P.blk[ix[2]];
-    KS_CUDA_TRY(cudaMemcpyAsync(x64, Xstart, (size_t)P.n * p * sizeof(double),
-                                cudaMemcpyDeviceToDevice, P.stream));
-    KS_TRY(orthonormalize<double>(P, x64, P.blk[iex[1]], P.blk[B_G], 2));
+    KS_TRY(orthonormalize<double>(P, Xstart, x64, P.blk[iex[1]], P.blk[B_G], 2, false));
     KS_TRY(launch_split_hilo(P, x64, base_hi(P), base_lo(P)));
     KS_CUDA_TRY(cudaMemsetAsync(lower32(P, ix[0]), 0, (size_t)P.n * p * sizeof(float),
                                 P.stream));
@@ -1126,6 +1137,7 @@ ks_status ks_problem_create(const ks_problem_desc *d, ks_problem **out) {
   if ((st = configure_small_kernels()) != KS_OK) return fail(st);
   if ((st = configure_tc_kernels()) != KS_OK) return fail(st);
   if ((st = configure_blas_kernels()) != KS_OK) return fail(st);
+  if ((st = configure_sym_kernels()) != KS_OK) return fail(st);
   if ((st = launch_setup(P)) != KS_OK) return fail(st);
   if ((st = launch_sine_setup(P)) != KS_OK) return fail(st);
   if ((st = sync_scalars(P)) != KS_OK) return fail(st);
@@ -1147,18 +1159,30 @@ ks_status ks_energy_grad(ks_problem *kp, const double *X, double *E, double *EX,
   Problem &P = kp->P;
   P.state.valid = false;   // the workspace below holds the saved state's blocks
   const size_t bytes = (size_t)P.n * P.p * sizeof(double);
-  double e = 0;
-  KS_TRY(evaluate<double>(P, X, P.blk[B_EX0], P.blk[B_MX0], &e));
-  if (D || gradnorm) {
-    Traces tr;
-    KS_TRY(project<double>(P, KS_QR, X, P.blk[B_EX0], P.blk[B_MX0], P.blk[B_D0], P.blk[B_MD0],
-                           nullptr, &tr));
-    if (gradnorm) *gradnorm = std::sqrt(std::fmax(tr.dnorm2, 0.0));
-    if (D) KS_CUDA_TRY(cudaMemcpyAsync(D, P.blk[B_D0], bytes, cudaMemcpyDeviceToDevice, P.stream));
+  const bool grad = D || gradnorm;
+  double e = 0, dn = 0;
+  // only what the caller asked for is formed: an energy alone stores no
+  // gradient, and M X, M D and D^T M D serve a retraction, not this call
+  KS_TRY(evaluate<double>(P, X, EX || grad ? P.blk[B_EX0] : nullptr, nullptr, &e));
+  if (grad) {
+    const double *Ex = P.blk[B_EX0];
+    double *G = P.blk[B_G], *Dw = P.blk[B_D0];
+    KS_TRY(launch_mass_inverse<double>(P, Ex, G));
+    KS_TRY(launch_gram_sym<double>(P, Ex, X, sm(P, S_S)));
+    KS_TRY(launch_combine<double>(P, X, P.p, sm(P, S_S), nullptr, 0, nullptr, -1.0, 1.0, G, Dw,
+                                  P.p));
+    KS_TRY(launch_mass_dots<double>(P, Dw, nullptr, nullptr, nullptr, nullptr,
+                                    P.scal + SC_DNORM2));
+    KS_TRY(sync_scalars(P));
+    const double d2 = P.scal_host[SC_DNORM2];
+    if (!std::isfinite(d2)) return set_error(KS_ENAN, "non-finite gradient norm");
+    dn = std::sqrt(std::fmax(d2, 0.0));
+    if (D) KS_CUDA_TRY(cudaMemcpyAsync(D, Dw, bytes, cudaMemcpyDeviceToDevice, P.stream));
   }
   if (EX) KS_CUDA_TRY(cudaMemcpyAsync(EX, P.blk[B_EX0], bytes, cudaMemcpyDeviceToDevice, P.stream));
   KS_CUDA_TRY(cudaStreamSynchronize(P.stream));
   *E = e;
+  if (gradnorm) *gradnorm = dn;
   return KS_OK;
 }
 
@@ -1175,11 +1199,30 @@ ks_status ks_retract(ks_problem *kp, int kind, const double *X, const double *EX
   if (Xout == X || Xout == EX) return set_error(KS_EINVAL, "Xout aliases an input");
   Problem &P = kp->P;
   P.state.valid = false;
-  KS_TRY(launch_mass<double>(P, X, P.blk[B_MX0]));
-  Traces tr;
-  KS_TRY(project<double>(P, kind, X, EX, P.blk[B_MX0], P.blk[B_D0], P.blk[B_MD0], nullptr, &tr));
-  KS_TRY(retract<double>(P, kind, X, P.blk[B_D0], tau, P.blk[B_X2]));
-  KS_TRY(sync_scalars(P));
+  const int p = P.p;
+  double *G = P.blk[B_G], *D = P.blk[B_D0], *MD = P.blk[B_MD0], *MX = P.blk[B_MX0];
+  // E_X is the caller's, so E_X^T X need not be symmetric
+  KS_TRY(launch_mass_inverse<double>(P, EX, G));
+  KS_TRY(launch_gram<double>(P, EX, p, X, p, sm(P, S_S)));
+  if (kind == KS_QR) {
+    KS_TRY(launch_combine<double>(P, X, p, sm(P, S_S), nullptr, 0, nullptr, -1.0, 1.0, G, D, p));
+    KS_TRY(launch_mass_dots<double>(P, D, MD, nullptr, nullptr, nullptr, P.scal + SC_DNORM2));
+    KS_TRY(launch_gram_sym<double>(P, D, MD, sm(P, S_DMD)));
+  } else {
+    // the step is written on X and G = M^{-1} E_X (Eq. WY3): no D; the
+    // traces carry any non-finite entry of X or E_X to the check below
+    KS_TRY(launch_mass<double>(P, X, MX));
+    KS_TRY(launch_transpose(P, sm(P, S_S), sm(P, S_A)));
+    KS_TRY(launch_gram_sym<double>(P, EX, G, sm(P, S_B)));
+    KS_TRY(launch_gram_sym<double>(P, X, MX, sm(P, S_O)));
+    KS_TRY(launch_trace_sum(P, sm(P, S_S), sm(P, S_B), sm(P, S_O), P.scal + SC_DNORM2));
+  }
+  KS_TRY(retract<double>(P, kind, X, D, tau, P.blk[B_X2]));
+  const ks_status st = sync_scalars(P);
+  if ((st == KS_OK || st == KS_ENOTPD || st == KS_ESINGULAR) &&
+      !std::isfinite(P.scal_host[SC_DNORM2]))
+    return set_error(KS_ENAN, "non-finite gradient norm");
+  KS_TRY(st);
   KS_CUDA_TRY(cudaMemcpyAsync(Xout, P.blk[B_X2], (size_t)P.n * P.p * sizeof(double),
                               cudaMemcpyDeviceToDevice, P.stream));
   KS_CUDA_TRY(cudaStreamSynchronize(P.stream));
@@ -1193,8 +1236,7 @@ ks_status ks_orthonormalize(ks_problem *kp, double *X) {
   // work on a copy, so that X is left unchanged when the factor fails
   const size_t bytes = (size_t)P.n * P.p * sizeof(double);
   double *W = P.blk[B_X1];
-  KS_CUDA_TRY(cudaMemcpyAsync(W, X, bytes, cudaMemcpyDeviceToDevice, P.stream));
-  KS_TRY(orthonormalize<double>(P, W, P.blk[B_X2], P.blk[B_MX2], 2));
+  KS_TRY(orthonormalize<double>(P, X, W, P.blk[B_X2], P.blk[B_MX2], 2, false));
   KS_CUDA_TRY(cudaMemcpyAsync(X, W, bytes, cudaMemcpyDeviceToDevice, P.stream));
   KS_CUDA_TRY(cudaStreamSynchronize(P.stream));
   return KS_OK;

@@ -256,6 +256,7 @@ ks_status launch_reduce(Problem &P, const double *partials, int nchan, int nb, d
 // Blocks of the grid-stride reduction kernels (their partials are nchan x this).
 int reduce_blocks(const Problem &P, long long work);
 // ks_stencil.cu (T = double or float; sums always returned in FP64)
+// (EX, MX may be null: not stored)
 template <typename T>
 ks_status launch_hamiltonian(Problem &P, const T *X, const double *veff, T *EX, T *MX,
                              double *ekin_out);
@@ -270,7 +271,8 @@ ks_status launch_mass(Problem &P, const T *X, T *MX);
 ks_status launch_hamiltonian_inc(Problem &P, const float *d, const double *veff,
                                  const double *veff_b, const float *xb, const float *eb,
                                  float *e, float *Md, double *dkin_out);
-// MD = M D; dnorm2 = sum D.MD; with prev != null also the BB traces.
+// MD = M D (null, without prev: not stored); dnorm2 = sum D.MD; with
+// prev != null also the BB traces.
 template <typename T>
 struct BBPrevT { const T *X, *MX, *D, *MD; };
 template <typename T>
@@ -283,6 +285,20 @@ ks_status launch_mass_inverse(Problem &P, const T *E, T *G, const T *add = nullp
 // out (pa x qb, FP64) = A^T B with A n x pa, B n x qb (row-major, ld = pa, qb)
 template <typename T>
 ks_status launch_gram(Problem &P, const T *A, int pa, const T *B, int qb, double *out);
+// ks_sym.cu: out (p x p) = A^T B of two n x p blocks whose product is symmetric
+// in exact arithmetic (FP64, 9 <= p <= 128: one triangle computed and
+// mirrored; otherwise the full Gram)
+template <typename T>
+ks_status launch_gram_sym(Problem &P, const T *A, const T *B, double *out);
+// out = (X - tau D) U for upper triangular U (p x p; D may be null: X U);
+// out may be X.  update_tri_applies says for which problems.
+bool update_tri_applies(const Problem &P);
+ks_status launch_update_tri(Problem &P, const double *X, const double *D, double tau,
+                            const double *U, double *out);
+ks_status configure_sym_kernels();
+// Sum of the diagonals of up to three p x p matrices (null: skipped) into *out
+ks_status launch_trace_sum(Problem &P, const double *A, const double *B, const double *C,
+                           double *out);
 // FP32: out = A1^T B1 + A2^T B2 (one pass when the pipelined kernel applies;
 // otherwise two Grams, tmp a p x p scratch matrix)
 ks_status launch_gram_pair(Problem &P, const float *A1, const float *B1, const float *A2,

@@ -169,6 +169,7 @@ void oob_read_minv(unsigned long long *, int *);
 void oob_read_cg(unsigned long long *, int *);
 void oob_read_split(unsigned long long *, int *);
 void oob_read_tc(unsigned long long *, int *);
+void oob_read_sym(unsigned long long *, int *);
 }  // namespace ks
 #endif
 
@@ -187,7 +188,8 @@ extern "C" int ks_debug_bounds(unsigned long long *count, const char **file, int
                             {"ks_minv.cu", ks::oob_read_minv},
                             {"ks_cg.cu", ks::oob_read_cg},
                             {"ks_split.cu", ks::oob_read_split},
-                            {"ks_tc.cu", ks::oob_read_tc}};
+                            {"ks_tc.cu", ks::oob_read_tc},
+                            {"ks_sym.cu", ks::oob_read_sym}};
   for (const Reader &r : readers) {
     unsigned long long c = 0;
     int l = 0;

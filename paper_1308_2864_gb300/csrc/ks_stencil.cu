@@ -202,7 +202,7 @@ __device__ __forceinline__ void stencil_plain_body(const StArgs &a, int vb) {
         const T m = m0 * centre + mf * faces + me * edges + mc * corners;
         if (Kind == SK_HAM) {
           const T kx = k0 * centre + ke * edges + kc * corners;
-          ((T *)a.out1)[idx] = kin * kx + vscale * (T)a.veff[k] * centre;
+          if (a.out1) ((T *)a.out1)[idx] = kin * kx + vscale * (T)a.veff[k] * centre;
           if (a.out2) ((T *)a.out2)[idx] = m;
           acc0 = fma(centre, kx, acc0);
         } else if (Kind == SK_HAM_INC) {
@@ -220,7 +220,7 @@ __device__ __forceinline__ void stencil_plain_body(const StArgs &a, int vb) {
           acc1 = (sum - acc0) - y;
           acc0 = sum;
         } else {
-          ((T *)a.out1)[idx] = m;
+          if (Kind != SK_MASS_DOT || a.out1) ((T *)a.out1)[idx] = m;
           if (Kind >= SK_MASS_DOT) acc0 = fma(centre, m, acc0);
           if (Kind == SK_MASS_BB) {
             const T dx = ((const T *)a.X)[idx] - ((const T *)a.Xp)[idx];
@@ -446,7 +446,8 @@ __global__ void __launch_bounds__(kStThreads, 2) stencil_tma_kernel(const __grid
           const T m = cf.m0 * centre + cf.mf * faces + cf.me * edges + cf.mc * corners;
           if (Kind == SK_HAM) {
             const T kx = cf.k0 * centre + cf.ke * edges + cf.kc * corners;
-            ((T *)a.out1)[idx] = cf.kin * kx + cf.vscale * vz[ly[r] * Tl::TX + lx[r]] * centre;
+            if (a.out1)
+              ((T *)a.out1)[idx] = cf.kin * kx + cf.vscale * vz[ly[r] * Tl::TX + lx[r]] * centre;
             if (a.out2) ((T *)a.out2)[idx] = m;
             acc0 = fma(centre, kx, acc0);
           } else if (Kind == SK_HAM_INC) {
@@ -464,7 +465,7 @@ __global__ void __launch_bounds__(kStThreads, 2) stencil_tma_kernel(const __grid
             acc1 = (sum - acc0) - y;
             acc0 = sum;
           } else {
-            ((T *)a.out1)[idx] = m;
+            if (Kind != SK_MASS_DOT || a.out1) ((T *)a.out1)[idx] = m;
             if (Kind >= SK_MASS_DOT) acc0 = fma(centre, m, acc0);
             if (Kind == SK_MASS_BB) {
               const T dx = bb[0][r] - bb[2][r];
@@ -652,7 +653,7 @@ ks_status launch_hamiltonian(Problem &P, const T *X, const double *veff, T *EX, 
   a.red_scale = 0.5 * a.kfac;
   const double total = (double)P.n * P.p;
   return stencil_launch<T, SK_HAM>(P, a, 1, 27.0 * total,
-                                   total * sizeof(T) * (MX ? 3 : 2) + 8.0 * P.n);
+                                   total * sizeof(T) * (1 + (EX ? 1 : 0) + (MX ? 1 : 0)) + 8.0 * P.n);
 }
 
 ks_status launch_hamiltonian_inc(Problem &P, const float *d, const double *veff,
@@ -703,7 +704,8 @@ ks_status launch_mass_dots(Problem &P, const T *D, T *MD, const T *X, const T *M
     a.MDp = prev->MD;
     return stencil_launch<T, SK_MASS_BB>(P, a, 4, 31.0 * total, 8.0 * total * sizeof(T));
   }
-  return stencil_launch<T, SK_MASS_DOT>(P, a, 1, 23.0 * total, 2.0 * total * sizeof(T));
+  return stencil_launch<T, SK_MASS_DOT>(P, a, 1, 23.0 * total,
+                                        (MD ? 2.0 : 1.0) * total * sizeof(T));
 }
 
 // ---------------------------------------------------------------- batched

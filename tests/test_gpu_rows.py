@@ -1,0 +1,72 @@
+"""The FP64 row kernels (symmetric Gram, triangular update, row update) through
+the calls that use them, against the oracle, at the edges of their blocks:
+9 and 128 are the ends of the range, 36 and 37 leave whole and ragged blocks of
+four columns, 33 and 127 have an odd row pitch; the grids leave ragged row
+tiles and fewer tiles than SMs.  Tolerance: the parity tests' 1e-12 relative
+for one product, 1e-11 for the products chained behind a Cholesky factor."""
+import numpy as np
+import pytest
+
+import ks_inputs as ki
+from oracle import energy as oe
+from oracle import stiefel as ost
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a, dtype=np.float64)).cuda()
+
+
+def assert_rel(got, want, rel, what):
+    got, want = np.asarray(got), np.asarray(want)
+    err = np.abs(got - want).max() / max(np.abs(want).max(), 1e-300)
+    assert err <= rel, f"{what}: {err:.3e} > {rel:.1e}"
+
+
+@pytest.mark.parametrize("N,p", [(7, 9), (11, 33), (13, 36), (13, 37), (11, 64), (9, 127),
+                                 (11, 128), (9, 130)])
+def test_row_kernels(N, p):
+    import paper_1308_2864_gb300 as ks
+    s = ki.small_system(N=N, L=6.0, natoms=2, p=p, Z=4.0, seed=21 + p)
+    model = oe.Model.from_system(s)
+    P = ks.Problem.from_system(s, cg_tol=1e-13)
+    X0 = s.x0()
+    X = ost.m_orthonormalize(model, X0)
+    Xd = dev(X0)
+    P.orthonormalize(Xd)
+    Xh = Xd.cpu().numpy()
+    assert_rel(Xh, X, 1e-11, "orthonormalize")
+    assert np.linalg.norm(Xh.T @ model.apply_M(Xh) - np.eye(p)) <= 1e-12 * np.sqrt(p)
+    pt = ost.point_at(model, X)
+    E, EX, D, g = P.energy_grad(dev(X), want_ex=True, want_d=True)
+    assert abs(E - pt.ev.E) <= 1e-11 * abs(pt.ev.E)
+    assert_rel(EX.cpu().numpy(), pt.ev.EX, 1e-10, "E_X")
+    assert_rel(D.cpu().numpy(), pt.D, 1e-9, "D")
+    assert abs(g - pt.dnorm) <= 1e-9 * pt.dnorm
+    # an energy alone (no gradient stored) is the same energy
+    assert P.energy_grad(dev(X), want_ex=False)[0] == pytest.approx(E, rel=1e-12)
+    for kind, ref in ((ks.KS_QR, ost.retract_qr), (ks.KS_CAYLEY, ost.retract_cayley)):
+        got = P.retract(kind, dev(X), dev(pt.ev.EX), 0.01).cpu().numpy()
+        assert_rel(got, ref(model, pt, 0.01), 1e-11, f"retract {kind}")
+
+
+def test_retract_takes_any_derivative_block():
+    # E_X of a caller need not come from a symmetric H: E_X^T X is then not symmetric
+    import paper_1308_2864_gb300 as ks
+    s = ki.small_system(N=11, L=6.0, natoms=2, p=20, Z=4.0, seed=5)
+    model = oe.Model.from_system(s)
+    X = ost.m_orthonormalize(model, s.x0())
+    ev = oe.evaluate(model, X)
+    ev.EX = np.random.default_rng(3).standard_normal(X.shape)
+    pt = ost.project(model, X, ev)
+    P = ks.Problem.from_system(s)
+    got = P.retract(ks.KS_CAYLEY, dev(X), dev(ev.EX), 1e-3).cpu().numpy()
+    assert_rel(got, ost.retract_cayley(model, pt, 1e-3), 1e-11, "retract")
+    bad = ev.EX.copy()
+    bad[17, 3] = np.nan
+    for kind in (ks.KS_QR, ks.KS_CAYLEY):
+        with pytest.raises(ks.KSError) as e:
+            P.retract(kind, dev(X), dev(bad), 1e-3)
+        assert e.value.status == ks.KS_ENAN
