@@ -61,11 +61,34 @@ struct StTile {
   static constexpr int HX = TX + 2, HY = TY + 2;
 };
 
+// Nodes of a thread.  FP64: consecutive in y, so that the column sums
+// u(x-1, y) + u(x+1, y) of six rows serve the four nodes.  FP32: one of each
+// quarter of the tile, consecutive groups on consecutive nodes.
+template <typename T, int PC>
+__device__ __forceinline__ void st_nodes(int grp, int (&lx)[kStNodesPerThread],
+                                         int (&ly)[kStNodesPerThread]) {
+  using Tl = StTile<PC>;
+  static_assert(Tl::G % Tl::TX == 0 && Tl::G / Tl::TX * kStNodesPerThread == Tl::TY,
+                "the groups' columns tile the block");
+#pragma unroll
+  for (int r = 0; r < kStNodesPerThread; ++r) {
+    if constexpr (sizeof(T) == 8) {
+      lx[r] = grp % Tl::TX;
+      ly[r] = grp / Tl::TX * kStNodesPerThread + r;
+    } else {
+      const int node = grp + r * Tl::G;
+      lx[r] = node % Tl::TX;
+      ly[r] = node / Tl::TX;
+    }
+  }
+}
+
 struct StArgs {
   int N, p, zseg, tiles_x, tiles_y, chunks;
   StencilCoef c;
   double occ, h3;
   double kfac;                // factor of K X in E_X: occ, or mu occ (TFW kinetic)
+  double k0r;                 // k0 / ke
   const void *A;              // input block (X or D)
   void *out1;                 // E_X (SK_HAM) or M A
   void *out2;                 // M X (SK_HAM, optional)
@@ -86,13 +109,116 @@ struct StArgs {
 template <typename T>
 struct StCoefT {
   T k0, ke, kc, m0, mf, me, mc, kin, vscale;
+  T k0r = 0;                  // FP64: k0 / ke
+  bool lumped = false;        // FP64: M = m0 I
   __device__ explicit StCoefT(const StArgs &a) {
     if constexpr (sizeof(T) == 4) {
       k0 = a.cf[0]; ke = a.cf[1]; kc = a.cf[2]; m0 = a.cf[3]; mf = a.cf[4];
       me = a.cf[5]; mc = a.cf[6]; kin = a.cf[7]; vscale = a.cf[8];
     } else {
       k0 = a.c.k0; ke = a.c.ke; kc = a.c.kc; m0 = a.c.m0; mf = a.c.mf;
-      me = a.c.me; mc = a.c.mc; kin = a.kfac; vscale = 2.0 * a.occ * a.h3;
+      me = a.c.me; mc = a.c.mc; vscale = 2.0 * a.occ * a.h3;
+      kin = a.kfac * ke;      // of K A in units of ke
+      k0r = a.k0r;
+      lumped = mc == 0.0;
+    }
+  }
+};
+
+// A thread's running plane sums.  With c, f, e the centre, face and corner
+// sums of a plane, a node's output plane needs
+//   M A = 4 a(z) + a(z-1) + a(z+1),       a = 16 c + 4 f + e   (times mc)
+//   K A = b0(z) + bn(z-1) + bn(z+1),      b0 = (k0/ke) c + e, bn = f + e/2 (times ke)
+// because the Q1 coefficients are products of 1-D ones (mass 4 : 1 per axis;
+// kc = ke/2, no face term in K).  FP64 carries a, b0 and bn from plane to
+// plane: 16.5 FP64 instructions per entry of the Hamiltonian with M X, 8 of
+// the mass alone, against 22 and 15 for the class sums (faces, edges,
+// corners) combined at the output plane.  The FP64 pipe (16 clocks per warp
+// instruction) is the bound of the FP64 stencils, so their time follows that
+// count.  FP32, which is bound by memory, keeps the class sums.
+template <typename T, int Kind>
+struct StCols {
+  static constexpr int R = kStNodesPerThread;
+  static constexpr bool kHam = Kind == SK_HAM || Kind == SK_HAM_INC;
+  static constexpr bool kNew = sizeof(T) == 8;
+  // c: centre; f: a (FP64) or the face sum; e: bn (FP64) or the corner sum; g: b0
+  T c_old[R], c_mid[R], c_new[R], f_old[R], f_mid[R], f_new[R], e_old[R], e_mid[R], e_new[R];
+  T g_mid[R], g_new[R];
+
+  // sums of one staged plane; at(r, dx, dy): value at offset (dx, dy) from node r
+  template <typename At>
+  __device__ __forceinline__ void plane(At at, const StCoefT<T> &cf, bool want_m) {
+    if constexpr (!kNew) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        c_new[r] = at(r, 0, 0);
+        f_new[r] = (at(r, -1, 0) + at(r, 1, 0)) + (at(r, 0, -1) + at(r, 0, 1));
+        e_new[r] = (at(r, -1, -1) + at(r, 1, -1)) + (at(r, -1, 1) + at(r, 1, 1));
+      }
+      return;
+    }
+    T c[R + 2], s[R + 2];
+#pragma unroll
+    for (int y = 0; y < R + 2; ++y) {
+      c[y] = at(0, 0, y - 1);
+      s[y] = at(0, -1, y - 1) + at(0, 1, y - 1);
+    }
+    if constexpr (kHam) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const T f = s[r + 1] + (c[r] + c[r + 2]);
+        const T e = s[r] + s[r + 2];
+        c_new[r] = c[r + 1];
+        if (want_m) f_new[r] = fma((T)16, c[r + 1], fma((T)4, f, e));
+        e_new[r] = fma((T)0.5, e, f);
+        g_new[r] = fma(cf.k0r, c[r + 1], e);
+      }
+    } else {
+#pragma unroll
+      for (int y = 0; y < R + 2; ++y) s[y] = fma((T)4, c[y], s[y]);
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        c_new[r] = c[r + 1];
+        f_new[r] = fma((T)4, s[r + 1], s[r] + s[r + 2]);
+      }
+    }
+  }
+  // M A at node r of the middle plane
+  __device__ __forceinline__ T mass(int r, const StCoefT<T> &cf) const {
+    if constexpr (kNew) {
+      if (cf.lumped) return cf.m0 * c_mid[r];
+      return cf.mc * fma((T)4, f_mid[r], f_old[r] + f_new[r]);
+    } else {
+      const T faces = f_mid[r] + (c_old[r] + c_new[r]);
+      const T edges = e_mid[r] + (f_old[r] + f_new[r]);
+      const T corners = e_old[r] + e_new[r];
+      return fma(cf.mc, corners, fma(cf.me, edges, fma(cf.m0, c_mid[r], cf.mf * faces)));
+    }
+  }
+  // K A, in units of ke for FP64
+  __device__ __forceinline__ T stiff(int r, const StCoefT<T> &cf) const {
+    if constexpr (kNew) {
+      return g_mid[r] + (e_old[r] + e_new[r]);
+    } else {
+      const T edges = e_mid[r] + (f_old[r] + f_new[r]);
+      const T corners = e_old[r] + e_new[r];
+      return fma(cf.kc, corners, fma(cf.k0, c_mid[r], cf.ke * edges));
+    }
+  }
+  __device__ __forceinline__ void shift() {
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      if constexpr (kNew) {
+        c_mid[r] = c_new[r];
+        f_old[r] = f_mid[r]; f_mid[r] = f_new[r];
+        if constexpr (kHam) {
+          e_old[r] = e_mid[r]; e_mid[r] = e_new[r];
+          g_mid[r] = g_new[r];
+        }
+      } else {
+        c_old[r] = c_mid[r]; f_old[r] = f_mid[r]; e_old[r] = e_mid[r];
+        c_mid[r] = c_new[r]; f_mid[r] = f_new[r]; e_mid[r] = e_new[r];
+      }
     }
   }
 };
@@ -121,14 +247,10 @@ __device__ __forceinline__ void stencil_plain_body(const StArgs &a, int vb) {
   const T *A = (const T *)a.A;
 
   int lx[kStNodesPerThread], ly[kStNodesPerThread];
-#pragma unroll
-  for (int r = 0; r < kStNodesPerThread; ++r) {
-    const int node = grp + r * Tl::G;
-    lx[r] = node % Tl::TX;
-    ly[r] = node / Tl::TX;
-  }
-  T c_old[kStNodesPerThread], f_old[kStNodesPerThread], e_old[kStNodesPerThread];
-  T c_mid[kStNodesPerThread], f_mid[kStNodesPerThread], e_mid[kStNodesPerThread];
+  st_nodes<T, PC>(grp, lx, ly);
+  const StCoefT<T> cf(a);
+  const bool want_m = Kind != SK_HAM || sizeof(T) == 4 || a.out2 != nullptr;
+  StCols<T, Kind> sc;
 
   // the halo box of the next plane travels in registers (pf) while the
   // current plane's outputs are formed; plane() stores it to the shared tile
@@ -150,7 +272,7 @@ __device__ __forceinline__ void stencil_plain_body(const StArgs &a, int vb) {
       pf[i] = v;
     }
   };
-  auto plane = [&](T *c, T *f, T *e) {
+  auto plane = [&]() {
     __syncthreads();
 #pragma unroll
     for (int i = 0; i < kPf; ++i) {
@@ -158,69 +280,58 @@ __device__ __forceinline__ void stencil_plain_body(const StArgs &a, int vb) {
       if (t < kBox) tile[t] = pf[i];
     }
     __syncthreads();
-#pragma unroll
-    for (int r = 0; r < kStNodesPerThread; ++r) {
-      const int hx = lx[r] + 1, hy = ly[r] + 1;
-      auto at = [&](int dx, int dy) {
-        const int ti = ((hy + dy) * Tl::HX + hx + dx) * PC + lane;
-        return KS_IN(ti, kBox) ? tile[ti] : (T)0;
-      };
-      c[r] = at(0, 0);
-      f[r] = (at(-1, 0) + at(1, 0)) + (at(0, -1) + at(0, 1));
-      e[r] = (at(-1, -1) + at(1, -1)) + (at(-1, 1) + at(1, 1));
-    }
+    sc.plane(
+        [&](int r, int dx, int dy) {
+          const int ti = ((ly[r] + 1 + dy) * Tl::HX + lx[r] + 1 + dx) * PC + lane;
+          return KS_IN(ti, kBox) ? tile[ti] : (T)0;
+        },
+        cf, want_m);
   };
 
   fetch(z0 - 1);
-  plane(c_old, f_old, e_old);
+  plane();
+  sc.shift();
   fetch(z0);
-  plane(c_mid, f_mid, e_mid);
+  plane();
+  sc.shift();
   if (z0 < z1) fetch(z0 + 1);
 
-  const StCoefT<T> cf(a);
-  const T k0 = cf.k0, ke = cf.ke, kc = cf.kc;
-  const T m0 = cf.m0, mf = cf.mf, me = cf.me, mc = cf.mc;
-  const T kin = cf.kin, vscale = cf.vscale;
   T acc0 = 0, acc1 = 0, acc2 = 0, acc3 = 0;
 
   for (int z = z0; z < z1; ++z) {
-    T c_new[kStNodesPerThread], f_new[kStNodesPerThread], e_new[kStNodesPerThread];
-    plane(c_new, f_new, e_new);                    // plane z + 1
+    plane();                                       // plane z + 1
     if (z + 1 < z1) fetch(z + 2);                  // in flight during the outputs of plane z
 #pragma unroll
     for (int r = 0; r < kStNodesPerThread; ++r) {
       const int gx = x0 + lx[r], gy = y0 + ly[r];
-      const T centre = c_mid[r];
-      const T faces = f_mid[r] + (c_old[r] + c_new[r]);
-      const T edges = e_mid[r] + (f_old[r] + f_new[r]);
-      const T corners = e_old[r] + e_new[r];
+      const T centre = sc.c_mid[r];
       const long long nodes = (long long)N * N * N;
       if (ovalid && gx < N && gy < N && KS_IN(((long long)z * N + gy) * N + gx, nodes) &&
           KS_IN((((long long)z * N + gy) * N + gx) * p + o, nodes * p)) {
         const long long k = ((long long)z * N + gy) * N + gx;
         const long long idx = k * p + o;
-        const T m = m0 * centre + mf * faces + me * edges + mc * corners;
+        const T m = want_m ? sc.mass(r, cf) : (T)0;
         if (Kind == SK_HAM) {
-          const T kx = k0 * centre + ke * edges + kc * corners;
-          if (a.out1) ((T *)a.out1)[idx] = kin * kx + vscale * (T)a.veff[k] * centre;
+          const T kx = sc.stiff(r, cf);
+          if (sizeof(T) == 4 || a.out1) ((T *)a.out1)[idx] = fma(cf.kin, kx, cf.vscale * (T)a.veff[k] * centre);
           if (a.out2) ((T *)a.out2)[idx] = m;
           acc0 = fma(centre, kx, acc0);
         } else if (Kind == SK_HAM_INC) {
-          const T kx = k0 * centre + ke * edges + kc * corners;
+          const T kx = sc.stiff(r, cf);
           const T xb = ((const T *)a.X)[idx], eb = ((const T *)a.MX)[idx];
           const T v = (T)a.veff[k], vb = (T)a.veff_b[k], dv = (T)(a.veff[k] - a.veff_b[k]);
-          ((T *)a.out1)[idx] = kin * kx + vscale * (dv * xb + v * centre);
+          ((T *)a.out1)[idx] = cf.kin * kx + cf.vscale * (dv * xb + v * centre);
           if (a.out2) ((T *)a.out2)[idx] = m;
           // compensated sum of delta . (2 f K X_b + f K delta); acc1 holds the
           // running rounding error
-          const T fkxb = eb - vscale * vb * xb;
-          const T t = centre * ((T)2 * fkxb + kin * kx);
+          const T fkxb = eb - cf.vscale * vb * xb;
+          const T t = centre * ((T)2 * fkxb + cf.kin * kx);
           const T y = t - acc1;
           const T sum = acc0 + y;
           acc1 = (sum - acc0) - y;
           acc0 = sum;
         } else {
-          if (Kind != SK_MASS_DOT || a.out1) ((T *)a.out1)[idx] = m;
+          if (Kind != SK_MASS_DOT || sizeof(T) == 4 || a.out1) ((T *)a.out1)[idx] = m;
           if (Kind >= SK_MASS_DOT) acc0 = fma(centre, m, acc0);
           if (Kind == SK_MASS_BB) {
             const T dx = ((const T *)a.X)[idx] - ((const T *)a.Xp)[idx];
@@ -233,11 +344,11 @@ __device__ __forceinline__ void stencil_plain_body(const StArgs &a, int vb) {
           }
         }
       }
-      c_old[r] = c_mid[r]; f_old[r] = f_mid[r]; e_old[r] = e_mid[r];
-      c_mid[r] = c_new[r]; f_mid[r] = f_new[r]; e_mid[r] = e_new[r];
     }
+    sc.shift();
   }
   if (Kind == SK_MASS) return;
+  if (Kind == SK_HAM && StCols<T, Kind>::kNew) acc0 *= cf.ke;
   const double s0 =
       block_sum(Kind == SK_HAM_INC ? (double)acc0 - (double)acc1 : (double)acc0, smem);
   if (threadIdx.x == 0) a.part[vb] = s0;
@@ -348,16 +459,13 @@ __global__ void __launch_bounds__(kStThreads, 2) stencil_tma_kernel(const __grid
     for (int q = 0; q < kStStages && q < nplanes; ++q) load_stage(q);
 
   int lx[kStNodesPerThread], ly[kStNodesPerThread];
-#pragma unroll
-  for (int r = 0; r < kStNodesPerThread; ++r) {
-    const int node = grp + r * Tl::G;
-    lx[r] = node % Tl::TX;
-    ly[r] = node / Tl::TX;
-  }
+  st_nodes<T, PC>(grp, lx, ly);
   // V_eff of plane z0 - 1 + q is read one iteration ahead by the thread that
   // owns the node, converted once and kept in vs[q % 3]
   const int vx = x0 + (int)threadIdx.x % Tl::TX, vy = y0 + (int)threadIdx.x / Tl::TX;
   constexpr bool kHam = Kind == SK_HAM || Kind == SK_HAM_INC;
+  // FP64 keeps 2 f h^3 V_eff: one product per node, not per entry
+  constexpr bool kScaledV = Kind == SK_HAM && sizeof(T) == 8;
   const bool vown = kHam && (int)threadIdx.x < TXY && vx < N && vy < N;
   double vreg = 0.0, vbreg = 0.0;
   const long long nodes = (long long)N * N * N;
@@ -368,14 +476,14 @@ __global__ void __launch_bounds__(kStThreads, 2) stencil_tma_kernel(const __grid
 
   const StCoefT<T> cf(a);
   T acc0 = 0, acc1 = 0, acc2 = 0, acc3 = 0;
-  T c_old[kStNodesPerThread], f_old[kStNodesPerThread], e_old[kStNodesPerThread];
-  T c_mid[kStNodesPerThread], f_mid[kStNodesPerThread], e_mid[kStNodesPerThread];
+  const bool want_m = Kind != SK_HAM || sizeof(T) == 4 || a.out2 != nullptr;
+  StCols<T, Kind> sc;
   int failed_at = -1;
   for (int q = 0; q < nplanes; ++q) {
     const int zp = z0 - 1 + q;
     const int st = q % kStStages;
     if (kHam && (int)threadIdx.x < TXY) {
-      vs[q % 3][threadIdx.x] = (T)vreg;
+      vs[q % 3][threadIdx.x] = kScaledV ? cf.vscale * (T)vreg : (T)vreg;
       if (Kind == SK_HAM_INC) {
         vbs[q % 3][threadIdx.x] = (T)vbreg;
         dvs[q % 3][threadIdx.x] = (T)(vreg - vbreg);
@@ -389,18 +497,12 @@ __global__ void __launch_bounds__(kStThreads, 2) stencil_tma_kernel(const __grid
     }
     const bool got = mbar_wait_parity(&full[st], (uint32_t)((q / kStStages) & 1));
     const T *tile = ring + st * Rg::STAGE;
-    T c_new[kStNodesPerThread], f_new[kStNodesPerThread], e_new[kStNodesPerThread];
-#pragma unroll
-    for (int r = 0; r < kStNodesPerThread; ++r) {
-      const int hx = lx[r] + 1, hy = ly[r] + 1;
-      auto at = [&](int dx, int dy) {
-        const int ti = ((hy + dy) * Tl::HX + hx + dx) * PC + lane;
-        return KS_IN(ti, Rg::BOX) ? tile[ti] : (T)0;
-      };
-      c_new[r] = at(0, 0);
-      f_new[r] = (at(-1, 0) + at(1, 0)) + (at(0, -1) + at(0, 1));
-      e_new[r] = (at(-1, -1) + at(1, -1)) + (at(-1, 1) + at(1, 1));
-    }
+    sc.plane(
+        [&](int r, int dx, int dy) {
+          const int ti = ((ly[r] + 1 + dy) * Tl::HX + lx[r] + 1 + dx) * PC + lane;
+          return KS_IN(ti, Rg::BOX) ? tile[ti] : (T)0;
+        },
+        cf, want_m);
     if (q >= 2) {
       const int z = zp - 1;
       const T *vz = vs[(q + 2) % 3];
@@ -435,23 +537,22 @@ __global__ void __launch_bounds__(kStThreads, 2) stencil_tma_kernel(const __grid
 #pragma unroll
       for (int r = 0; r < kStNodesPerThread; ++r) {
         const int gx = x0 + lx[r], gy = y0 + ly[r];
-        const T centre = c_mid[r];
-        const T faces = f_mid[r] + (c_old[r] + c_new[r]);
-        const T edges = e_mid[r] + (f_old[r] + f_new[r]);
-        const T corners = e_old[r] + e_new[r];
+        const T centre = sc.c_mid[r];
         if (ovalid && gx < N && gy < N && KS_IN(((long long)z * N + gy) * N + gx, nodes) &&
             KS_IN((((long long)z * N + gy) * N + gx) * p + o, nodes * p)) {
           const long long k = ((long long)z * N + gy) * N + gx;
           const long long idx = k * p + o;
-          const T m = cf.m0 * centre + cf.mf * faces + cf.me * edges + cf.mc * corners;
+          const T m = want_m ? sc.mass(r, cf) : (T)0;
           if (Kind == SK_HAM) {
-            const T kx = cf.k0 * centre + cf.ke * edges + cf.kc * corners;
-            if (a.out1)
-              ((T *)a.out1)[idx] = cf.kin * kx + cf.vscale * vz[ly[r] * Tl::TX + lx[r]] * centre;
+            const T kx = sc.stiff(r, cf);
+            if (sizeof(T) == 4 || a.out1) {
+              const T v = vz[ly[r] * Tl::TX + lx[r]];
+              ((T *)a.out1)[idx] = fma(cf.kin, kx, (kScaledV ? v : cf.vscale * v) * centre);
+            }
             if (a.out2) ((T *)a.out2)[idx] = m;
             acc0 = fma(centre, kx, acc0);
           } else if (Kind == SK_HAM_INC) {
-            const T kx = cf.k0 * centre + cf.ke * edges + cf.kc * corners;
+            const T kx = sc.stiff(r, cf);
             const T xb = bb[0][r], eb = bb[1][r];
             const int nd = ly[r] * Tl::TX + lx[r];
             const int pl = (q + 2) % 3;
@@ -465,7 +566,7 @@ __global__ void __launch_bounds__(kStThreads, 2) stencil_tma_kernel(const __grid
             acc1 = (sum - acc0) - y;
             acc0 = sum;
           } else {
-            if (Kind != SK_MASS_DOT || a.out1) ((T *)a.out1)[idx] = m;
+            if (Kind != SK_MASS_DOT || sizeof(T) == 4 || a.out1) ((T *)a.out1)[idx] = m;
             if (Kind >= SK_MASS_DOT) acc0 = fma(centre, m, acc0);
             if (Kind == SK_MASS_BB) {
               const T dx = bb[0][r] - bb[2][r];
@@ -486,11 +587,7 @@ __global__ void __launch_bounds__(kStThreads, 2) stencil_tma_kernel(const __grid
       break;
     }
     if (threadIdx.x == 0 && q + kStStages < nplanes) load_stage(q + kStStages);
-#pragma unroll
-    for (int r = 0; r < kStNodesPerThread; ++r) {
-      c_old[r] = c_mid[r]; f_old[r] = f_mid[r]; e_old[r] = e_mid[r];
-      c_mid[r] = c_new[r]; f_mid[r] = f_new[r]; e_mid[r] = e_new[r];
-    }
+    sc.shift();
   }
   if (failed_at >= 0) {
     // record the timeout, give the copies still in flight a bounded wait,
@@ -503,6 +600,7 @@ __global__ void __launch_bounds__(kStThreads, 2) stencil_tma_kernel(const __grid
     acc0 = acc1 = acc2 = acc3 = 0;
   }
   if (Kind == SK_MASS) return;
+  if (Kind == SK_HAM && StCols<T, Kind>::kNew) acc0 *= cf.ke;
   const double s0 =
       block_sum(Kind == SK_HAM_INC ? (double)acc0 - (double)acc1 : (double)acc0, smem);
   if (threadIdx.x == 0) a.part[blockIdx.x] = s0;
@@ -522,8 +620,18 @@ __global__ void __launch_bounds__(kStThreads, 2) stencil_tma_kernel(const __grid
 
 // Geometry of a launch: tiles, orbital chunks and z segments; the number of
 // segments is lowered until the block partials (nchan per block) fit.
+// `halo` > 0 (one system alone on the device): the segment length with the
+// shortest schedule.  The blocks of an SM share its pipes, so an SM with k
+// blocks needs k (zseg + halo) plane times, halo being the cost of a block's
+// two extra planes; a few blocks too many per SM (a nearly empty last wave)
+// cost as much as the shortest segments' halos, and a grid with fewer blocks
+// than SMs leaves SMs idle, so both are weighed: 24^3 x 4 runs 96 blocks of
+// one plane (12 of 8 before), 64^3 x 64 1024 of 16 planes (7 per SM).
+// `halo` = 0 (jobs that share the device): about 8 blocks per SM, segments of
+// at least 8 planes, or segments of `planes` planes when given.
 template <int PC>
-static ks_status stencil_geometry(const Problem &P, int nchan, StArgs &a, int planes = 0) {
+static ks_status stencil_geometry(const Problem &P, int nchan, StArgs &a, double halo,
+                                  int planes = 0) {
   using Tl = StTile<PC>;
   a.N = P.N;
   a.p = P.p;
@@ -531,12 +639,21 @@ static ks_status stencil_geometry(const Problem &P, int nchan, StArgs &a, int pl
   a.tiles_y = (P.N + Tl::TY - 1) / Tl::TY;
   a.chunks = (P.p + PC - 1) / PC;
   const long long base = (long long)a.tiles_x * a.tiles_y * a.chunks;
-  // aim for about 8 blocks per SM, with segments of at least 8 planes (or
-  // segments of `planes` planes when given)
   long long segs = (8LL * P.sms + base - 1) / base;
   const long long maxsegs = (P.N + 7) / 8;
   if (segs > maxsegs) segs = maxsegs;
   if (planes > 0) segs = (P.N + planes - 1) / planes;
+  if (halo > 0.0) {
+    double best = 1e300;
+    for (int z = P.N; z >= 1; --z) {
+      const long long used = (P.N + z - 1) / z;
+      const double cost = (double)((base * used + P.sms - 1) / P.sms) * (z + halo);
+      if (cost < best) {
+        best = cost;
+        segs = used;
+      }
+    }
+  }
   if (segs < 1) segs = 1;
   for (;;) {
     a.zseg = (int)((P.N + segs - 1) / segs);
@@ -603,8 +720,12 @@ static bool stencil_launch_tma(Problem &P, const StArgs &a, int cls, double flop
 
 template <typename T, int PC, int Kind>
 static ks_status stencil_launch_pc(Problem &P, StArgs &a, int nchan, double flops, double bytes) {
-  KS_TRY(stencil_geometry<PC>(P, nchan, a));
+  // FP64: a halo plane costs its in-plane sums, over half of a plane's
+  // instructions, two of them 1.2 planes.  FP32 reads it from L2 and is
+  // bound by memory, where more and shorter segments overlap better
+  KS_TRY(stencil_geometry<PC>(P, nchan, a, sizeof(T) == 8 ? 1.2 : 0.0));
   a.c = q1_coefficients(P.h);
+  a.k0r = a.c.k0 / a.c.ke;
   if (P.mass == KS_MASS_LUMPED) {      // row sums of M: h^3 on the centre
     a.c.m0 = P.h * P.h * P.h;
     a.c.mf = a.c.me = a.c.mc = 0.0;
@@ -732,6 +853,7 @@ __global__ void __launch_bounds__(kStThreads) stencil_batch_kernel(
   a.c.m0 = b.qc[4]; a.c.mf = b.qc[5]; a.c.me = b.qc[6]; a.c.mc = b.qc[7];
 #pragma unroll
   for (int i = 0; i < 9; ++i) a.cf[i] = b.qcf[i];
+  a.k0r = a.c.k0 / a.c.ke;
   a.occ = b.occ;
   a.kfac = b.occ;
   a.h3 = b.h3;
@@ -804,10 +926,10 @@ ks_status batch_stencil_geometry(Batch &B) {
     Problem &P = B.probs[j]->P;
     BJob &b = B.jobs_host[j];
     StArgs a{};
-    if (P.p >= 32) KS_TRY(stencil_geometry<32>(P, 4, a, planes));
-    else if (P.p >= 16) KS_TRY(stencil_geometry<16>(P, 4, a, planes));
-    else if (P.p >= 8) KS_TRY(stencil_geometry<8>(P, 4, a, planes));
-    else KS_TRY(stencil_geometry<4>(P, 4, a, planes));
+    if (P.p >= 32) KS_TRY(stencil_geometry<32>(P, 4, a, 0.0, planes));
+    else if (P.p >= 16) KS_TRY(stencil_geometry<16>(P, 4, a, 0.0, planes));
+    else if (P.p >= 8) KS_TRY(stencil_geometry<8>(P, 4, a, 0.0, planes));
+    else KS_TRY(stencil_geometry<4>(P, 4, a, 0.0, planes));
     b.st_zseg = a.zseg;
     b.st_tiles_x = a.tiles_x;
     b.st_tiles_y = a.tiles_y;
