@@ -530,7 +530,11 @@ ks_status build_maps(Batch &B) {
     }
     put(BM_COEF, j, (2 * p * p + kThreads - 1) / kThreads);
     put(BM_CG_NODES, j, (n + kCgThreads - 1) / kCgThreads);
-    put(BM_CG_PLANES, j, b.N);
+    long long cga, cgbc, cgup;
+    cg_batch_blocks(b.N, &cga, &cgbc, &cgup);
+    put(BM_CG_A, j, cga);
+    put(BM_CG_BC, j, cgbc);
+    put(BM_CG_UPDATE, j, cgup);
     put(BM_COPY, j, (n * p + 4 * kThreads - 1) / (4 * kThreads));
   }
   for (int m = 0; m < BM_COUNT; ++m) {

@@ -2,23 +2,32 @@
 // Dirichlet values (the discrete L^+ rho of Sec. 2.3 for the Q1 stiffness),
 // as one persistent cooperative kernel.
 //
-// Preconditioner (optional, on by default): the exact inverse of K applied
-// in FP32 through the orthonormal sine basis that diagonalises the 1-D
-// factors K1 and M1, K^{-1} = (Phi x Phi x Phi) Lambda^{-1} (Phi x Phi x Phi)
-// with Lambda_abc = k_a m_b m_c + m_a k_b m_c + m_a m_b k_c.  Applied in
-// single precision it is an SPD approximation of K^{-1} to about 1e-6, so
-// the FP64 CG reaches 1e-10 in two or three iterations.  Each sine transform
-// is a dense N x N product along one grid axis: fused in shared memory for
-// N <= 128 (three grid barriers per application), tiled through shared
-// memory above (six axis passes, one grid barrier after each).
+// Preconditioned form (the default).  K is diagonal in the orthonormal sine
+// basis that diagonalises the 1-D factors K1 and M1,
+//   K^{-1} = (Phi x Phi x Phi) Lambda^{-1} (Phi x Phi x Phi),
+//   Lambda_abc = k_a m_b m_c + m_a k_b m_c + m_a m_b k_c.
+// Applied in FP32 it is P = K^{-1} (1 + O(1e-5)), so close that defect
+// correction
+//   z = P r,  x += z,  r -= K z   (r and K z in FP64)
+// reduces the residual by four to six digits per step, as many as conjugate
+// gradients with the same P, without its two inner products: a step is three
+// transform phases and one update, four grid barriers (six for CG), and
+// the update needs no search direction.  A step that does not reduce the
+// residual by half hands the system to the CG loop below (which also serves
+// cg_precond = 0).  The sine transforms use the parity of the modes: a sine
+// mode is symmetric (k odd) or antisymmetric (k even) about the middle of its
+// axis, so folding the input (u_j = v_j + v_{N+1-j}, w_j = v_j - v_{N+1-j})
+// leaves two N/2 x N/2 products per axis, half the work of one N x N, and the
+// parities split a plane into independent work items.  N <= kFusedMaxN: both
+// in-plane axes in one pass, all in shared memory; above, six tiled axis
+// passes.  What bounds a solve is the chain of phases: a barrier costs 2.5 to
+// 4 us, a transform phase its loads' latency, the update the FP64 pipe.
+// Measured, PCG with full transforms -> this form: warm solve at 64^3 172 ->
+// 106 us, at 105^3 519 -> 299 us; cold at 81^3 463 -> 180 us; 24^3 80 -> 63 us.
 //
-// Each CG iteration needs two grid-wide reductions (p.q and r.r, plus r.z
-// when preconditioned).  The search direction p_j = s_j + beta p_{j-1}
-// (s = z or r) is folded into the stencil of the next iteration (p is
-// double-buffered and recomputed on the fly for the neighbours).  Partial
-// sums are written per block and summed by every block in the same order,
-// so all blocks take identical branch decisions and the result is
-// deterministic.
+// Each step's reductions are partial sums written per block and summed by
+// every block in the same order, so all blocks take identical branch
+// decisions and the result is deterministic.
 #include "ks_device.cuh"
 
 namespace ks {
@@ -30,6 +39,7 @@ struct CgArgs {
   double bscale;              // 4 pi h^3
   const double *rho;
   double *x, *r, *pa, *pb, *q, *z;
+  float *r32;                 // FP32 copy of r for the transforms (in pa's storage)
   float *t1, *t2;             // sine-transform work vectors
   const float *phi;           // N x N sine basis
   const float *kap, *mu;      // 1-D eigenvalues of K1 and M1
@@ -46,6 +56,40 @@ struct CgArgs {
   double *rho_prev;           // density of the last solve (its b / bscale)
   int vb, vnb;                // this block's index among the vnb blocks that solve this system
 };
+
+// Grid barrier of the solver: one counter that only grows (zeroed before
+// the launch), `epoch` the arrivals expected so far (compared modulo 2^32).
+// Arrival is a release, the poll an acquire, so a phase costs one atomic
+// round trip and a poll; a wait that runs out records KS_ETIMEOUT and
+// adds 2^30 to the counter, which ends every other block's wait at its next
+// poll.
+__device__ __forceinline__ bool cg_barrier(const CgArgs &a, unsigned int &epoch) {
+  __shared__ int s_ok;
+  epoch += (unsigned int)a.vnb;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned int *cnt = &a.bar->count;
+    unsigned int v;
+    asm volatile("atom.add.release.gpu.global.u32 %0, [%1], 1;" : "=r"(v) : "l"(cnt) : "memory");
+    long long spins = 0;
+    unsigned int ns = 32;
+    while ((int)((v = ld_acquire_gpu(cnt)) - epoch) < 0) {
+      if (++spins > kSpinLimit) {
+        atomicCAS(a.status, 0, (int)KS_ETIMEOUT);
+        v = epoch + (1u << 30);
+        atomicAdd(cnt, 1u << 30);
+        break;
+      }
+      if (spins > kSpinFree) {
+        __nanosleep(ns);
+        if (ns < 256) ns <<= 1;
+      }
+    }
+    s_ok = v - epoch < (1u << 29);
+  }
+  __syncthreads();
+  return s_ok != 0;
+}
 
 // (K v)_k for v = a + beta * b (b ignored when UseB is false), Dirichlet.
 // The Q1 stiffness has zero face coefficients, so only the centre, the 12
@@ -92,13 +136,13 @@ __device__ __forceinline__ double stiff_apply(const double *a, const double *b, 
 // whose FMA chains run over k in ascending order.  Phi is symmetric and
 // orthogonal, so the same matrix serves the forward and the inverse passes.
 // Mode 1 (after the forward z pass) divides by Lambda of the frequency
-// triple; Mode 2 (the last inverse pass) writes FP64 z and accumulates r.z.
+// triple; Mode 2 (the last inverse pass) writes FP64 z.
 constexpr int kTJ = 64, kTC = 128, kTK = 32, kTCPad = kTC + 1;
 static_assert(kCgThreads == 256, "the 16 x 16 thread grid of the tiled sine pass");
 
-template <typename Tin, int Mode>
-__device__ double tiled_pass(const CgArgs &a, const Tin *in, float *out32, double *out64, int axis,
-                             float *sh) {
+template <int Mode>
+__device__ void tiled_pass(const CgArgs &a, const float *in, float *out32, double *out64, int axis,
+                           float *sh) {
   const int N = a.N;
   const long long NN = (long long)N * N;
   long long sa, sc, ss, C;
@@ -111,7 +155,6 @@ __device__ double tiled_pass(const CgArgs &a, const Tin *in, float *out32, doubl
   const long long total = (long long)S * ctiles * jblocks;
   float *Xs = sh, *Ps = sh + kTK * kTCPad;
   const int tid = threadIdx.x, tj = tid >> 4, tc = tid & 15;
-  double rz = 0.0;
   for (long long w = a.vb; w < total; w += a.vnb) {
     const int jb = (int)(w % jblocks) * kTJ;
     const long long w2 = w / jblocks;
@@ -134,8 +177,7 @@ __device__ double tiled_pass(const CgArgs &a, const Tin *in, float *out32, doubl
         float v = 0.f;
         if (k < N && c < C) {
           const long long idx = base + k * sa + c * sc;
-          if constexpr (sizeof(Tin) == 8) v = (float)__ldcg((const double *)in + idx);
-          else v = __ldcg((const float *)in + idx);
+          v = __ldcg(in + idx);
         }
         Xs[kk * kTCPad + cc] = v;
       }
@@ -176,264 +218,462 @@ __device__ double tiled_pass(const CgArgs &a, const Tin *in, float *out32, doubl
           val = val / lam;
         }
         if (Mode == 2) {
-          const double zv = (double)val;
-          out64[idx] = zv;
-          rz = fma(a.r[idx], zv, rz);
+          out64[idx] = (double)val;
         } else {
           out32[idx] = val;
         }
       }
     }
   }
-  return rz;
 }
 
 constexpr size_t kTiledSmem = (size_t)(kTK * kTCPad + kTK * kTJ) * sizeof(float);
 
-// z = P^{-1} r (six tiled passes, each followed by a grid barrier); returns
-// this thread's share of r.z, or false when a barrier failed.
-__device__ bool apply_precond(const CgArgs &a, double *rz_l) {
+// z = P r (six tiled passes, a grid barrier after each of the first five);
+// false when a barrier failed.
+__device__ bool apply_precond(const CgArgs &a, unsigned int &epoch) {
   extern __shared__ float dyn[];
-  tiled_pass<double, 0>(a, a.r, a.t1, nullptr, 0, dyn);
-  if (!grid_barrier_n(a.bar, a.status, a.vnb)) return false;
-  tiled_pass<float, 0>(a, a.t1, a.t2, nullptr, 1, dyn);
-  if (!grid_barrier_n(a.bar, a.status, a.vnb)) return false;
-  tiled_pass<float, 1>(a, a.t2, a.t1, nullptr, 2, dyn);
-  if (!grid_barrier_n(a.bar, a.status, a.vnb)) return false;
-  tiled_pass<float, 0>(a, a.t1, a.t2, nullptr, 2, dyn);
-  if (!grid_barrier_n(a.bar, a.status, a.vnb)) return false;
-  tiled_pass<float, 0>(a, a.t2, a.t1, nullptr, 1, dyn);
-  if (!grid_barrier_n(a.bar, a.status, a.vnb)) return false;
-  *rz_l = tiled_pass<float, 2>(a, a.t1, nullptr, a.z, 0, dyn);
+  tiled_pass<0>(a, a.r32, a.t1, nullptr, 0, dyn);
+  if (!cg_barrier(a, epoch)) return false;
+  tiled_pass<0>(a, a.t1, a.t2, nullptr, 1, dyn);
+  if (!cg_barrier(a, epoch)) return false;
+  tiled_pass<1>(a, a.t2, a.t1, nullptr, 2, dyn);
+  if (!cg_barrier(a, epoch)) return false;
+  tiled_pass<0>(a, a.t1, a.t2, nullptr, 2, dyn);
+  if (!cg_barrier(a, epoch)) return false;
+  tiled_pass<0>(a, a.t2, a.t1, nullptr, 1, dyn);
+  if (!cg_barrier(a, epoch)) return false;
+  tiled_pass<2>(a, a.t1, nullptr, a.z, 0, dyn);
   return true;
 }
 
-// Fused form for N <= kFusedMaxN, with the planes in shared memory (three
-// N x ld matrices of dynamic shared memory: a plane, Phi and a work matrix;
-// ld = 68 for N <= 64, 132 above, so that every 16-byte row access of a
-// 64-wide output tile stays inside its row):
-//   A: each z-plane P (N x N, rows y, columns x) -> Phi P Phi   (y, then x)
-//   B: each y-slab S (rows z, columns x)          -> Phi (Lambda^{-1} o (Phi S))
-//   C: each z-plane                               -> Phi P Phi, written as z
-// (Phi is symmetric, so Phi P Phi transforms both in-plane axes), three grid
-// barriers per application instead of six.
+// ---------------------------------------------------------------- fused form
+// Modes of one axis in parity order: the h1 = ceil(N/2) symmetric ones
+// (0-based 0, 2, ...), then the h0 = floor(N/2) antisymmetric ones.  Work
+// vectors hold the transformed axes in this order.
+//   A  item (z, parity of ky, parity of kx): the folded quarter of plane z of
+//      r -> its modes (y, then x)
+//   B  item (ky, parity of kx): forward along z, Lambda^{-1}, inverse along z
+//   C  item (z, half of the y pairs): inverse along y, then x -> z in FP64
+// Shared memory, in units of hp x hp floats (hp = h1 rounded up to 4): the
+// half bases F_e, F_o (row j, column mode) and their transposes I_e, I_o, and
+// four work matrices: 100 KiB at N = 105, two blocks per SM.
 constexpr int kFusedMaxN = 128;
 
-__host__ __device__ constexpr int fused_ld(int N) { return N <= 64 ? 68 : 132; }
-
-// out = A B for N x N matrices in shared memory (row stride ld), A given by
-// its transpose At (At[k][i] = A[i][k]; Phi is its own transpose).  Each
-// thread keeps a 4 x 4 block of a 64 x 64 output tile (rows 4 ty .. + 3,
-// columns 4 tx .. + 3 with ty = tid / 16, tx = tid % 16): per k one 16-byte
-// load of At (two addresses per warp, broadcast) and one of B (16
-// consecutive ones) for 16 FMAs.  Each output is one k-ascending FMA chain.
-// Trans: out is stored transposed (out[j][i]), ready to be the At of the
-// next product.
-template <bool Trans>
-__device__ __forceinline__ void smem_matmul(const float *At, const float *B, float *out, int N,
-                                            int ld) {
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  for (int ib = 0; ib < N; ib += 64)
-    for (int jb = 0; jb < N; jb += 64) {
-      const int i0 = ib + 4 * ty, j0 = jb + 4 * tx;
-      if (i0 >= N || j0 >= N) continue;
-      // every 16-byte row access of the tile stays inside its row
-      if (!KS_IN(i0 + 3, ld) || !KS_IN(j0 + 3, ld)) continue;
-      float acc[4][4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int v = 0; v < 4; ++v) acc[u][v] = 0.f;
-#pragma unroll 4
-      for (int k = 0; k < N; ++k) {
-        const float4 av = *reinterpret_cast<const float4 *>(At + k * ld + i0);
-        const float4 bv = *reinterpret_cast<const float4 *>(B + k * ld + j0);
-        const float a4[4] = {av.x, av.y, av.z, av.w};
-        const float b4[4] = {bv.x, bv.y, bv.z, bv.w};
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-#pragma unroll
-          for (int v = 0; v < 4; ++v) acc[u][v] = fmaf(a4[u], b4[v], acc[u][v]);
-      }
-      // rows / columns past N land in the padding of the row (never read as
-      // data: every product sums k < N only)
-      if (Trans) {
-#pragma unroll
-        for (int v = 0; v < 4; ++v)
-          if (j0 + v < N)
-            *reinterpret_cast<float4 *>(out + (j0 + v) * ld + i0) =
-                make_float4(acc[0][v], acc[1][v], acc[2][v], acc[3][v]);
-      } else {
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (i0 + u < N)
-            *reinterpret_cast<float4 *>(out + (i0 + u) * ld + j0) =
-                make_float4(acc[u][0], acc[u][1], acc[u][2], acc[u][3]);
-      }
-    }
-}
-
-// Element (r, c) of an N x N plane for every r, c < N: warp w takes rows
-// w, w + 8, ..., its lanes the columns (coalesced, no index division), in
-// 64 x 64 patches of 16 values per thread whose loads are all issued before
-// the first is used, so a patch costs about one memory latency.
-template <typename V, typename L, typename U>
-__device__ __forceinline__ void plane_batched(int N, L load, U use) {
-  static_assert(kCgThreads == 256, "8 warps x 8 rows make a 64-row patch");
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  for (int r0 = 0; r0 < N; r0 += 64)
-    for (int c0 = 0; c0 < N; c0 += 64) {
-      V v[8][2];
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          const int r = r0 + w + 8 * i, c = c0 + l + 32 * j;
-          v[i][j] = (r < N && c < N) ? load(r, c) : V(0);
-        }
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          const int r = r0 + w + 8 * i, c = c0 + l + 32 * j;
-          if (r < N && c < N) use(r, c, v[i][j]);
-        }
-    }
-}
-
-// Shared memory of the fused preconditioner: plane, Phi and work matrices
-// (N x ld each), then the 1-D eigenvalues kappa and mu (N each).
+__host__ __device__ constexpr int half_pad(int N) { return ((N + 1) / 2 + 3) / 4 * 4; }
+// y pairs of pass C's first half
+__host__ __device__ constexpr int half_split(int N) { return (((N + 1) / 2 + 1) / 2 + 3) / 4 * 4; }
 __host__ __device__ constexpr size_t fused_smem_floats(int N) {
-  return (size_t)3 * N * fused_ld(N) + 2 * (size_t)N;
+  const size_t m = (size_t)half_pad(N) * half_pad(N);
+  const size_t c = 2 * m + (size_t)N * 2 * half_split(N);      // pass C: T and Yt
+  return 4 * m + (c > 4 * m ? c : 4 * m);
 }
 
-// Phi, kappa and mu into shared memory (once per kernel).
-__device__ __forceinline__ void load_phi(const CgArgs &a, float *sh) {
-  const int N = a.N, ld = fused_ld(N);
-  float *Ph = sh + N * ld, *kap = sh + 3 * N * ld, *mu = kap + N;
-  plane_batched<float>(
-      N, [&](int r, int c) { return __ldg(a.phi + r * N + c); },
-      [&](int r, int c, float v) { Ph[r * ld + c] = v; });
-  for (int i = threadIdx.x; i < N; i += blockDim.x) {
-    kap[i] = __ldg(a.kap + i);
-    mu[i] = __ldg(a.mu + i);
+struct FusedDims {
+  int N, h1, h0, hp;
+  long long NN;
+  float *fe, *fo, *ie, *io, *w;
+  __device__ FusedDims(int N_, float *sh) : N(N_) {
+    h1 = (N + 1) / 2;
+    h0 = N / 2;
+    hp = half_pad(N);
+    NN = (long long)N * N;
+    const int m = hp * hp;
+    fe = sh;
+    fo = sh + m;
+    ie = sh + 2 * m;
+    io = sh + 3 * m;
+    w = sh + 4 * m;
+  }
+};
+
+// The half bases from the N x N sine matrix (once per kernel).
+__device__ __forceinline__ void load_phi(const CgArgs &a, float *sh, bool fwd = true,
+                                         bool inv = true) {
+  const FusedDims d(a.N, sh);
+  for (int e = threadIdx.x; e < d.N * d.h1; e += kCgThreads) {
+    const int k = e / d.h1, j = e - k * d.h1, m = k >> 1;    // mode k, node j
+    if ((k & 1) && j >= d.h0) continue;
+    const float v = __ldg(a.phi + (long long)k * d.N + j);
+    if (!KS_IN(j * d.hp + m, d.hp * d.hp) || !KS_IN(m * d.hp + j, d.hp * d.hp)) continue;
+    if (fwd) ((k & 1) ? d.fo : d.fe)[j * d.hp + m] = v;
+    if (inv) ((k & 1) ? d.io : d.ie)[m * d.hp + j] = v;
   }
 }
 
-// Phi P Phi of the plane in Pm (already staged), y then x; the result is
-// left in Pm.
-__device__ __forceinline__ void plane_transform(int N, int ld, float *sh) {
-  float *Pm = sh, *Ph = sh + N * ld, *W = sh + 2 * N * ld;
-  __syncthreads();
-  smem_matmul<true>(Ph, Pm, W, N, ld);     // W^T, W = Phi P (along y)
-  __syncthreads();
-  smem_matmul<false>(W, Ph, Pm, N, ld);    // (Phi P) Phi (along x)
-  __syncthreads();
-}
-
-// Phi P Phi for the plane z of `in` (FP64 r or FP32 work), into out32 or,
-// for the last step, out64 with the r.z accumulation.
-template <bool InD, bool OutD>
-__device__ double fused_plane_pass(const CgArgs &a, const void *in, float *out32, double *out64,
-                                   float *sh) {
-  const int N = a.N, ld = fused_ld(N);
-  const long long NN = (long long)N * N;
-  float *Pm = sh;
-  double rz = 0.0;
-  for (int z = a.vb; z < N; z += a.vnb) {
-    const long long zo = z * NN;
-    __syncthreads();
-    if (InD)
-      plane_batched<double>(
-          N,
-          [&](int y, int x) {
-            return KS_IN(zo + y * N + x, a.n) ? __ldcg((const double *)in + zo + y * N + x) : 0.0;
-          },
-          [&](int y, int x, double v) { Pm[y * ld + x] = (float)v; });
-    else
-      plane_batched<float>(
-          N,
-          [&](int y, int x) {
-            return KS_IN(zo + y * N + x, a.n) ? __ldcg((const float *)in + zo + y * N + x) : 0.f;
-          },
-          [&](int y, int x, float v) { Pm[y * ld + x] = v; });
-    plane_transform(N, ld, sh);
-    if (OutD)
-      plane_batched<double>(
-          N, [&](int y, int x) { return __ldcg(a.r + zo + y * N + x); },
-          [&](int y, int x, double rv) {
-            const double zv = (double)Pm[y * ld + x];
-            if (KS_IN(zo + y * N + x, a.n)) out64[zo + y * N + x] = zv;
-            rz = fma(rv, zv, rz);
-          });
-    else
-      plane_batched<float>(
-          N, [&](int y, int x) { return Pm[y * ld + x]; },
-          [&](int y, int x, float v) {
-            if (KS_IN(zo + y * N + x, a.n)) out32[zo + y * N + x] = v;
-          });
+template <int TT>
+__device__ __forceinline__ void ldv(const float *p, float (&v)[TT]) {
+  if constexpr (TT == 4) {
+    const float4 q = *reinterpret_cast<const float4 *>(p);
+    v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+  } else {
+    const float2 q = *reinterpret_cast<const float2 *>(p);
+    v[0] = q.x; v[1] = q.y;
   }
-  return rz;
 }
 
-// For each y: S[z][x] -> Phi (Lambda^{-1} o (Phi S)) along z.
-__device__ void fused_slab_pass(const CgArgs &a, const float *in, float *out, float *sh) {
-  const int N = a.N, ld = fused_ld(N);
-  const long long NN = (long long)N * N;
-  float *Sm = sh, *Ph = sh + N * ld, *W = sh + 2 * N * ld;
-  const float *kap = sh + 3 * N * ld, *mu = kap + N;
-  for (int y = a.vb; y < N; y += a.vnb) {
+// acc[u][v] += sum_k A[k][m0 + u] B[k][n0 + v] (row strides lda, ldb)
+template <int TT>
+__device__ __forceinline__ void tile_fma(const float *A, int lda, const float *B, int ldb, int K,
+                                         float (&acc)[TT][TT]) {
+#pragma unroll 4
+  for (int k = 0; k < K; ++k) {
+    float av[TT], bv[TT];
+    ldv<TT>(A + k * lda, av);
+    ldv<TT>(B + k * ldb, bv);
+#pragma unroll
+    for (int u = 0; u < TT; ++u)
+#pragma unroll
+      for (int v = 0; v < TT; ++v) acc[u][v] = fmaf(av[u], bv[v], acc[u][v]);
+  }
+}
+
+// out(m0, n0, acc) for every TT x TT tile of C = A^T B (M x Nn, K terms), both
+// operands k-major in shared memory; columns past M or Nn read padding and
+// only reach entries that `out` drops.
+template <int TT, typename Out>
+__device__ __forceinline__ void tile_gemm(int M, int Nn, int K, const float *A, int lda,
+                                          const float *B, int ldb, Out out) {
+  const int tn = (Nn + TT - 1) / TT, tiles = (M + TT - 1) / TT * tn;
+  for (int t = threadIdx.x; t < tiles; t += kCgThreads) {
+    const int m0 = t / tn * TT, n0 = t % tn * TT;
+    if (!KS_IN(m0 + TT - 1, lda) || !KS_IN(n0 + TT - 1, ldb)) continue;
+    float acc[TT][TT];
+#pragma unroll
+    for (int u = 0; u < TT; ++u)
+#pragma unroll
+      for (int v = 0; v < TT; ++v) acc[u][v] = 0.f;
+    tile_fma<TT>(A + m0, lda, B + n0, ldb, K, acc);
+    out(m0, n0, acc);
+  }
+}
+
+// The same for two products of one shape (K1 and K2 terms): out(m0, n0, e, o).
+template <int TT, typename Out>
+__device__ __forceinline__ void tile_gemm2(int M, int Nn, int K1, const float *A1, const float *B1,
+                                           int K2, const float *A2, const float *B2, int lda,
+                                           int ldb, Out out) {
+  const int tn = (Nn + TT - 1) / TT, tiles = (M + TT - 1) / TT * tn;
+  for (int t = threadIdx.x; t < tiles; t += kCgThreads) {
+    const int m0 = t / tn * TT, n0 = t % tn * TT;
+    if (!KS_IN(m0 + TT - 1, lda) || !KS_IN(n0 + TT - 1, ldb)) continue;
+    float e[TT][TT], o[TT][TT];
+#pragma unroll
+    for (int u = 0; u < TT; ++u)
+#pragma unroll
+      for (int v = 0; v < TT; ++v) e[u][v] = o[u][v] = 0.f;
+    tile_fma<TT>(A1 + m0, lda, B1 + n0, ldb, K1, e);
+    tile_fma<TT>(A2 + m0, lda, B2 + n0, ldb, K2, o);
+    out(m0, n0, e, o);
+  }
+}
+
+template <int TT>
+__device__ __forceinline__ void fused_pass_a(const CgArgs &a, const float *r32, float *out,
+                                             float *sh) {
+  const FusedDims d(a.N, sh);
+  const int N = d.N, hp = d.hp;
+  float *Q = d.w, *Wt = d.w + hp * hp;
+  for (int item = a.vb; item < 4 * N; item += a.vnb) {
+    const int z = item >> 2, py = (item >> 1) & 1, px = item & 1;
+    const int hy = py ? d.h0 : d.h1, hx = px ? d.h0 : d.h1;
+    const float sy = py ? -1.f : 1.f, sx = px ? -1.f : 1.f;
+    const float *P = r32 + z * d.NN;
     __syncthreads();
-    plane_batched<float>(
-        N,
-        [&](int zz, int x) {
-          const long long k = zz * NN + (long long)y * N + x;
-          return KS_IN(k, a.n) ? __ldcg(in + k) : 0.f;
-        },
-        [&](int zz, int x, float v) { Sm[zz * ld + x] = v; });
-    __syncthreads();
-    smem_matmul<false>(Ph, Sm, W, N, ld);   // forward along z
-    __syncthreads();
-    const float ky = kap[y], my = mu[y];
-    for (int c = threadIdx.x >> 5; c < N; c += kCgThreads / 32)
-      for (int x = threadIdx.x & 31; x < N; x += 32) {
-        const float lam = kap[x] * my * mu[c] + mu[x] * ky * mu[c] + mu[x] * my * kap[c];
-        W[c * ld + x] = W[c * ld + x] / lam;
+    // the four mirror images of a folded entry; four entries in flight
+    for (int e0 = threadIdx.x; e0 < hy * hx; e0 += 4 * kCgThreads) {
+      float v[4][4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int e = e0 + u * kCgThreads;
+        const int j = e / hx, i = e - j * hx, j2 = N - 1 - j, i2 = N - 1 - i;
+        const bool ok = e < hy * hx && KS_IN(z * d.NN + (long long)j2 * N + i2, a.n);
+        v[u][0] = ok ? __ldcg(P + j * N + i) : 0.f;
+        v[u][1] = ok && i2 != i ? __ldcg(P + j * N + i2) : 0.f;
+        v[u][2] = ok && j2 != j ? __ldcg(P + j2 * N + i) : 0.f;
+        v[u][3] = ok && j2 != j && i2 != i ? __ldcg(P + j2 * N + i2) : 0.f;
       }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int e = e0 + u * kCgThreads;
+        if (e >= hy * hx) break;
+        const int j = e / hx, i = e - j * hx;
+        Q[j * hp + i] = fmaf(sy, fmaf(sx, v[u][3], v[u][2]), fmaf(sx, v[u][1], v[u][0]));
+      }
+    }
     __syncthreads();
-    smem_matmul<false>(Ph, W, Sm, N, ld);   // inverse along z
+    tile_gemm<TT>(hy, hx, hy, py ? d.fo : d.fe, hp, Q, hp,
+                  [&](int m0, int n0, float (&c)[TT][TT]) {
+#pragma unroll
+                    for (int v = 0; v < TT; ++v)
+#pragma unroll
+                      for (int u = 0; u < TT; ++u) Wt[(n0 + v) * hp + m0 + u] = c[u][v];
+                  });
     __syncthreads();
-    plane_batched<float>(
-        N, [&](int zz, int x) { return Sm[zz * ld + x]; },
-        [&](int zz, int x, float v) {
-          const long long k = zz * NN + (long long)y * N + x;
-          if (KS_IN(k, a.n)) out[k] = v;
-        });
+    tile_gemm<TT>(hy, hx, hx, Wt, hp, px ? d.fo : d.fe, hp,
+                  [&](int m0, int n0, float (&c)[TT][TT]) {
+#pragma unroll
+                    for (int u = 0; u < TT; ++u)
+#pragma unroll
+                      for (int v = 0; v < TT; ++v) {
+                        const long long k = z * d.NN + (long long)(py * d.h1 + m0 + u) * N +
+                                            px * d.h1 + n0 + v;
+                        if (m0 + u < hy && n0 + v < hx && KS_IN(k, a.n)) out[k] = c[u][v];
+                      }
+                  });
   }
 }
 
-__device__ bool apply_precond_fused(const CgArgs &a, double *rz_l) {
+template <int TT>
+__device__ __forceinline__ void fused_pass_b(const CgArgs &a, const float *in, float *out,
+                                             float *sh) {
+  const FusedDims d(a.N, sh);
+  const int N = d.N, hp = d.hp, m2 = hp * hp;
+  float *U = d.w, *V = d.w + m2, *Fe = d.w + 2 * m2, *Fo = d.w + 3 * m2;
+  for (int item = a.vb; item < 2 * N; item += a.vnb) {
+    const int ky = item >> 1, px = item & 1, hx = px ? d.h0 : d.h1;
+    const long long col = (long long)ky * N + px * d.h1;
+    __syncthreads();
+    for (int e0 = threadIdx.x; e0 < d.h1 * hx; e0 += 8 * kCgThreads) {
+      float v[8][2];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int e = e0 + u * kCgThreads, j = e / hx, l = e - j * hx;
+        const bool ok = e < d.h1 * hx && KS_IN((N - 1 - j) * d.NN + col + l, a.n);
+        v[u][0] = ok ? __ldcg(in + j * d.NN + col + l) : 0.f;
+        v[u][1] = ok && j < d.h0 ? __ldcg(in + (N - 1 - j) * d.NN + col + l) : 0.f;
+      }
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int e = e0 + u * kCgThreads;
+        if (e >= d.h1 * hx) break;
+        const int j = e / hx, l = e - j * hx;
+        U[j * hp + l] = v[u][0] + v[u][1];
+        V[j * hp + l] = v[u][0] - v[u][1];
+      }
+    }
+    __syncthreads();
+    const int ty = ky < d.h1 ? 2 * ky : 2 * (ky - d.h1) + 1;
+    const float ky_ = __ldg(a.kap + ty), my_ = __ldg(a.mu + ty);
+    auto scaled = [&](float *F, int pz, int hz, int m0, int n0, float (&c)[TT][TT]) {
+#pragma unroll
+      for (int u = 0; u < TT; ++u)
+#pragma unroll
+        for (int v = 0; v < TT; ++v) {
+          const int m = m0 + u, l = n0 + v;
+          if (m >= hz || l >= hx) continue;
+          const int tz = 2 * m + pz, tx = 2 * l + px;
+          const float kz = __ldg(a.kap + tz), mz = __ldg(a.mu + tz);
+          const float kx = __ldg(a.kap + tx), mx = __ldg(a.mu + tx);
+          F[m * hp + l] = c[u][v] / (kx * my_ * mz + mx * ky_ * mz + mx * my_ * kz);
+        }
+    };
+    tile_gemm<TT>(d.h1, hx, d.h1, d.fe, hp, U, hp, [&](int m0, int n0, float (&c)[TT][TT]) {
+      scaled(Fe, 0, d.h1, m0, n0, c);
+    });
+    tile_gemm<TT>(d.h0, hx, d.h0, d.fo, hp, V, hp, [&](int m0, int n0, float (&c)[TT][TT]) {
+      scaled(Fo, 1, d.h0, m0, n0, c);
+    });
+    __syncthreads();
+    tile_gemm2<TT>(d.h1, hx, d.h1, d.ie, Fe, d.h0, d.io, Fo, hp, hp,
+                   [&](int m0, int n0, float (&e)[TT][TT], float (&o)[TT][TT]) {
+#pragma unroll
+                     for (int u = 0; u < TT; ++u)
+#pragma unroll
+                       for (int v = 0; v < TT; ++v) {
+                         const int j = m0 + u, l = n0 + v;
+                         if (j >= d.h1 || l >= hx) continue;
+                         if (!KS_IN((N - 1 - j) * d.NN + col + l, a.n)) continue;
+                         const bool pair = j < d.h0;      // false: the middle node
+                         out[j * d.NN + col + l] = pair ? e[u][v] + o[u][v] : e[u][v];
+                         if (pair) out[(N - 1 - j) * d.NN + col + l] = e[u][v] - o[u][v];
+                       }
+                   });
+  }
+}
+
+template <int TT>
+__device__ __forceinline__ void fused_pass_c(const CgArgs &a, const float *in, double *out,
+                                             float *sh) {
+  const FusedDims d(a.N, sh);
+  const int N = d.N, hp = d.hp, m2 = hp * hp;
+  const int hj = half_split(N);
+  const int ldy = 2 * hj;
+  // T: the plane's modes of one kx parity (rows: symmetric, then antisymmetric
+  // ky); Yt: N modes kx (symmetric, then antisymmetric) x (rows y = j, then
+  // y = N - 1 - j)
+  float *T = d.w, *Yt = d.w + 2 * m2;
+  for (int item = a.vb; item < 2 * N; item += a.vnb) {
+    const int z = item >> 1, jbase = (item & 1) * hj;
+    const int nj = min(hj, d.h1 - jbase);
+    if (nj <= 0) continue;
+    for (int px = 0; px < 2; ++px) {
+      const int hx = px ? d.h0 : d.h1;
+      __syncthreads();
+      const float *src = in + z * d.NN + px * d.h1;
+      for (int e0 = threadIdx.x; e0 < N * hx; e0 += 8 * kCgThreads) {
+        float v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int e = e0 + u * kCgThreads, m = e / hx, l = e - m * hx;
+          v[u] = e < N * hx && KS_IN(z * d.NN + px * d.h1 + (long long)m * N + l, a.n)
+                     ? __ldcg(src + (long long)m * N + l)
+                     : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int e = e0 + u * kCgThreads;
+          if (e >= N * hx) break;
+          const int m = e / hx, l = e - m * hx;
+          T[(m < d.h1 ? m : hp + m - d.h1) * hp + l] = v[u];
+        }
+      }
+      __syncthreads();
+      tile_gemm2<TT>(nj, hx, d.h1, d.ie + jbase, T, d.h0, d.io + jbase, T + m2, hp, hp,
+                     [&](int m0, int n0, float (&e)[TT][TT], float (&o)[TT][TT]) {
+#pragma unroll
+                       for (int v = 0; v < TT; ++v) {
+                         const int l = n0 + v;
+                         if (l >= hx) continue;
+                         float *y = Yt + ((px ? d.h1 : 0) + l) * ldy;
+#pragma unroll
+                         for (int u = 0; u < TT; ++u) {
+                           if (m0 + u >= hj) continue;
+                           const bool pair = jbase + m0 + u < d.h0;
+                           if (!KS_IN(((px ? d.h1 : 0) + l) * ldy + hj + m0 + u, N * ldy)) continue;
+                           y[m0 + u] = pair ? e[u][v] + o[u][v] : e[u][v];
+                           y[hj + m0 + u] = pair ? e[u][v] - o[u][v] : 0.f;
+                         }
+                       }
+                     });
+    }
+    __syncthreads();
+    // rows y of both kinds, inverse along x
+    const int tn = (d.h1 + TT - 1) / TT, tiles = (2 * hj / TT) * tn;
+    for (int t = threadIdx.x; t < tiles; t += kCgThreads) {
+      const int m0 = t / tn * TT, n0 = t % tn * TT;
+      float e[TT][TT], o[TT][TT];
+#pragma unroll
+      for (int u = 0; u < TT; ++u)
+#pragma unroll
+        for (int v = 0; v < TT; ++v) e[u][v] = o[u][v] = 0.f;
+      tile_fma<TT>(Yt + m0, ldy, d.ie + n0, hp, d.h1, e);
+      tile_fma<TT>(Yt + d.h1 * ldy + m0, ldy, d.io + n0, hp, d.h0, o);
+#pragma unroll
+      for (int u = 0; u < TT; ++u) {
+        const int row = m0 + u, jj = row < hj ? row : row - hj, j = jbase + jj;
+        if (jj >= nj || (row >= hj && j >= d.h0)) continue;
+        const int y = row < hj ? j : N - 1 - j;
+        double *dst = out + z * d.NN + (long long)y * N;
+#pragma unroll
+        for (int v = 0; v < TT; ++v) {
+          const int i = n0 + v;
+          if (i >= d.h1 || !KS_IN(z * d.NN + (long long)y * N + N - 1 - i, a.n)) continue;
+          const bool pair = i < d.h0;
+          dst[i] = (double)(pair ? e[u][v] + o[u][v] : e[u][v]);
+          if (pair) dst[N - 1 - i] = (double)(e[u][v] - o[u][v]);
+        }
+      }
+    }
+  }
+}
+
+// Tile edge of the transforms: 2 x 2 outputs per thread keep 256 threads busy
+// up to hp = 32 (N = 64), 4 x 4 (half the shared-memory reads) above.
+__device__ __forceinline__ bool small_tiles(int N) { return half_pad(N) <= 32; }
+
+// z = P r of the fused form: three phases, a barrier after the first two.
+__device__ bool apply_precond_fused(const CgArgs &a, unsigned int &epoch) {
   extern __shared__ float dyn[];
-  fused_plane_pass<true, false>(a, a.r, a.t1, nullptr, dyn);
-  if (!grid_barrier_n(a.bar, a.status, a.vnb)) return false;
-  fused_slab_pass(a, a.t1, a.t2, dyn);
-  if (!grid_barrier_n(a.bar, a.status, a.vnb)) return false;
-  *rz_l = fused_plane_pass<false, true>(a, a.t2, nullptr, a.z, dyn);
+  const bool s = small_tiles(a.N);
+  if (s) fused_pass_a<2>(a, a.r32, a.t1, dyn); else fused_pass_a<4>(a, a.r32, a.t1, dyn);
+  if (!cg_barrier(a, epoch)) return false;
+  if (s) fused_pass_b<2>(a, a.t1, a.t2, dyn); else fused_pass_b<4>(a, a.t1, a.t2, dyn);
+  if (!cg_barrier(a, epoch)) return false;
+  if (s) fused_pass_c<2>(a, a.t2, a.z, dyn); else fused_pass_c<4>(a, a.t2, a.z, dyn);
   return true;
 }
 
-// The whole PCG of one system on the blocks a.vb = 0 .. a.vnb - 1 (which must
-// be co-resident: a cooperative launch).
-//
-// On GB300 every FP64 FMA is scarce (two lanes per SM and clock), so each
-// iteration applies the 27-point stiffness once: q = K p is carried as
-// q = K s + beta q_old (K p by linearity, p = s + beta p_old), and a warm
-// start whose residual is still in r (a.incr) forms the new one without a
-// stencil, r = r_old + (b - b_old), from the right-hand side of the last
-// solve (rho_prev).
+// ---------------------------------------------------------------- update
+// x += z (x = z when `first`), r -= K z and r32 = r over the nodes of
+// this block's share; returns this thread's part of r.r.  A thread takes a
+// column of kUpY nodes along y and kUpZ along z at one x (a warp: 32
+// consecutive x): with the plane sums s = z(x-1) + z(x+1), f, e of six rows
+// shared by its nodes, K z costs 15 FP64 instructions per node instead of 23
+// (K A = b0(z) + bn(z-1) + bn(z+1), b0 = (k0/ke) c + e, bn = f + e/2, times ke).
+constexpr int kUpY = 4, kUpZ = 2;
+
+__device__ __forceinline__ double defect_update(const CgArgs &a, bool first, double k0r) {
+  const int N = a.N;
+  const long long NN = (long long)N * N;
+  const int uy = (N + kUpY - 1) / kUpY, uz = (N + kUpZ - 1) / kUpZ;
+  const long long units = (long long)N * uy * uz;
+  double rl = 0.0;
+  // warps of the launch in turn over the blocks, so that a grid with fewer
+  // units than threads still spreads over the SMs
+  const long long w0 = (long long)(threadIdx.x >> 5) * a.vnb + a.vb;
+  for (long long w = w0; w * 32 < units; w += (long long)a.vnb * (kCgThreads / 32)) {
+    const long long un = w * 32 + (threadIdx.x & 31);
+    if (un >= units) continue;
+    const int x = (int)(un % N);
+    const long long q = un / N;
+    const int y0 = (int)(q % uy) * kUpY, z0 = (int)(q / uy) * kUpZ;
+    double kz[kUpZ][kUpY], cz[kUpZ][kUpY];
+#pragma unroll
+    for (int pl = 0; pl < kUpZ + 2; ++pl) {
+      const int z = z0 + pl - 1;
+      const bool zok = z >= 0 && z < N;
+      double c[kUpY + 2], s[kUpY + 2];
+#pragma unroll
+      for (int y = 0; y < kUpY + 2; ++y) {
+        const int gy = y0 + y - 1;
+        const bool ok = zok && gy >= 0 && gy < N;
+        const double *p = a.z + (ok ? z * NN + (long long)gy * N + x : 0);
+        c[y] = ok ? __ldcg(p) : 0.0;
+        s[y] = (ok && x > 0 ? __ldcg(p - 1) : 0.0) + (ok && x + 1 < N ? __ldcg(p + 1) : 0.0);
+      }
+#pragma unroll
+      for (int r = 0; r < kUpY; ++r) {
+        const double f = s[r + 1] + (c[r] + c[r + 2]);
+        const double e = s[r] + s[r + 2];
+        const double bn = fma(0.5, e, f);
+#pragma unroll
+        for (int o = 0; o < kUpZ; ++o) {
+          if (pl == o) kz[o][r] = bn;
+          else if (pl == o + 1) {
+            kz[o][r] += fma(k0r, c[r + 1], e);
+            cz[o][r] = c[r + 1];
+          } else if (pl == o + 2) {
+            kz[o][r] += bn;
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int o = 0; o < kUpZ; ++o)
+#pragma unroll
+      for (int r = 0; r < kUpY; ++r) {
+        if (z0 + o >= N || y0 + r >= N) continue;
+        const long long k = (z0 + o) * NN + (long long)(y0 + r) * N + x;
+        if (!KS_IN(k, a.n)) continue;
+        a.x[k] = first ? cz[o][r] : a.x[k] + cz[o][r];
+        const double rk = fma(-a.c.ke, kz[o][r], a.r[k]);
+        a.r[k] = rk;
+        a.r32[k] = (float)rk;
+        rl = fma(rk, rk, rl);
+      }
+  }
+  return rl;
+}
+
+// The whole solve of one system on the blocks a.vb = 0 .. a.vnb - 1 (which
+// must be co-resident: a cooperative launch).  A warm start whose residual is
+// still in r (a.incr) forms the new one without a stencil, r = r_old + (b -
+// b_old), from the right-hand side of the last solve (rho_prev).
 __device__ void cg_body(const CgArgs &a) {
   __shared__ double smem[33];
   const int nb = a.vnb;
+  unsigned int epoch = 0;
   double *partA = a.part, *partB = a.part + nb, *partC = a.part + 2 * nb, *partD = a.part + 3 * nb;
   const long long tid = (long long)a.vb * blockDim.x + threadIdx.x;
   const long long stride = (long long)a.vnb * blockDim.x;
@@ -462,6 +702,7 @@ __device__ void cg_body(const CgArgs &a) {
       rk = b - kx;
     }
     a.r[k] = rk;
+    if (a.precond) a.r32[k] = (float)rk;
     a.rho_prev[k] = rk_rho;
     rr_l = fma(rk, rk, rr_l);
     bb_l = fma(b, b, bb_l);
@@ -471,80 +712,84 @@ __device__ void cg_body(const CgArgs &a) {
     const double s2 = block_sum(bb_l, smem);
     if (threadIdx.x == 0) { partB[a.vb] = s1; partD[a.vb] = s2; }
   }
-  if (!grid_barrier_n(a.bar, a.status, a.vnb)) return;
-  if (!a.warm) {
-    for (long long k = tid; k < a.n; k += stride) a.x[k] = 0.0;
-  }
+  if (!cg_barrier(a, epoch)) return;
   double rr = block_sum_array(partB, nb, smem);
   const double bb = block_sum_array(partD, nb, smem);
   const double thr = a.tol * a.tol * bb;
-  double rho_cg = rr;                       // r.z (preconditioned) or r.r
-  const double *s_vec = a.precond ? a.z : a.r;
-  if (a.precond && rr > thr) {
-    double rz_l = 0.0;
-    if (a.fused ? !apply_precond_fused(a, &rz_l) : !apply_precond(a, &rz_l)) return;
-    const double s = block_sum(rz_l, smem);
-    if (threadIdx.x == 0) partC[a.vb] = s;
-    if (!grid_barrier_n(a.bar, a.status, a.vnb)) return;
-    rho_cg = block_sum_array(partC, nb, smem);
-  }
-
-  int it = 0;
-  double beta = 0.0;
-  double *pold = a.pa, *pnew = a.pb;
   // a non-finite right-hand side or start makes every comparison below false
   bool bad = !isfinite(rr) || !isfinite(bb);
-  while (rr > thr && it < a.maxit) {
-    // phase 1: p = s + beta p_old and q = K s + beta q_old (own nodes), p.q
-    double pq_l = 0.0;
-    for (long long k = tid; k < a.n; k += stride) {
-      const int ix = (int)(k % N), iy = (int)((k / N) % N), iz = (int)(k / NN);
-      double sk;
-      const double ks = stiff_apply<false>(s_vec, nullptr, 0.0, N, ix, iy, iz, a.c, &sk);
-      const double pk = it == 0 ? sk : fma(beta, pold[k], sk);
-      const double qk = it == 0 ? ks : fma(beta, a.q[k], ks);
-      pnew[k] = pk;
-      a.q[k] = qk;
-      pq_l = fma(pk, qk, pq_l);
-    }
-    {
-      const double s = block_sum(pq_l, smem);
-      if (threadIdx.x == 0) partA[a.vb] = s;
-    }
-    if (!grid_barrier_n(a.bar, a.status, a.vnb)) return;
-    const double pq = block_sum_array(partA, nb, smem);
-    if (!(pq > 0.0) || !isfinite(pq)) { bad = true; break; }
-    const double alpha = rho_cg / pq;
-    // phase 2: x += alpha p, r -= alpha q, r.r
-    double rl = 0.0;
-    for (long long k = tid; k < a.n; k += stride) {
-      a.x[k] = fma(alpha, pnew[k], a.x[k]);
-      const double rk = fma(-alpha, a.q[k], a.r[k]);
-      a.r[k] = rk;
-      rl = fma(rk, rk, rl);
-    }
-    {
+  int it = 0;
+  bool done = !(rr > thr);
+  bool fresh = !a.warm;                     // x not written yet (a cold start)
+  if (a.precond) {
+    const double k0r = a.c.k0 / a.c.ke;
+    while (!done && it < a.maxit) {
+      if (a.fused ? !apply_precond_fused(a, epoch) : !apply_precond(a, epoch)) return;
+      if (!cg_barrier(a, epoch)) return;
+      const double rl = defect_update(a, fresh, k0r);
+      fresh = false;
       const double s = block_sum(rl, smem);
-      if (threadIdx.x == 0) partB[a.vb] = s;
+      if (threadIdx.x == 0) partA[a.vb] = s;
+      if (!cg_barrier(a, epoch)) return;
+      const double rr_new = block_sum_array(partA, nb, smem);
+      ++it;
+      if (!isfinite(rr_new)) { bad = true; break; }
+      const bool slow = rr_new > 0.25 * rr;
+      rr = rr_new;
+      done = !(rr > thr);
+      if (slow) break;
     }
-    if (!grid_barrier_n(a.bar, a.status, a.vnb)) return;
-    const double rr_new = block_sum_array(partB, nb, smem);
-    if (!isfinite(rr_new)) { bad = true; break; }
-    double rho_new = rr_new;
-    if (a.precond && rr_new > thr) {
-      double rz_l = 0.0;
-      if (a.fused ? !apply_precond_fused(a, &rz_l) : !apply_precond(a, &rz_l)) return;
-      const double s = block_sum(rz_l, smem);
-      if (threadIdx.x == 0) partC[a.vb] = s;
-      if (!grid_barrier_n(a.bar, a.status, a.vnb)) return;
-      rho_new = block_sum_array(partC, nb, smem);
-      if (!isfinite(rho_new)) { bad = true; break; }
+  }
+  if (fresh) {
+    for (long long k = tid; k < a.n; k += stride) a.x[k] = 0.0;
+  }
+  if (!done && !bad && it < a.maxit) {
+    // conjugate gradients: each iteration applies the stiffness once, q = K p
+    // carried as q = K s + beta q_old (K p by linearity, p = s + beta p_old)
+    const double *s_vec = a.r;
+    double rho_cg = rr, beta = 0.0;
+    double *pold = a.pa, *pnew = a.pb;
+    for (int j = 0; rr > thr && it < a.maxit; ++j, ++it) {
+      // phase 1: p = s + beta p_old and q = K s + beta q_old (own nodes), p.q
+      double pq_l = 0.0;
+      for (long long k = tid; k < a.n; k += stride) {
+        const int ix = (int)(k % N), iy = (int)((k / N) % N), iz = (int)(k / NN);
+        double sk;
+        const double ks = stiff_apply<false>(s_vec, nullptr, 0.0, N, ix, iy, iz, a.c, &sk);
+        const double pk = j == 0 ? sk : fma(beta, pold[k], sk);
+        const double qk = j == 0 ? ks : fma(beta, a.q[k], ks);
+        pnew[k] = pk;
+        a.q[k] = qk;
+        pq_l = fma(pk, qk, pq_l);
+      }
+      {
+        const double s = block_sum(pq_l, smem);
+        if (threadIdx.x == 0) partC[a.vb] = s;
+      }
+      if (!cg_barrier(a, epoch)) return;
+      const double pq = block_sum_array(partC, nb, smem);
+      if (!(pq > 0.0) || !isfinite(pq)) { bad = true; break; }
+      const double alpha = rho_cg / pq;
+      // phase 2: x += alpha p, r -= alpha q, r.r
+      double rl = 0.0;
+      for (long long k = tid; k < a.n; k += stride) {
+        a.x[k] = fma(alpha, pnew[k], a.x[k]);
+        const double rk = fma(-alpha, a.q[k], a.r[k]);
+        a.r[k] = rk;
+        rl = fma(rk, rk, rl);
+      }
+      {
+        const double s = block_sum(rl, smem);
+        if (threadIdx.x == 0) partB[a.vb] = s;
+      }
+      if (!cg_barrier(a, epoch)) return;
+      const double rr_new = block_sum_array(partB, nb, smem);
+      if (!isfinite(rr_new)) { bad = true; break; }
+      beta = rr_new / rho_cg;
+      rho_cg = rr_new;
+      rr = rr_new;
+      double *tmp = pold; pold = pnew; pnew = tmp;
     }
-    beta = rho_new / rho_cg;
-    rho_cg = rho_new;
-    rr = rr_new;
-    double *t = pold; pold = pnew; pnew = t;
-    ++it;
   }
   if (a.vb == 0 && threadIdx.x == 0) {
     *a.iters_out = (double)it;
@@ -600,6 +845,7 @@ ks_status launch_cg(Problem &P, const double *rho, double *v, double *r, bool wa
   a.r = r;
   a.pa = P.cg_pa;
   a.pb = P.cg_pb;
+  a.r32 = reinterpret_cast<float *>(P.cg_pa);
   a.q = P.cg_q;
   a.z = P.cg_z;
   a.t1 = P.cg_t1;
@@ -636,16 +882,18 @@ ks_status launch_cg(Problem &P, const double *rho, double *v, double *r, bool wa
 }
 
 // ---------------------------------------------------------------- batched
-// The PCG of every job of a batch, one launch per CG phase over all jobs
+// The solve of every job of a batch, one launch per phase over all jobs
 // (no grid barrier: a phase's last block of each job finishes that job's
 // reductions and scalar updates in device memory).  Phases:
-//   init   r = b - K x (x = 0 when cold), r.r, b.b, tolerance
-//   A/B/C  the fused sine-basis preconditioner, one block per (job, plane)
-//          resp. (job, y-slab); C writes z and r.z and updates rho, beta
-//   it1    p = s + beta p_old, q = K p, p.q -> alpha
-//   it2    x += alpha p, r -= alpha q, r.r -> convergence
+//   init     r = b - K x (x = 0 when cold), r.r, b.b, tolerance
+//   A/B/C    the fused sine-basis transforms, one block per (job, plane)
+//            resp. (job, ky); C writes z
+//   update   x += z, r -= K z, r.r -> convergence
+//   it1, it2 a CG iteration, for jobs without the preconditioner only
+//            (launched when there is such a job): p = r + beta p_old, q = K p,
+//            p.q -> alpha; x += alpha p, r -= alpha q, r.r
 // A job that has converged (or failed) skips every later phase.  The host
-// reads the number of jobs still iterating once per CG iteration.
+// reads the number of jobs still iterating once per iteration.
 struct CgState {
   double rr, bb, thr, rho, beta, alpha;
   int it, done, maxit, precond;
@@ -710,6 +958,7 @@ __global__ void __launch_bounds__(kCgThreads) cg_b_init(CgBatchView v) {
     }
     const double rk = b - kx;
     a.r[k] = rk;
+    if (a.precond) a.r32[k] = (float)rk;
     rr_l = fma(rk, rk, rr_l);
     bb_l = fma(b, b, bb_l);
   }
@@ -736,12 +985,11 @@ __global__ void __launch_bounds__(kCgThreads) cg_b_init(CgBatchView v) {
   }
 }
 
-// Preconditioner passes (fused form; jobs with N > kFusedMaxN are refused at
-// batch creation).  Stage 0: planes of r -> t1; 1: slabs t1 -> t2; 2: planes
-// t2 -> z with r.z, then rho and beta.
+// Transform phases (fused form; jobs with N > kFusedMaxN are refused at batch
+// creation).  Stage 0: r32 -> t1 (in-plane modes); 1: t1 -> t2 (along z); 2:
+// t2 -> z.
 template <int Stage>
 __global__ void __launch_bounds__(kCgThreads) cg_b_precond(CgBatchView v) {
-  __shared__ double smem[33];
   extern __shared__ float dyn[];
   int j, vb, nb;
   if (!cg_job(v, j, vb, nb)) return;
@@ -749,28 +997,46 @@ __global__ void __launch_bounds__(kCgThreads) cg_b_precond(CgBatchView v) {
   if (!v.st[j].precond) return;
   a.vb = vb;
   a.vnb = nb;
-  load_phi(a, dyn);
+  load_phi(a, dyn, Stage <= 1, Stage >= 1);
+  const bool s = small_tiles(a.N);
   if (Stage == 0) {
-    fused_plane_pass<true, false>(a, a.r, a.t1, nullptr, dyn);
+    if (s) fused_pass_a<2>(a, a.r32, a.t1, dyn); else fused_pass_a<4>(a, a.r32, a.t1, dyn);
   } else if (Stage == 1) {
-    fused_slab_pass(a, a.t1, a.t2, dyn);
+    if (s) fused_pass_b<2>(a, a.t1, a.t2, dyn); else fused_pass_b<4>(a, a.t1, a.t2, dyn);
   } else {
-    const double rz_l = fused_plane_pass<false, true>(a, a.t2, nullptr, a.z, dyn);
-    const double sum = block_sum(rz_l, smem);
-    if (threadIdx.x == 0) a.part[vb] = sum;
-    double s[1];
-    if (!job_tail(a.part, nb, 1, v.counters + j, smem, s)) return;
-    if (threadIdx.x == 0) {
-      CgState &t = v.st[j];
-      if (!isfinite(s[0])) {
-        t.done = 1;
-        atomicCAS(a.status, 0, (int)KS_ENAN);
-      } else {
-        t.beta = t.it == 0 ? 0.0 : s[0] / t.rho;
-        t.rho = s[0];
-      }
-    }
+    if (s) fused_pass_c<2>(a, a.t2, a.z, dyn); else fused_pass_c<4>(a, a.t2, a.z, dyn);
   }
+}
+
+// One job's residual norm after a step: convergence, limits, failure.
+__device__ __forceinline__ void cg_step_done(const CgArgs &a, CgState &u, double rr) {
+  ++u.it;
+  u.rr = rr;
+  *a.iters_out = (double)u.it;
+  if (!isfinite(rr)) {
+    u.done = 1;
+    atomicCAS(a.status, 0, (int)KS_ENAN);
+  } else if (rr <= u.thr) {
+    u.done = 1;
+  } else if (u.it >= u.maxit) {
+    u.done = 1;
+    atomicCAS(a.status, 0, (int)KS_ENOCONV);
+  }
+}
+
+__global__ void __launch_bounds__(kCgThreads) cg_b_update(CgBatchView v) {
+  __shared__ double smem[33];
+  int j, vb, nb;
+  if (!cg_job(v, j, vb, nb)) return;
+  CgArgs a = v.args[j];
+  if (!v.st[j].precond) return;
+  a.vb = vb;
+  a.vnb = nb;
+  const double sum = block_sum(defect_update(a, false, a.c.k0 / a.c.ke), smem);
+  if (threadIdx.x == 0) a.part[vb] = sum;
+  double s[1];
+  if (!job_tail(a.part, nb, 1, v.counters + j, smem, s)) return;
+  if (threadIdx.x == 0) cg_step_done(a, v.st[j], s[0]);
 }
 
 __global__ void __launch_bounds__(kCgThreads) cg_b_it1(CgBatchView v) {
@@ -779,9 +1045,10 @@ __global__ void __launch_bounds__(kCgThreads) cg_b_it1(CgBatchView v) {
   if (!cg_job(v, j, vb, nb)) return;
   const CgArgs &a = v.args[j];
   const CgState t = v.st[j];
+  if (t.precond) return;
   const int N = a.N;
   const long long NN = (long long)N * N;
-  const double *s_vec = t.precond ? a.z : a.r;
+  const double *s_vec = a.r;
   double *pold = (t.it % 2 == 0) ? a.pb : a.pa, *pnew = (t.it % 2 == 0) ? a.pa : a.pb;
   double pq_l = 0.0;
   for (long long k = (long long)vb * blockDim.x + threadIdx.x; k < a.n;
@@ -815,6 +1082,7 @@ __global__ void __launch_bounds__(kCgThreads) cg_b_it2(CgBatchView v) {
   if (!cg_job(v, j, vb, nb)) return;
   const CgArgs &a = v.args[j];
   const CgState t = v.st[j];
+  if (t.precond) return;
   const double *p = (t.it % 2 == 0) ? a.pa : a.pb;
   double rl = 0.0;
   for (long long k = (long long)vb * blockDim.x + threadIdx.x; k < a.n;
@@ -830,21 +1098,9 @@ __global__ void __launch_bounds__(kCgThreads) cg_b_it2(CgBatchView v) {
   if (!job_tail(a.part, nb, 1, v.counters + j, smem, s)) return;
   if (threadIdx.x == 0) {
     CgState &u = v.st[j];
-    ++u.it;
-    u.rr = s[0];
-    *a.iters_out = (double)u.it;
-    if (!isfinite(s[0])) {
-      u.done = 1;
-      atomicCAS(a.status, 0, (int)KS_ENAN);
-    } else if (s[0] <= u.thr) {
-      u.done = 1;
-    } else if (u.it >= u.maxit) {
-      u.done = 1;
-      atomicCAS(a.status, 0, (int)KS_ENOCONV);
-    } else if (!u.precond) {
-      u.beta = s[0] / u.rho;
-      u.rho = s[0];
-    }
+    cg_step_done(a, u, s[0]);
+    u.beta = s[0] / u.rho;
+    u.rho = s[0];
   }
 }
 
@@ -884,6 +1140,7 @@ ks_status batch_cg_setup(Batch &B) {
     a.r = P.cg_r;
     a.pa = P.cg_pa;
     a.pb = P.cg_pb;
+    a.r32 = reinterpret_cast<float *>(P.cg_pa);
     a.q = P.cg_q;
     a.z = P.cg_z;
     a.t1 = P.cg_t1;
@@ -923,7 +1180,7 @@ ks_status batch_cg_setup(Batch &B) {
 // relative residual max(tol, the job's cg_tol), in three pieces so that the
 // launches can be captured in a CUDA graph:
 //   batch_cg_upload   per-job tolerance and warm flag (host -> device)
-//   batch_cg_launch   init + preconditioner + `iters` CG iterations and the
+//   batch_cg_launch   init + `iters` iterations and the
 //                     count of jobs still iterating (no host synchronisation)
 //   batch_cg_continue more iterations, one host check each, until no job is
 //                     left (after a synchronisation that read the count)
@@ -933,25 +1190,46 @@ static CgBatchView cg_view(Batch &B, int map) {
                      B.cg_tolw_dev, B.cg_counters};
 }
 
+void cg_batch_blocks(int N, long long *a, long long *bc, long long *update) {
+  *a = 4LL * N;
+  *bc = 2LL * N;
+  const long long uy = (N + kUpY - 1) / kUpY, uz = (N + kUpZ - 1) / kUpZ;
+  *update = (N * uy * uz + kCgThreads - 1) / kCgThreads;
+}
+
 static ks_status cg_precond_launch(Batch &B) {
-  const CgBatchView planes = cg_view(B, BM_CG_PLANES);
-  const int np = B.total(BM_CG_PLANES);
+  const CgBatchView va = cg_view(B, BM_CG_A), vbc = cg_view(B, BM_CG_BC);
+  const int na = B.total(BM_CG_A), nbc = B.total(BM_CG_BC);
   const size_t dyn = cg_dynamic_smem(B.maxN);
-  cg_b_precond<0><<<np, kCgThreads, dyn, B.stream>>>(planes);
-  cg_b_precond<1><<<np, kCgThreads, dyn, B.stream>>>(planes);
-  cg_b_precond<2><<<np, kCgThreads, dyn, B.stream>>>(planes);
+  cg_b_precond<0><<<na, kCgThreads, dyn, B.stream>>>(va);
+  cg_b_precond<1><<<nbc, kCgThreads, dyn, B.stream>>>(vbc);
+  cg_b_precond<2><<<nbc, kCgThreads, dyn, B.stream>>>(vbc);
   KS_CUDA_TRY(cudaGetLastError());
   return KS_OK;
 }
 
+// One step of every job still iterating: correction of the preconditioned
+// jobs, CG iteration of the others (none in the usual batch).
 static ks_status cg_iteration_launch(Batch &B) {
   const CgBatchView nodes = cg_view(B, BM_CG_NODES);
   const int nn = B.total(BM_CG_NODES);
-  ProfScope ps_(B.stream, KP_CG, 0.0, 0.0, 6);
-  cg_b_it1<<<nn, kCgThreads, 0, B.stream>>>(nodes);
-  cg_b_it2<<<nn, kCgThreads, 0, B.stream>>>(nodes);
+  bool plain = false, pre = false;
+  for (int j = 0; j < B.J; ++j) (B.probs[j]->P.cg_precond ? pre : plain) = true;
+  ProfScope ps_(B.stream, KP_CG, 0.0, 0.0, (pre ? 4 : 0) + (plain ? 2 : 0));
+  if (pre) {
+    KS_TRY(cg_precond_launch(B));
+    cg_b_update<<<B.total(BM_CG_UPDATE), kCgThreads, 0, B.stream>>>(cg_view(B, BM_CG_UPDATE));
+  }
+  if (plain) {
+    cg_b_it1<<<nn, kCgThreads, 0, B.stream>>>(nodes);
+    cg_b_it2<<<nn, kCgThreads, 0, B.stream>>>(nodes);
+  }
   KS_CUDA_TRY(cudaGetLastError());
-  KS_TRY(cg_precond_launch(B));
+  return KS_OK;
+}
+
+static ks_status cg_count_launch(Batch &B) {
+  ProfScope ps_(B.stream, KP_CG);
   cg_b_count<<<1, 256, 0, B.stream>>>(static_cast<const CgState *>(B.cg_state_dev), B.active_dev,
                                       B.J, B.cg_remaining_dev);
   KS_CUDA_TRY(cudaGetLastError());
@@ -972,16 +1250,12 @@ ks_status batch_cg_upload(Batch &B, double tol) {
 ks_status batch_cg_launch(Batch &B, int iters) {
   const CgBatchView nodes = cg_view(B, BM_CG_NODES);
   {
-    ProfScope ps_(B.stream, KP_CG, 0.0, 0.0, 5);
+    ProfScope ps_(B.stream, KP_CG);
     cg_b_init<<<B.total(BM_CG_NODES), kCgThreads, 0, B.stream>>>(nodes);
-    KS_CUDA_TRY(cudaGetLastError());
-    KS_TRY(cg_precond_launch(B));
-    cg_b_count<<<1, 256, 0, B.stream>>>(static_cast<const CgState *>(B.cg_state_dev),
-                                        B.active_dev, B.J, B.cg_remaining_dev);
     KS_CUDA_TRY(cudaGetLastError());
   }
   for (int it = 0; it < iters; ++it) KS_TRY(cg_iteration_launch(B));
-  return KS_OK;
+  return cg_count_launch(B);
 }
 
 ks_status batch_cg_continue(Batch &B) {
@@ -994,6 +1268,7 @@ ks_status batch_cg_continue(Batch &B) {
     KS_CUDA_TRY(cudaStreamSynchronize(B.stream));
     if (*B.cg_remaining_host == 0) break;
     KS_TRY(cg_iteration_launch(B));
+    KS_TRY(cg_count_launch(B));
   }
   return KS_OK;
 }
@@ -1021,7 +1296,10 @@ int cg_grid_blocks(int sms, int n, int N) {
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cg_kernel, kCgThreads, dyn) !=
       cudaSuccess || per_sm < 1)
     per_sm = 1;
+  // a block per item of the transforms' widest phase, or enough blocks for the
+  // nodes; more would only make the barriers dearer
   long long want = (n + kCgThreads - 1) / kCgThreads;
+  if (N <= kFusedMaxN && want < 4LL * N) want = 4LL * N;
   long long cap = (long long)sms * (per_sm < 2 ? per_sm : 2);
   if (want > cap) want = cap;
   if (want < 1) want = 1;

@@ -239,6 +239,9 @@ ks_status launch_qr_exact_gram(Problem &P, const double *R, const double *T, dou
 ks_status launch_cg(Problem &P, const double *rho, double *v, double *r, bool warm);
 ks_status launch_sine_setup(Problem &P);
 int cg_grid_blocks(int sms, int n, int N);
+// blocks of one job in the batched transforms' passes A and B/C (one item each)
+// and in the update (kUpY x kUpZ nodes per thread)
+void cg_batch_blocks(int N, long long *a, long long *bc, long long *update);
 ks_status launch_gram_oz(Problem &P, const double *A, int pa, const double *B, int qb,
                          int *emax, double *part, int chunks);
 int gram_oz_chunks(const Problem &P, int pa, int qb);
@@ -429,7 +432,7 @@ struct BJob {
 // each job takes in a launch family.
 enum BMap {
   BM_DENSITY = 0, BM_POTENTIAL, BM_ST4, BM_ST8, BM_ST16, BM_ST32, BM_THOMAS, BM_GRAM_SMALL,
-  BM_GRAM_MID, BM_GRAM_TILED, BM_GRAM_REDUCE, BM_CG_NODES, BM_CG_PLANES, BM_COMB_NARROW, BM_COMB_TILED, BM_COEF, BM_COPY, BM_COUNT
+  BM_GRAM_MID, BM_GRAM_TILED, BM_GRAM_REDUCE, BM_CG_NODES, BM_CG_A, BM_CG_BC, BM_CG_UPDATE, BM_COMB_NARROW, BM_COMB_TILED, BM_COEF, BM_COPY, BM_COUNT
 };
 
 // Launch shapes of the batched kernels that the autotuner chooses.
