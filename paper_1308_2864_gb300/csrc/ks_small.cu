@@ -7,6 +7,8 @@
 //   cayley_factor: LU with partial pivoting of I + tau/2 V^T U (2p x 2p) and
 //                  the solve against V^T Y (Eq. WY3); for p = 1 the closed
 //                  form of Lemma 3.1 (3) (Eq. WY-1d), no solve.
+#include <algorithm>
+
 #include "ks_device.cuh"
 
 namespace ks {
@@ -307,6 +309,16 @@ ks_status batch_qr_factor(Batch &B, int smDMD, int smO, bool with_tau, int smC1,
   return KS_OK;
 }
 
+// 2p x 3p system, permutation and reciprocal pivots of the Cayley step
+constexpr int kCayleySmemP = 68;
+static size_t cayley_smem(int p, bool in_smem) {
+  const size_t n2 = 2 * (size_t)p;
+  return (n2 + p + (in_smem ? n2 * 3 * p : 0)) * sizeof(double);
+}
+__global__ void cayley_factor_kernel(int p, const double *A, const double *S, const double *B,
+                                     const double *O, double tau, double *Wg, int in_smem,
+                                     double *C1, double *C2, int *status);
+
 // Opt the shared-memory factor kernel into its dynamic shared memory (on the
 // current device; called when a problem is created).
 ks_status configure_small_kernels() {
@@ -315,6 +327,9 @@ ks_status configure_small_kernels() {
                                    cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   KS_CUDA_TRY(cudaFuncSetAttribute(qr_factor_batch_kernel,
                                    cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  KS_CUDA_TRY(cudaFuncSetAttribute(cayley_factor_kernel,
+                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)cayley_smem(kCayleySmemP, true)));
   return KS_OK;
 }
 
@@ -343,14 +358,25 @@ ks_status launch_qr_factor(Problem &P, const double *DMD, const double *O, doubl
 
 // Solve (I + tau/2 N) P = R with N = [[A, O], [-B, -S]] and R = [O; -S]
 // (all p x p blocks, O = I when null), by Gaussian elimination with partial
-// pivoting on the augmented 2p x 3p matrix W.
-__global__ void __launch_bounds__(kSmallThreads) cayley_factor_kernel(
+// pivoting on the augmented 2p x 3p matrix W, in shared memory up to
+// p = kCayleySmemP (2p x 3p doubles in 227 KiB), in global scratch above.
+//
+// One CTA, bound by its SM's FP64 pipe and by the pivot steps' latency.  A
+// step is two block barriers: warp 0 finds the pivot and its reciprocal
+// (rows are exchanged in the permutation only), then each warp takes whole
+// rows, one multiplier per row and one FMA per entry.  (With a division per
+// entry, some 25 FP64 instructions, the step took 823 us at p = 30, now about
+// 200.)  The back substitution is column-oriented for the same reason: every
+// row above takes its update as soon as an unknown is final, so no thread
+// runs a chain of 2p^2 dependent FMAs.
+constexpr int kCayleyThreads = 512;      // 16 warps fill the FP64 pipe; no spills
+
+__global__ void __launch_bounds__(kCayleyThreads) cayley_factor_kernel(
     int p, const double *A, const double *S, const double *B, const double *O, double tau,
-    double *W, double *C1, double *C2, int *status) {
-  __shared__ double s_val[32];
-  __shared__ int s_idx[32];
-  __shared__ int s_piv;
+    double *Wg, int in_smem, double *C1, double *C2, int *status) {
+  extern __shared__ __align__(16) double cy_smem[];
   __shared__ int s_fail;
+  __shared__ double s_inv;
   const int n2 = 2 * p, w = 3 * p;
   const double ht = 0.5 * tau;
   if (p == 1) {
@@ -372,6 +398,10 @@ __global__ void __launch_bounds__(kSmallThreads) cayley_factor_kernel(
     }
     return;
   }
+  // shared: permutation (n2 ints), reciprocal pivots (n2), then W when it fits
+  double *inv = cy_smem;
+  int *perm = reinterpret_cast<int *>(cy_smem + n2);
+  double *W = in_smem ? cy_smem + n2 + p : Wg;
   for (int e = threadIdx.x; e < n2 * w; e += blockDim.x) {
     const int i = e / w, j = e % w;
     double v;
@@ -390,69 +420,65 @@ __global__ void __launch_bounds__(kSmallThreads) cayley_factor_kernel(
     }
     W[e] = v;
   }
+  for (int i = threadIdx.x; i < n2; i += blockDim.x) perm[i] = i;
   if (threadIdx.x == 0) s_fail = 0;
   __syncthreads();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   for (int j = 0; j < n2; ++j) {
-    // pivot search over rows j..n2-1 (largest |W[i][j]|, lowest index on ties)
-    double best = -1.0;
-    int bi = n2;
-    for (int i = j + threadIdx.x; i < n2; i += blockDim.x) {
-      const double a = fabs(W[i * w + j]);
-      if (a > best) { best = a; bi = i; }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const double ob = __shfl_xor_sync(0xffffffffu, best, o);
-      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-      if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-    }
-    if (lane == 0) { s_val[warp] = best; s_idx[warp] = bi; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double bb = -1.0;
-      int ib = n2;
-      for (int t = 0; t < (int)(blockDim.x >> 5); ++t)
-        if (s_val[t] > bb || (s_val[t] == bb && s_idx[t] < ib)) { bb = s_val[t]; ib = s_idx[t]; }
-      if (!(bb > 1e-300) || !isfinite(bb)) {
-        s_fail = 1;
-        atomicCAS(status, 0, (int)KS_ESINGULAR);
+    if (warp == 0) {
+      // largest |W[i][j]| over the remaining rows, the lowest position on ties
+      double best = -1.0;
+      int bi = n2;
+      for (int i = j + lane; i < n2; i += 32) {
+        const double a = fabs(W[perm[i] * w + j]);
+        if (a > best) { best = a; bi = i; }
       }
-      s_piv = ib;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+        if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
+      }
+      if (lane == 0) {
+        if (!(best > 1e-300) || !isfinite(best)) {
+          s_fail = 1;
+          atomicCAS(status, 0, (int)KS_ESINGULAR);
+        } else {
+          const int t = perm[j];
+          perm[j] = perm[bi];
+          perm[bi] = t;
+          s_inv = inv[j] = 1.0 / W[perm[j] * w + j];
+        }
+      }
     }
     __syncthreads();
     if (s_fail) return;
-    const int pv = s_piv;
-    if (pv != j) {
-      for (int c = threadIdx.x; c < w; c += blockDim.x) {
-        const double t = W[j * w + c];
-        W[j * w + c] = W[pv * w + c];
-        W[pv * w + c] = t;
-      }
-      __syncthreads();
-    }
-    const double d = W[j * w + j];
-    const int rows = n2 - j - 1, cols = w - j - 1;
-    for (int t = threadIdx.x; t < rows * cols; t += blockDim.x) {
-      const int i = j + 1 + t / cols, c = j + 1 + t % cols;
-      W[i * w + c] = fma(-W[i * w + j] / d, W[j * w + c], W[i * w + c]);
+    const double d = s_inv;
+    const double *pr = W + perm[j] * w;
+    for (int i = j + 1 + warp; i < n2; i += nw) {
+      double *row = W + perm[i] * w;
+      const double l = -(row[j] * d);
+      for (int c = j + 1 + lane; c < w; c += 32) row[c] = fma(l, pr[c], row[c]);
     }
     __syncthreads();
   }
-  // back substitution, one right-hand side column per thread
-  for (int c = threadIdx.x; c < p; c += blockDim.x) {
-    const int col = n2 + c;
-    for (int i = n2 - 1; i >= 0; --i) {
-      double s = W[i * w + col];
-      for (int k = i + 1; k < n2; ++k) s = fma(-W[i * w + k], W[k * w + col], s);
-      W[i * w + col] = s / W[i * w + i];
+  // back substitution: row i's unknowns are final once it is scaled; the rows
+  // above subtract them at once
+  for (int i = n2 - 1; i >= 0; --i) {
+    double *ri = W + perm[i] * w;
+    const double d = inv[i];
+    for (int k = i - 1 - warp; k >= 0; k -= nw) {
+      double *row = W + perm[k] * w;
+      const double l = -(row[i] * d);
+      for (int c = n2 + lane; c < w; c += 32) row[c] = fma(l, ri[c], row[c]);
     }
+    __syncthreads();
   }
-  __syncthreads();
   // X+ = X (I - tau P2) + G (-tau P1)
   for (int e = threadIdx.x; e < p * p; e += blockDim.x) {
     const int i = e / p, j = e % p;
-    const double p1 = W[i * w + n2 + j], p2 = W[(p + i) * w + n2 + j];
+    const double p1 = W[perm[i] * w + n2 + j] * inv[i];
+    const double p2 = W[perm[p + i] * w + n2 + j] * inv[p + i];
     C1[e] = (i == j ? 1.0 : 0.0) - tau * p2;
     C2[e] = -tau * p1;
   }
@@ -460,10 +486,13 @@ __global__ void __launch_bounds__(kSmallThreads) cayley_factor_kernel(
 
 ks_status launch_cayley_factor(Problem &P, const double *A, const double *S, const double *B,
                                const double *O, double tau, double *C1, double *C2) {
+  const bool in_smem = P.p <= kCayleySmemP;
+  // a warp per row of the first step, at most the whole block
+  const int threads = std::min(kCayleyThreads, 32 * std::max(1, 2 * P.p - 1));
   {
     ProfScope ps_(P.stream, KP_SMALL);
-    cayley_factor_kernel<<<1, kSmallThreads, 0, P.stream>>>(P.p, A, S, B, O, tau, P.pp, C1, C2,
-                                                            P.dstatus);
+    cayley_factor_kernel<<<1, threads, cayley_smem(P.p, in_smem), P.stream>>>(
+        P.p, A, S, B, O, tau, P.pp, in_smem ? 1 : 0, C1, C2, P.dstatus);
   }
   KS_CUDA_TRY(cudaGetLastError());
   return KS_OK;

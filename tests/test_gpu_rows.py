@@ -70,3 +70,18 @@ def test_retract_takes_any_derivative_block():
         with pytest.raises(ks.KSError) as e:
             P.retract(kind, dev(X), dev(bad), 1e-3)
         assert e.value.status == ks.KS_ENAN
+
+
+@pytest.mark.parametrize("p", [2, 3, 4, 17, 68, 69])
+def test_cayley_factor_sizes(p):
+    # 68 | 69: the 2p x 3p system in shared memory | in global scratch; a large step, so
+    # that rows are exchanged.  1e-11: as the other retractions above
+    import paper_1308_2864_gb300 as ks
+    s = ki.small_system(N=9, L=5.0, natoms=2, p=p, Z=4.0, seed=60 + p)
+    model = oe.Model.from_system(s)
+    X = ost.m_orthonormalize(model, s.x0())
+    pt = ost.point_at(model, X)
+    P = ks.Problem.from_system(s, cg_tol=1e-13)
+    for tau in (1e-3, 0.5):
+        got = P.retract(ks.KS_CAYLEY, dev(X), dev(pt.ev.EX), tau).cpu().numpy()
+        assert_rel(got, ost.retract_cayley(model, pt, tau), 1e-11, f"tau {tau}")
