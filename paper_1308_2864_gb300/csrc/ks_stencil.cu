@@ -192,7 +192,9 @@ struct StCols {
       const T faces = f_mid[r] + (c_old[r] + c_new[r]);
       const T edges = e_mid[r] + (f_old[r] + f_new[r]);
       const T corners = e_old[r] + e_new[r];
-      return fma(cf.mc, corners, fma(cf.me, edges, fma(cf.m0, c_mid[r], cf.mf * faces)));
+      // (the order of the first two products is part of the FP32 result)
+      const T mcf = kHam ? fma(cf.m0, c_mid[r], cf.mf * faces) : fma(cf.mf, faces, cf.m0 * c_mid[r]);
+      return fma(cf.mc, corners, fma(cf.me, edges, mcf));
     }
   }
   // K A, in units of ke for FP64
