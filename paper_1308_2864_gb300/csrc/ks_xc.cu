@@ -17,19 +17,57 @@ constexpr double kPzDen1 = 1.0 + kPzBeta1 + kPzBeta2;
 constexpr double kPzD = kPzGamma / kPzDen1 - kPzB;
 constexpr double kPzC = -kPzGamma * (0.5 * kPzBeta1 + kPzBeta2) / (kPzDen1 * kPzDen1) - kPzA - kPzD;
 
-// rho^(-1/3) for rho >= 1e-30: single-precision start, then two Newton steps
-// on f(z) = z^-3 - rho, z <- z (4 - rho z^3) / 3 (no division; each step
-// squares the relative error, 1e-7 -> 1e-14 -> below FP64 rounding).  On
-// GB300 every FP64 instruction is a 16-cycle issue, so this replaces two
-// library cube roots and three divisions per point.
+// Elementary functions of the FP64 potential.  On GB300 every FP64 warp
+// instruction holds the pipe for 16 clocks and the kernel is bound by it, so
+// each function is a single-precision start (relative error e ~ 1e-7) and one
+// third-order step of the binomial series, which leaves e^3 ~ 1e-21, below
+// FP64 rounding: with e = 1 - rho z^3, (1 - e)^(-1/3) = 1 + e/3 + 2 e^2/9 + ...
+// With library log, rsqrt and division and two Newton steps per cube root
+// (taken twice in the orbital-free model) the kernel took 200 us at 105^3.
+// rho^(-1/3) for rho >= 1e-30 (six FP64 instructions; two Newton steps took ten)
 __device__ __forceinline__ double inv_cbrt(double rho) {
-  double z = (double)rcbrtf((float)rho);
-#pragma unroll
-  for (int it = 0; it < 2; ++it) {
-    const double z3 = z * z * z;
-    z = z * fma(-rho, z3, 4.0) * (1.0 / 3.0);
-  }
-  return z;
+  const double z = (double)rcbrtf((float)rho);
+  const double e = fma(-rho, z * z * z, 1.0);
+  return fma(z, e * fma(2.0 / 9.0, e, 1.0 / 3.0), z);
+}
+
+// x^(-1/2): e = 1 - x y^2, (1 - e)^(-1/2) = 1 + e/2 + 3 e^2/8 + ...
+__device__ __forceinline__ double inv_sqrt(double x) {
+  const double y = (double)rsqrtf((float)x);
+  const double e = fma(-x, y * y, 1.0);
+  return fma(y, e * fma(0.375, e, 0.5), y);
+}
+
+// 1 / x: e = 1 - x y, (1 - e)^(-1) = 1 + e + e^2 + ...
+__device__ __forceinline__ double inv_of(double x) {
+  const double y = (double)__frcp_rn((float)x);
+  const double e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+}
+
+// ln x for normal x > 0: x = 2^k m with m in [sqrt(1/2), sqrt(2)), and the
+// area-tangent series ln m = 2 (s + s^3/3 + s^5/5 + ...), s = (m - 1)/(m + 1),
+// |s| <= 0.1716: the terms through s^21 leave 2 s^23/23 < 3e-19.
+__device__ __forceinline__ double ln_series(double x) {
+  const long long bits = __double_as_longlong(x);
+  // exponent of x / sqrt(1/2), by its high word (sqrt(1/2) = 0x3fe6a09e...)
+  const int hi = (int)(bits >> 32);
+  const int k = (hi - 0x3fe6a09e) >> 20;
+  const double m = __longlong_as_double(bits - ((long long)k << 52));
+  const double s = (m - 1.0) * inv_of(m + 1.0);
+  const double q = s * s;
+  double t = 1.0 / 21.0;
+  t = fma(t, q, 1.0 / 19.0);
+  t = fma(t, q, 1.0 / 17.0);
+  t = fma(t, q, 1.0 / 15.0);
+  t = fma(t, q, 1.0 / 13.0);
+  t = fma(t, q, 1.0 / 11.0);
+  t = fma(t, q, 1.0 / 9.0);
+  t = fma(t, q, 1.0 / 7.0);
+  t = fma(t, q, 0.2);
+  t = fma(t, q, 1.0 / 3.0);
+  const double s2 = s + s;
+  return fma((double)k, 0.69314718055994530942, fma(s2 * q, t, s2));
 }
 
 // eps_xc and v_xc = d(rho eps_xc)/d rho at one point, in precision R
@@ -39,8 +77,10 @@ __device__ __forceinline__ double inv_cbrt(double rho) {
 //   PZ81 (r_s = (3 / (4 pi rho))^(1/3)): eps_c = gamma / (1 + beta1 sqrt(r_s)
 //   + beta2 r_s) for r_s >= 1, A ln r_s + B + C r_s ln r_s + D r_s below;
 //   v_c = eps_c - (r_s / 3) d eps_c / d r_s.
+// z: rho^(-1/3) where rho >= 1e-30, for the Thomas-Fermi term.
 template <typename R>
-__device__ __forceinline__ void lda_point(double rho_d, int xc, R &eps, R &v) {
+__device__ __forceinline__ void lda_point(double rho_d, int xc, R &eps, R &v, R &z) {
+  z = 0;
   if (!(rho_d >= 1e-30)) {
     eps = 0;
     v = 0;
@@ -49,7 +89,6 @@ __device__ __forceinline__ void lda_point(double rho_d, int xc, R &eps, R &v) {
   const R c = (R)0.98474502184269654;              // (3/pi)^(1/3)
   const R crs = (R)0.62035049089940001;            // (3/(4 pi))^(1/3)
   const R rho = (R)rho_d;
-  R z;                                             // rho^(-1/3)
   if constexpr (sizeof(R) == 8) z = inv_cbrt(rho_d);
   else z = rcbrtf(rho);
   const R r13 = rho * z * z;                       // rho^(1/3)
@@ -60,22 +99,26 @@ __device__ __forceinline__ void lda_point(double rho_d, int xc, R &eps, R &v) {
     R ec, dec;
     if (rs >= (R)1) {
       R irs;                                       // 1 / sqrt(r_s)
-      if constexpr (sizeof(R) == 8) irs = rsqrt(rs);
+      if constexpr (sizeof(R) == 8) irs = inv_sqrt(rs);
       else irs = rsqrtf(rs);
       const R srs = rs * irs;
-      const R iden = (R)1 / ((R)1 + (R)kPzBeta1 * srs + (R)kPzBeta2 * rs);
+      R iden;
+      if constexpr (sizeof(R) == 8)
+        iden = inv_of((R)1 + (R)kPzBeta1 * srs + (R)kPzBeta2 * rs);
+      else iden = (R)1 / ((R)1 + (R)kPzBeta1 * srs + (R)kPzBeta2 * rs);
       ec = (R)kPzGamma * iden;
       dec = -(R)kPzGamma * ((R)(0.5 * kPzBeta1) * irs + (R)kPzBeta2) * (iden * iden);
     } else {
       R lrs;
-      if constexpr (sizeof(R) == 8) lrs = log(rs);
+      if constexpr (sizeof(R) == 8) lrs = ln_series(rs);
       else lrs = logf(rs);
       ec = (R)kPzA * lrs + (R)kPzB + (R)kPzC * rs * lrs + (R)kPzD * rs;
       // A / r_s = A rho^(1/3) / crs
       dec = (R)kPzA * (r13 * (R)(1.0 / 0.62035049089940001)) + (R)kPzC * (lrs + (R)1) + (R)kPzD;
     }
     eps += ec;
-    v += ec - (rs / (R)3) * dec;
+    if constexpr (sizeof(R) == 8) v += ec - (rs * (R)(1.0 / 3.0)) * dec;
+    else v += ec - (rs / (R)3) * dec;
   }
 }
 
@@ -83,16 +126,13 @@ __device__ __forceinline__ void lda_point(double rho_d, int xc, R &eps, R &v) {
 // derivative v_TF = (5/3) C_TF rho^(2/3) (the T_TF term of Eq. TFW), both 0
 // below the density floor; ctf = C_TF and vtf = (5/3) C_TF in precision R.
 template <typename R>
-__device__ __forceinline__ void tf_point(double rho_d, R ctf, R vtf, R &e, R &v) {
+__device__ __forceinline__ void tf_point(double rho_d, R z, R ctf, R vtf, R &e, R &v) {
   if (!(rho_d >= 1e-30)) {
     e = 0;
     v = 0;
     return;
   }
   const R rho = (R)rho_d;
-  R z;                                             // rho^(-1/3)
-  if constexpr (sizeof(R) == 8) z = inv_cbrt(rho_d);
-  else z = rcbrtf(rho);
   const R r23 = rho * z;                           // rho^(2/3)
   v = vtf * r23;
   e = ctf * rho * r23;
@@ -119,8 +159,8 @@ __device__ __forceinline__ void potential_body(long long n, double h3, int xc, i
   for (long long k = (long long)vb * blockDim.x + threadIdx.x; k < n;
        k += (long long)vnb * blockDim.x) {
     const double rk = rho[k], ve = vext[k];
-    R eps_r, vxc_r;
-    lda_point<R>(rk, xc, eps_r, vxc_r);
+    R eps_r, vxc_r, z_r;
+    lda_point<R>(rk, xc, eps_r, vxc_r, z_r);
     const double eps = (double)eps_r;
     double v = ve + (double)vxc_r;
     e_ext = fma(h3 * ve, rk, e_ext);
@@ -132,7 +172,7 @@ __device__ __forceinline__ void potential_body(long long n, double h3, int xc, i
     }
     if (ctf != 0.0) {
       R etf_r, vtf_p;
-      tf_point<R>(rk, ctf_r, vtf_r, etf_r, vtf_p);
+      tf_point<R>(rk, z_r, ctf_r, vtf_r, etf_r, vtf_p);
       v += (double)vtf_p;
       e_tf = fma(h3, (double)etf_r, e_tf);
     }
