@@ -620,6 +620,267 @@ __global__ void __launch_bounds__(kStThreads, 2) stencil_tma_kernel(const __grid
                    smem);
 }
 
+// ---------------------------------------------------------------- FP32, p >= 32
+// The TMA form in FP32 with 32-orbital chunks.  Memory should bound it (three
+// to nine blocks of 4 bytes per entry), but one entry at a time cost some 55
+// warp instructions per 32 entries and 1.9 loaded halo entries per node, and the
+// kernel ran at 3.6 TB/s, bound by issue.  Here a thread owns two adjacent
+// orbitals of a column of four nodes: 8-byte shared loads, packed FP32
+// arithmetic (add / mul / fma.rn.f32x2, the same roundings as the scalar
+// forms), column sums shared by the four nodes, offsets formed once per
+// kernel; the 8 x 8 node tile loads 1.6 halo entries per node.  96^3 x 128,
+// Hamiltonian with M X: 383 -> 278 us (3.6 -> 4.9 TB/s of 1.37 GB).
+struct StF2 {
+  static constexpr int TX = 8, TY = 8, PC = 32, HX = TX + 2, HY = TY + 2, R = 4;
+  static constexpr int BOX = HX * HY * PC, AUX = TX * TY * PC;       // floats
+  static_assert(BOX * 4 % 128 == 0 && AUX * 4 % 128 == 0, "stages stay 128-byte aligned");
+  static_assert(kStThreads == PC / 2 * TX * (TY / R), "one thread per orbital pair and column");
+};
+
+using f2_t = unsigned long long;
+__device__ __forceinline__ f2_t f2_add(f2_t a, f2_t b) {
+  f2_t d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ f2_t f2_mul(f2_t a, f2_t b) {
+  f2_t d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ f2_t f2_fma(f2_t a, f2_t b, f2_t c) {
+  f2_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ f2_t f2_dup(float x) {
+  f2_t d;
+  asm("mov.b64 %0, {%1, %1};" : "=l"(d) : "f"(x));
+  return d;
+}
+// a - b (one rounding)
+__device__ __forceinline__ f2_t f2_sub(f2_t a, f2_t b) { return f2_fma(b, f2_dup(-1.f), a); }
+__device__ __forceinline__ double f2_sum(f2_t a) {
+  float x, y;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(a));
+  return (double)x + (double)y;
+}
+
+template <int Kind>
+constexpr size_t st_f2_smem() {
+  return (size_t)kStStages * (StF2::BOX + st_naux<float, Kind>() * StF2::AUX) * sizeof(float) + 128;
+}
+
+template <int Kind>
+__global__ void __launch_bounds__(kStThreads, Kind == SK_MASS_BB ? 1 : 2)
+    stencil_f32x2_kernel(const __grid_constant__ StTmaArgs ta) {
+  using S = StF2;
+  constexpr int NAUX = st_naux<float, Kind>(), STAGE = S::BOX + NAUX * S::AUX, TXY = S::TX * S::TY;
+  constexpr bool kHam = Kind == SK_HAM || Kind == SK_HAM_INC;
+  extern __shared__ __align__(128) unsigned char st_ring_raw[];
+  float *ring =
+      reinterpret_cast<float *>(st_ring_raw + ((128u - (smem_addr(st_ring_raw) & 127u)) & 127u));
+  __shared__ __align__(8) uint64_t full[kStStages];
+  // SK_HAM: 2 f h^3 V; SK_HAM_INC: V, V_b and V - V_b (formed in FP64)
+  __shared__ float vs[kHam ? 3 : 1][kHam ? TXY : 1];
+  __shared__ float vbs[Kind == SK_HAM_INC ? 3 : 1][Kind == SK_HAM_INC ? TXY : 1];
+  __shared__ float dvs[Kind == SK_HAM_INC ? 3 : 1][Kind == SK_HAM_INC ? TXY : 1];
+  __shared__ double smem[33];
+  const StArgs &a = ta.a;
+  const int N = a.N, p = a.p;
+  int b = blockIdx.x;
+  const int x0 = b % a.tiles_x * S::TX; b /= a.tiles_x;
+  const int y0 = b % a.tiles_y * S::TY; b /= a.tiles_y;
+  const int o0 = b % a.chunks * S::PC; b /= a.chunks;
+  const int z0 = b * a.zseg;
+  const int z1 = min(z0 + a.zseg, N);
+  const int nplanes = z1 - z0 + 2;
+  const int pair = threadIdx.x % (S::PC / 2), col = threadIdx.x / (S::PC / 2);
+  const int lx = col % S::TX, ly = col / S::TX * S::R;
+
+  auto load_stage = [&](int q) {
+    float *dst = ring + (q % kStStages) * STAGE;
+    uint64_t *bar = &full[q % kStStages];
+    const bool with_aux = NAUX > 0 && q >= 2;
+    mbar_arrive_expect_tx(bar, (S::BOX + (with_aux ? NAUX * S::AUX : 0)) * 4u);
+    tma_load_4d(dst, &ta.map, bar, o0, x0 - 1, y0 - 1, z0 - 1 + q);
+    if (with_aux)
+#pragma unroll
+      for (int i = 0; i < NAUX; ++i)
+        tma_load_4d(dst + S::BOX + i * S::AUX, &ta.aux[i], bar, o0, x0, y0, z0 - 2 + q);
+  };
+  if (threadIdx.x == 0) {
+    prefetch_tensor_map(&ta.map);
+#pragma unroll
+    for (int i = 0; i < NAUX; ++i) prefetch_tensor_map(&ta.aux[i]);
+#pragma unroll
+    for (int st = 0; st < kStStages; ++st) mbar_init(&full[st], 1);
+    fence_barrier_init();
+  }
+  __syncthreads();
+  if (threadIdx.x == 0)
+    for (int q = 0; q < kStStages && q < nplanes; ++q) load_stage(q);
+
+  // V_eff of plane z0 - 1 + q, read one step ahead by the thread that owns the node
+  const int vx = x0 + (int)threadIdx.x % S::TX, vy = y0 + (int)threadIdx.x / S::TX;
+  const bool vown = kHam && (int)threadIdx.x < TXY && vx < N && vy < N;
+  const long long NN = (long long)N * N;
+  double vreg = 0.0, vbreg = 0.0;
+  if (vown && z0 >= 1) {
+    vreg = a.veff[(z0 - 1) * NN + (long long)vy * N + vx];
+    if (Kind == SK_HAM_INC) vbreg = a.veff_b[(z0 - 1) * NN + (long long)vy * N + vx];
+  }
+  // entry offsets of the four nodes in plane z0 (p is a multiple of 4: a pair
+  // is inside the row as a whole)
+  const int o = o0 + 2 * pair, gx = x0 + lx;
+  bool ok[S::R];
+  long long at[S::R];
+#pragma unroll
+  for (int r = 0; r < S::R; ++r) {
+    const int gy = y0 + ly + r;
+    ok[r] = o < p && gx < N && gy < N &&
+            KS_IN((((long long)(z1 - 1) * N + gy) * N + gx) * p + o + 1, NN * N * p);
+    at[r] = (((long long)z0 * N + gy) * N + gx) * p + o;
+  }
+  const long long plane = NN * p;
+  const f2_t k0 = f2_dup(a.cf[0]), ke = f2_dup(a.cf[1]), kc = f2_dup(a.cf[2]);
+  const f2_t m0 = f2_dup(a.cf[3]), mf = f2_dup(a.cf[4]), me = f2_dup(a.cf[5]), mc = f2_dup(a.cf[6]);
+  const f2_t kin = f2_dup(a.cf[7]), vscale = f2_dup(a.cf[8]);
+  f2_t acc[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) acc[i] = 0ull;
+  f2_t co[S::R], fo[S::R], eo[S::R], cm[S::R], fm[S::R], em[S::R];
+#pragma unroll
+  for (int r = 0; r < S::R; ++r) co[r] = fo[r] = eo[r] = cm[r] = fm[r] = em[r] = 0ull;
+  const int base = (ly * S::HX + lx) * S::PC + 2 * pair;      // row y - 1, column x - 1
+  const int nbase = (ly * S::TX + lx) * S::PC + 2 * pair;     // node boxes
+  auto ld = [](const float *q) { return *reinterpret_cast<const f2_t *>(q); };
+  int failed_at = -1;
+  for (int q = 0; q < nplanes; ++q) {
+    const int zp = z0 - 1 + q, st = q % kStStages;
+    if (kHam && (int)threadIdx.x < TXY) {
+      vs[q % 3][threadIdx.x] = Kind == SK_HAM ? a.cf[8] * (float)vreg : (float)vreg;
+      if (Kind == SK_HAM_INC) {
+        vbs[q % 3][threadIdx.x] = (float)vbreg;
+        dvs[q % 3][threadIdx.x] = (float)(vreg - vbreg);
+      }
+      vreg = 0.0;
+      vbreg = 0.0;
+      if (vown && zp + 1 < N) {
+        vreg = a.veff[(zp + 1) * NN + (long long)vy * N + vx];
+        if (Kind == SK_HAM_INC) vbreg = a.veff_b[(zp + 1) * NN + (long long)vy * N + vx];
+      }
+    }
+    const bool got = mbar_wait_parity(&full[st], (uint32_t)((q / kStStages) & 1));
+    const float *tile = ring + st * STAGE;
+    f2_t cn[S::R], fn[S::R], en[S::R];
+    {
+      f2_t c[S::R + 2], s[S::R + 2];
+#pragma unroll
+      for (int y = 0; y < S::R + 2; ++y) {
+        const float *row = tile + base + y * S::HX * S::PC;
+        c[y] = ld(row + S::PC);
+        s[y] = f2_add(ld(row), ld(row + 2 * S::PC));
+      }
+#pragma unroll
+      for (int r = 0; r < S::R; ++r) {
+        cn[r] = c[r + 1];
+        fn[r] = f2_add(s[r + 1], f2_add(c[r], c[r + 2]));
+        en[r] = f2_add(s[r], s[r + 2]);
+      }
+    }
+    if (q >= 2) {
+      const long long zo = (long long)(q - 2) * plane;
+#pragma unroll
+      for (int r = 0; r < S::R; ++r) {
+        const f2_t edges = f2_add(em[r], f2_add(fo[r], fn[r]));
+        const f2_t corners = f2_add(eo[r], en[r]);
+        const f2_t faces = f2_add(fm[r], f2_add(co[r], cn[r]));
+        // (the same order of products as the scalar forms, StCols::mass)
+        const f2_t mcf =
+            kHam ? f2_fma(m0, cm[r], f2_mul(mf, faces)) : f2_fma(mf, faces, f2_mul(m0, cm[r]));
+        const f2_t m = f2_fma(mc, corners, f2_fma(me, edges, mcf));
+        const int nd = (ly + r) * S::TX + lx, pl = (q + 2) % 3;
+        const float *aux = tile + S::BOX + nbase + r * S::TX * S::PC;
+        if (kHam) {
+          const f2_t kx = f2_fma(kc, corners, f2_fma(k0, cm[r], f2_mul(ke, edges)));
+          f2_t ex;
+          if (Kind == SK_HAM) {
+            ex = f2_fma(kin, kx, f2_mul(f2_dup(vs[pl][nd]), cm[r]));
+            if (ok[r]) acc[0] = f2_fma(cm[r], kx, acc[0]);
+          } else {
+            const f2_t xb = ld(aux), eb = ld(aux + S::AUX);
+            const f2_t v = f2_dup(vs[pl][nd]), vb = f2_dup(vbs[pl][nd]), dv = f2_dup(dvs[pl][nd]);
+            const f2_t kd = f2_mul(kin, kx);
+            ex = f2_fma(vscale, f2_fma(dv, xb, f2_mul(v, cm[r])), kd);
+            // compensated sum of delta . (2 f K X_b + f K delta); acc[1] holds the
+            // running rounding error
+            const f2_t fkxb = f2_sub(eb, f2_mul(f2_mul(vscale, vb), xb));
+            const f2_t t = f2_mul(cm[r], f2_fma(f2_dup(2.f), fkxb, kd));
+            if (ok[r]) {
+              const f2_t y = f2_sub(t, acc[1]);
+              const f2_t sum = f2_add(acc[0], y);
+              acc[1] = f2_sub(f2_sub(sum, acc[0]), y);
+              acc[0] = sum;
+            }
+          }
+          if (ok[r]) {
+            *reinterpret_cast<f2_t *>((float *)a.out1 + at[r] + zo) = ex;
+            if (a.out2) *reinterpret_cast<f2_t *>((float *)a.out2 + at[r] + zo) = m;
+          }
+        } else if (ok[r]) {
+          *reinterpret_cast<f2_t *>((float *)a.out1 + at[r] + zo) = m;
+          if (Kind >= SK_MASS_DOT) acc[0] = f2_fma(cm[r], m, acc[0]);
+          if (Kind == SK_MASS_BB) {
+            const f2_t dx = f2_sub(ld(aux), ld(aux + 2 * S::AUX));
+            const f2_t dmx = f2_sub(ld(aux + S::AUX), ld(aux + 3 * S::AUX));
+            const f2_t dd = f2_sub(cm[r], ld(aux + 4 * S::AUX));
+            const f2_t dmd = f2_sub(m, ld(aux + 5 * S::AUX));
+            acc[1] = f2_fma(dx, dmx, acc[1]);
+            acc[2] = f2_fma(dx, dmd, acc[2]);
+            acc[3] = f2_fma(dd, dmd, acc[3]);
+          }
+        }
+      }
+    }
+    // every thread is done with this stage: refill it kStStages planes ahead
+    if (__syncthreads_or(!got)) {
+      failed_at = q;
+      break;
+    }
+    if (threadIdx.x == 0 && q + kStStages < nplanes) load_stage(q + kStStages);
+#pragma unroll
+    for (int r = 0; r < S::R; ++r) {
+      co[r] = cm[r]; fo[r] = fm[r]; eo[r] = em[r];
+      cm[r] = cn[r]; fm[r] = fn[r]; em[r] = en[r];
+    }
+  }
+  if (failed_at >= 0) {
+    // record the timeout, give the copies still in flight a bounded wait,
+    // and still take part in the reduction so that its counter re-arms
+    if (threadIdx.x == 0) {
+      atomicCAS(a.status, 0, (int)KS_ETIMEOUT);
+      for (int q = failed_at; q < failed_at + kStStages && q < nplanes; ++q)
+        mbar_wait_parity(&full[q % kStStages], (uint32_t)((q / kStStages) & 1));
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) acc[i] = 0ull;
+  }
+  if (Kind == SK_MASS) return;
+  const double s0 = block_sum(
+      Kind == SK_HAM_INC ? f2_sum(acc[0]) - f2_sum(acc[1]) : f2_sum(acc[0]), smem);
+  if (threadIdx.x == 0) a.part[blockIdx.x] = s0;
+  if (Kind == SK_MASS_BB) {
+#pragma unroll
+    for (int i = 1; i < 4; ++i) {
+      const double s = block_sum(f2_sum(acc[i]), smem);
+      if (threadIdx.x == 0) a.part[i * a.nb + blockIdx.x] = s;
+    }
+  }
+  grid_reduce_tail(a.part, a.nb, Kind == SK_MASS_BB ? 4 : 1, a.red_out, a.red_scale, a.counter,
+                   smem);
+}
+
 // Geometry of a launch: tiles, orbital chunks and z segments; the number of
 // segments is lowered until the block partials (nchan per block) fit.
 // `halo` > 0 (one system alone on the device): the segment length with the
@@ -631,15 +892,13 @@ __global__ void __launch_bounds__(kStThreads, 2) stencil_tma_kernel(const __grid
 // one plane (12 of 8 before), 64^3 x 64 1024 of 16 planes (7 per SM).
 // `halo` = 0 (jobs that share the device): about 8 blocks per SM, segments of
 // at least 8 planes, or segments of `planes` planes when given.
-template <int PC>
-static ks_status stencil_geometry(const Problem &P, int nchan, StArgs &a, double halo,
-                                  int planes = 0) {
-  using Tl = StTile<PC>;
+static ks_status stencil_geometry_of(const Problem &P, int tx, int ty, int pc, int nchan,
+                                     StArgs &a, double halo, int planes) {
   a.N = P.N;
   a.p = P.p;
-  a.tiles_x = (P.N + Tl::TX - 1) / Tl::TX;
-  a.tiles_y = (P.N + Tl::TY - 1) / Tl::TY;
-  a.chunks = (P.p + PC - 1) / PC;
+  a.tiles_x = (P.N + tx - 1) / tx;
+  a.tiles_y = (P.N + ty - 1) / ty;
+  a.chunks = (P.p + pc - 1) / pc;
   const long long base = (long long)a.tiles_x * a.tiles_y * a.chunks;
   long long segs = (8LL * P.sms + base - 1) / base;
   const long long maxsegs = (P.N + 7) / 8;
@@ -671,30 +930,71 @@ static ks_status stencil_geometry(const Problem &P, int nchan, StArgs &a, double
   }
 }
 
-// TMA form of one launch; false (and nothing launched) when the input
-// cannot be described by a tensor map (row pitch or base address not a
-// multiple of 16 bytes).
-template <typename T, int PC, int Kind>
-static bool stencil_launch_tma(Problem &P, const StArgs &a, int cls, double flops, double bytes,
-                               ks_status *st) {
+template <int PC>
+static ks_status stencil_geometry(const Problem &P, int nchan, StArgs &a, double halo,
+                                  int planes = 0) {
   using Tl = StTile<PC>;
-  using Rg = StRing<T, PC, Kind>;
-  *st = KS_OK;
+  return stencil_geometry_of(P, Tl::TX, Tl::TY, PC, nchan, a, halo, planes);
+}
+
+// Whether a launch's operands can be described by tensor maps (row pitch and
+// bases multiples of 16 bytes).
+template <typename T, int Kind>
+static bool stencil_tma_ok(const Problem &P, const StArgs &a) {
   const void *aux[6] = {a.X, a.MX, a.Xp, a.MXp, a.Dp, a.MDp};
   if (!P.use_tma || ((size_t)P.p * sizeof(T)) % 16 != 0 ||
       reinterpret_cast<uintptr_t>(a.A) % 16 != 0)
     return false;
-  for (int i = 0; i < Rg::NAUX; ++i)
+  for (int i = 0; i < st_naux<T, Kind>(); ++i)
     if (!aux[i] || reinterpret_cast<uintptr_t>(aux[i]) % 16 != 0) return false;
+  return sizeof(T) == 8 || (reinterpret_cast<uintptr_t>(a.out1) % 8 == 0 &&
+                            reinterpret_cast<uintptr_t>(a.out2) % 8 == 0);
+}
+
+// TMA form of one launch; false (and nothing launched) when the input
+// cannot be described by a tensor map (row pitch or base address not a
+// multiple of 16 bytes).
+// (The packed FP32 kernel also stores pairs: 8-byte aligned outputs.)
+template <typename T, int PC, int Kind>
+static bool stencil_launch_tma(Problem &P, const StArgs &a, int cls, double flops, double bytes,
+                               ks_status *st) {
+  constexpr bool kF2 = sizeof(T) == 4 && PC == 32;
+  constexpr int TX = kF2 ? StF2::TX : StTile<PC>::TX, TY = kF2 ? StF2::TY : StTile<PC>::TY;
+  constexpr int NAUX = st_naux<T, Kind>();
+  *st = KS_OK;
+  const void *aux[6] = {a.X, a.MX, a.Xp, a.MXp, a.Dp, a.MDp};
+  if (!stencil_tma_ok<T, Kind>(P, a)) return false;
   StTmaArgs ta;
   ta.a = a;
   const uint64_t dims[4] = {(uint64_t)P.p, (uint64_t)P.N, (uint64_t)P.N, (uint64_t)P.N};
-  const uint32_t box[4] = {(uint32_t)PC, (uint32_t)Tl::HX, (uint32_t)Tl::HY, 1u};
-  const uint32_t nbox[4] = {(uint32_t)PC, (uint32_t)Tl::TX, (uint32_t)Tl::TY, 1u};
+  const uint32_t box[4] = {(uint32_t)PC, (uint32_t)TX + 2, (uint32_t)TY + 2, 1u};
+  const uint32_t nbox[4] = {(uint32_t)PC, (uint32_t)TX, (uint32_t)TY, 1u};
   if (encode_tensor_map_4d(&ta.map, a.A, (int)sizeof(T), dims, box) != KS_OK) return false;
-  for (int i = 0; i < Rg::NAUX; ++i)
+  for (int i = 0; i < NAUX; ++i)
     if (encode_tensor_map_4d(&ta.aux[i], aux[i], (int)sizeof(T), dims, nbox) != KS_OK)
       return false;
+  if constexpr (kF2) {
+    static std::once_flag once;
+    static cudaError_t attr = cudaSuccess;
+    static_assert(st_f2_smem<Kind>() <= 224 * 1024, "the ring fits an SM");
+    std::call_once(once, [] {
+      attr = cudaFuncSetAttribute(stencil_f32x2_kernel<Kind>,
+                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)st_f2_smem<Kind>());
+    });
+    if (attr != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    {
+      ProfScope ps_(P.stream, cls, flops, bytes);
+      stencil_f32x2_kernel<Kind><<<a.nb, kStThreads, st_f2_smem<Kind>(), P.stream>>>(ta);
+    }
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) *st = cuda_error(e, "stencil_f32x2_kernel");
+    return true;
+  } else {
+  using Rg = StRing<T, PC, Kind>;
   // the ring plus the static shared memory (mbarriers, V_eff planes,
   // reduction scratch: up to ~10 KiB) for two blocks per SM; the kernel
   // opts in to the ring's size once
@@ -718,6 +1018,7 @@ static bool stencil_launch_tma(Problem &P, const StArgs &a, int cls, double flop
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) *st = cuda_error(e, "stencil_tma_kernel");
   return true;
+  }
 }
 
 template <typename T, int PC, int Kind>
@@ -725,7 +1026,10 @@ static ks_status stencil_launch_pc(Problem &P, StArgs &a, int nchan, double flop
   // FP64: a halo plane costs its in-plane sums, over half of a plane's
   // instructions, two of them 1.2 planes.  FP32 reads it from L2 and is
   // bound by memory, where more and shorter segments overlap better
-  KS_TRY(stencil_geometry<PC>(P, nchan, a, sizeof(T) == 8 ? 1.2 : 0.0));
+  constexpr bool kF2 = sizeof(T) == 4 && PC == 32;
+  const bool f2 = kF2 && stencil_tma_ok<T, Kind>(P, a);
+  if (f2) KS_TRY(stencil_geometry_of(P, StF2::TX, StF2::TY, StF2::PC, nchan, a, 0.0, 0));
+  else KS_TRY(stencil_geometry<PC>(P, nchan, a, sizeof(T) == 8 ? 1.2 : 0.0));
   a.c = q1_coefficients(P.h);
   a.k0r = a.c.k0 / a.c.ke;
   if (P.mass == KS_MASS_LUMPED) {      // row sums of M: h^3 on the centre
@@ -742,8 +1046,11 @@ static ks_status stencil_launch_pc(Problem &P, StArgs &a, int nchan, double flop
   ks_status st;
   // one amplitude (PC = 1, p = 1) has an 8-byte row pitch, which no tensor
   // map can describe: plain staging only
-  if constexpr (PC >= 4)
+  if constexpr (PC >= 4) {
     if (stencil_launch_tma<T, PC, Kind>(P, a, cls, flops, bytes, &st)) return st;
+    // plain staging has its own tiles
+    if (f2) KS_TRY(stencil_geometry<PC>(P, nchan, a, 0.0));
+  }
   {
     ProfScope ps_(P.stream, cls, flops, bytes);
     stencil_kernel<T, PC, Kind><<<a.nb, kStThreads, 0, P.stream>>>(a);
