@@ -320,47 +320,56 @@ __global__ void __launch_bounds__(256) gram_small_kernel(long long n, int pa, in
 }
 
 // Pipelined FP32 Grams for 32 < max(pa, qb) <= 64 and 16-byte-aligned
-// operands (widths multiples of 4): persistent blocks take stages of 32 rows
-// in turn (block b: stages b, b + G, ...), copied global -> shared by
-// cp.async three stages ahead (columns beyond pa, qb zero-filled), and keep
-// 64 x 64 FP32 tiles (4 x 4 per thread) over all their rows; each block
-// writes its FP32 partial tiles, summed afterwards in FP64 in block order.
-// Two forms:
+// operands (widths multiples of 4).  Two forms:
 //   pair   (Dual = false): out = A1^T B1 + A2^T B2 -- the rows of the second
 //          pair follow those of the first (A2 null: one Gram);
-//   shared (Dual = true):  out1 = A1^T B, out2 = A2^T B with B read once.
-constexpr int kGaStages = 3, kGaRows = 32;
+//   shared (Dual = true):  out1 = A1^T B, out2 = A2^T B (even warps take A1,
+//          odd warps A2, on the same rows, so B comes from DRAM once).
+// FP32 FMAs bound it, and next to them shared memory (128 bytes per clock):
+// a 4 x 4 block of outputs per thread reads two bytes per FMA, the 8 x 16
+// block per lane here three quarters of one.  A warp keeps the whole 64 x 64
+// tile and runs alone on stages of kGaRows rows (a ring of kGaStages, cp.async
+// 16 bytes per copy, zero-filled past the last row and past pa, qb); lane
+// (ty, tx) of 8 x 4 owns columns 4 ty + 32 h of A and 4 tx + 16 j of B.  The
+// warps' tiles (chains of about 200 rows at 64^3) are added in pairs in FP32 (in
+// FP64 those 4096 x 8 adds per block took 17 us), the blocks' sums in FP64 in
+// block order.  One Gram at 64^3 x 64: 63 us for 4 x 4 per thread (34 TF/s), 56
+// here (38); packed FMAs cost more in duplicating A than they save (65).
+constexpr int kGaStages = 3, kGaRows = 16, kGaWarps = 8;
 
-template <bool Dual>
-constexpr size_t gram_ta_smem() {
-  return (size_t)kGaStages * (Dual ? 3 : 2) * kGaRows * kTile * sizeof(float);
+constexpr size_t gram_wa_smem() {
+  // the rings; the same memory then holds the warps' tiles
+  constexpr size_t ring = (size_t)kGaWarps * kGaStages * 2 * kGaRows * kTile * sizeof(float);
+  static_assert(ring >= (size_t)kGaWarps * kTile * kTile * sizeof(float), "the tiles fit");
+  return ring;
 }
 
 template <bool Dual>
-__global__ void __launch_bounds__(256, Dual ? 3 : 4) gram2_ta_kernel(
+__global__ void __launch_bounds__(32 * kGaWarps, 1) gram2_wa_kernel(
     long long n, int pa, int qb, const float *__restrict__ A1, const float *__restrict__ B1,
     const float *__restrict__ A2, const float *__restrict__ B2, float *__restrict__ part) {
   extern __shared__ __align__(16) float ga_smem[];
-  constexpr int kOps = Dual ? 3 : 2;                 // staged operands: A1, B (, A2)
-  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+  constexpr int kStage = 2 * kGaRows * kTile;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, ty = lane >> 2, tx = lane & 3;
+  float *ring = ga_smem + (size_t)warp * kGaStages * kStage;
   const long long nv = (!Dual && A2) ? 2 * n : n;    // rows streamed (both pairs)
   const long long nst = (nv + kGaRows - 1) / kGaRows;
-  const long long W = nst > blockIdx.x ? (nst - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
+  // stages of this warp (of this warp's pair in the shared form)
+  const long long first = (long long)(Dual ? warp >> 1 : warp) * gridDim.x + blockIdx.x;
+  const long long step = (long long)(Dual ? kGaWarps / 2 : kGaWarps) * gridDim.x;
+  const long long W = nst > first ? (nst - first + step - 1) / step : 0;
+  const float *Aw = Dual && (warp & 1) ? A2 : A1;
   auto issue = [&](long long w) {
-    const long long r0 = (blockIdx.x + w * gridDim.x) * kGaRows;
-    float *dst = ga_smem + (size_t)(w % kGaStages) * kOps * kGaRows * kTile;
+    const long long r0 = (first + w * step) * kGaRows;
+    float *dst = ring + (w % kGaStages) * kStage;
 #pragma unroll
-    for (int t = 0; t < kOps * 2; ++t) {
-      const int idx = tid + t * 256;               // operand, row, 4-column chunk
-      const int op = idx >> 9, rr = (idx >> 4) & 31, c4 = (idx & 15) * 4;
+    for (int t = 0; t < kStage / 128; ++t) {           // operand, row, 4-column chunk
+      const int idx = lane + 32 * t, op = idx / (kGaRows * 16);
+      const int rr = idx / 16 % kGaRows, c4 = idx % 16 * 4;
       long long row = r0 + rr;
       const int w_ = op == 1 ? qb : pa;
-      const float *M;
-      if (Dual) {
-        M = op == 0 ? A1 : op == 1 ? B1 : A2;
-      } else if (row < n) {
-        M = op == 0 ? A1 : B1;
-      } else {
+      const float *M = op == 0 ? Aw : B1;
+      if (!Dual && row >= n) {
         M = op == 0 ? A2 : B2;
         row -= n;
       }
@@ -370,73 +379,78 @@ __global__ void __launch_bounds__(256, Dual ? 3 : 4) gram2_ta_kernel(
         src = M + row * w_ + c4;
         bytes = 16;
       }
-      const int di = op * kGaRows * kTile + rr * kTile + c4;
-      if (KS_IN(di + 3, kOps * kGaRows * kTile)) cp_async16(smem_addr(dst + di), src, bytes);
+      cp_async16(smem_addr(dst + op * kGaRows * kTile + rr * kTile + c4), src, bytes);
     }
   };
-  float acc[4][4], acc2[4][4];
+  float acc[8][16];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < 8; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = acc2[i][j] = 0.f;
+    for (int j = 0; j < 16; ++j) acc[i][j] = 0.f;
   for (int st = 0; st < kGaStages - 1; ++st) {
     if (st < W) issue(st);
     cp_async_commit();
   }
   for (long long w = 0; w < W; ++w) {
     asm volatile("cp.async.wait_group %0;\n" ::"n"(kGaStages - 2) : "memory");
-    __syncthreads();
+    __syncwarp();
     if (w + kGaStages - 1 < W) issue(w + kGaStages - 1);
     cp_async_commit();
-    const float *As = ga_smem + (size_t)(w % kGaStages) * kOps * kGaRows * kTile;
-    const float *Bs = As + kGaRows * kTile;
-    const float *A2s = Bs + kGaRows * kTile;
-#pragma unroll 8
+    const float *As = ring + (w % kGaStages) * kStage + 4 * ty;
+    const float *Bs = ring + (w % kGaStages) * kStage + kGaRows * kTile + 4 * tx;
+#pragma unroll 2
     for (int r = 0; r < kGaRows; ++r) {
-      const float4 av = *reinterpret_cast<const float4 *>(As + r * kTile + 4 * ty);
-      const float4 bv = *reinterpret_cast<const float4 *>(Bs + r * kTile + 4 * tx);
-      const float a4[4] = {av.x, av.y, av.z, av.w};
-      const float b4[4] = {bv.x, bv.y, bv.z, bv.w};
+      float av[8], bv[16];
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a4[i], b4[j], acc[i][j]);
-      if (Dual) {
-        const float4 cv = *reinterpret_cast<const float4 *>(A2s + r * kTile + 4 * ty);
-        const float c4[4] = {cv.x, cv.y, cv.z, cv.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) acc2[i][j] = fmaf(c4[i], b4[j], acc2[i][j]);
+      for (int h = 0; h < 2; ++h) {
+        const float4 v = *reinterpret_cast<const float4 *>(As + r * kTile + 32 * h);
+        av[4 * h] = v.x; av[4 * h + 1] = v.y; av[4 * h + 2] = v.z; av[4 * h + 3] = v.w;
       }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float4 v = *reinterpret_cast<const float4 *>(Bs + r * kTile + 16 * j);
+        bv[4 * j] = v.x; bv[4 * j + 1] = v.y; bv[4 * j + 2] = v.z; bv[4 * j + 3] = v.w;
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 16; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
     }
   }
   asm volatile("cp.async.wait_all;\n" ::: "memory");
-  const long long len = (long long)pa * qb;
+  __syncthreads();
+  float *tile = ga_smem + (size_t)warp * kTile * kTile;
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      *reinterpret_cast<float4 *>(tile + (32 * (i >> 2) + 4 * ty + (i & 3)) * kTile + 16 * j +
+                                  4 * tx) =
+          make_float4(acc[i][4 * j], acc[i][4 * j + 1], acc[i][4 * j + 2], acc[i][4 * j + 3]);
+  __syncthreads();
+  const int len = pa * qb;
   float *dst = part + (long long)blockIdx.x * (Dual ? 2 : 1) * len;
+  for (int e = threadIdx.x; e < (Dual ? 2 : 1) * len; e += 32 * kGaWarps) {
+    const int which = e >= len ? 1 : 0, f = e - which * len, at = f / qb * kTile + f % qb;
+    constexpr int kTiles = Dual ? kGaWarps / 2 : kGaWarps;
+    float v[kTiles];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int a = 4 * ty + i;
-    if (a >= pa) continue;
+    for (int s = 0; s < kTiles; ++s)
+      v[s] = ga_smem[(size_t)(s * (Dual ? 2 : 1) + which) * kTile * kTile + at];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int b = 4 * tx + j;
-      if (b >= qb) continue;
-      if (!KS_IN((long long)blockIdx.x * (Dual ? 2 : 1) * len + (Dual ? len : 0) + a * qb + b,
-                 (long long)gridDim.x * (Dual ? 2 : 1) * len))
-        continue;
-      dst[(long long)a * qb + b] = acc[i][j];
-      if (Dual) dst[len + (long long)a * qb + b] = acc2[i][j];
-    }
+    for (int o = kTiles / 2; o > 0; o >>= 1)
+#pragma unroll
+      for (int s = 0; s < o; ++s) v[s] += v[s + o];
+    dst[e] = v[0];
   }
 }
 
-// FP64 sums of FP32 chunk partials in chunk order: element e < len1 of each
-// chunk goes to out1[e], the rest to out2[e - len1]; out32 (optional) gets
-// every sum rounded to FP32 at index e.
-__global__ void gram_reduce_f32_kernel(int chunks, long long len, long long len1,
-                                       const float *__restrict__ part, double *__restrict__ out1,
-                                       double *__restrict__ out2, float *__restrict__ out32) {
+// FP64 sums of the blocks' partials in block order: element e < len1 of each
+// goes to out1[e], the rest to out2[e - len1]; out32 (optional) gets every sum
+// rounded to FP32 at index e.
+__global__ void gram_reduce2_kernel(int chunks, long long len, long long len1,
+                                    const float *__restrict__ part, double *__restrict__ out1,
+                                    double *__restrict__ out2, float *__restrict__ out32) {
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long e = t >> 3;
   const int sub = (int)(t & 7);
@@ -455,7 +469,7 @@ __global__ void gram_reduce_f32_kernel(int chunks, long long len, long long len1
 
 // The pipelined Gram kernels apply: FP32, 32 < max(pa, qb) <= 64, widths
 // multiples of 4 and 16-byte-aligned operands.
-static bool gram_ta_applies(int pa, int qb, std::initializer_list<const float *> ops) {
+static bool gram_wa_applies(int pa, int qb, std::initializer_list<const float *> ops) {
   if (pa > kTile || qb > kTile || (pa <= kMidPQ && qb <= kMidPQ) || pa % 4 || qb % 4) return false;
   for (const float *A : ops)
     if (reinterpret_cast<uintptr_t>(A) % 16) return false;
@@ -463,12 +477,12 @@ static bool gram_ta_applies(int pa, int qb, std::initializer_list<const float *>
 }
 
 template <bool Dual>
-static ks_status launch_gram2_ta(Problem &P, int pa, int qb, const float *A1, const float *B1,
+static ks_status launch_gram2_wa(Problem &P, int pa, int qb, const float *A1, const float *B1,
                                  const float *A2, const float *B2, double *out1, double *out2,
                                  float *out32 = nullptr) {
   const long long nv = (!Dual && A2) ? 2 * P.n : P.n;
   const long long nst = (nv + kGaRows - 1) / kGaRows;
-  long long blocks = (Dual ? 3LL : 4LL) * P.sms;
+  long long blocks = P.sms;
   if (blocks > nst) blocks = nst;
   const long long len = (long long)pa * qb * (Dual ? 2 : 1);
   // FP32 partials in the FP64 partial buffer
@@ -478,13 +492,13 @@ static ks_status launch_gram2_ta(Problem &P, int pa, int qb, const float *A1, co
   {
     ProfScope ps_(P.stream, KP_GRAM, 2.0 * nv * pa * qb * (Dual ? 2 : 1),
                   (double)nv * (pa + qb + (Dual ? pa : 0)) * sizeof(float));
-    gram2_ta_kernel<Dual><<<(int)blocks, 256, gram_ta_smem<Dual>(), P.stream>>>(
+    gram2_wa_kernel<Dual><<<(int)blocks, 32 * kGaWarps, gram_wa_smem(), P.stream>>>(
         P.n, pa, qb, A1, B1, A2, B2, part);
   }
   KS_CUDA_TRY(cudaGetLastError());
   {
     ProfScope ps_(P.stream, KP_REDUCE);
-    gram_reduce_f32_kernel<<<(int)((8 * len + kThreads - 1) / kThreads), kThreads, 0, P.stream>>>(
+    gram_reduce2_kernel<<<(int)((8 * len + kThreads - 1) / kThreads), kThreads, 0, P.stream>>>(
         (int)blocks, len, (long long)pa * qb, part, out1, out2, out32);
   }
   KS_CUDA_TRY(cudaGetLastError());
@@ -525,8 +539,8 @@ ks_status launch_gram(Problem &P, const T *A, int pa, const T *B, int qb, double
     KS_CUDA_TRY(cudaGetLastError());
     return KS_OK;
   }
-  if (sizeof(T) == 4 && gram_ta_applies(pa, qb, {(const float *)A, (const float *)B}))
-    return launch_gram2_ta<false>(P, pa, qb, (const float *)A, (const float *)B, nullptr, nullptr,
+  if (sizeof(T) == 4 && gram_wa_applies(pa, qb, {(const float *)A, (const float *)B}))
+    return launch_gram2_wa<false>(P, pa, qb, (const float *)A, (const float *)B, nullptr, nullptr,
                                   out, nullptr);
   const int chunks = gram_chunks(P, pa, qb);
   long long rows_per = (P.n + chunks - 1) / chunks;
@@ -558,8 +572,8 @@ ks_status launch_gram(Problem &P, const T *A, int pa, const T *B, int qb, double
 
 ks_status launch_gram_pair(Problem &P, const float *A1, const float *B1, const float *A2,
                            const float *B2, int pa, int qb, double *out, double *tmp) {
-  if (gram_ta_applies(pa, qb, {A1, B1, A2, B2}))
-    return launch_gram2_ta<false>(P, pa, qb, A1, B1, A2, B2, out, nullptr, nullptr);
+  if (gram_wa_applies(pa, qb, {A1, B1, A2, B2}))
+    return launch_gram2_wa<false>(P, pa, qb, A1, B1, A2, B2, out, nullptr, nullptr);
   KS_TRY(launch_gram<float>(P, A1, pa, B1, qb, out));
   KS_TRY(launch_gram<float>(P, A2, pa, B2, qb, tmp));
   return launch_add_pp(P, out, 1.0, tmp, out);
@@ -575,8 +589,8 @@ __global__ void pair_to_f32_kernel(long long len, const double *__restrict__ a,
 
 ks_status launch_gram_dual(Problem &P, const float *A1, const float *A2, const float *B, int pa,
                            int qb, double *out1, double *out2, float *out32) {
-  if (gram_ta_applies(pa, qb, {A1, A2, B}))
-    return launch_gram2_ta<true>(P, pa, qb, A1, B, A2, nullptr, out1, out2, out32);
+  if (gram_wa_applies(pa, qb, {A1, A2, B}))
+    return launch_gram2_wa<true>(P, pa, qb, A1, B, A2, nullptr, out1, out2, out32);
   KS_TRY(launch_gram<float>(P, A1, pa, B, qb, out1));
   KS_TRY(launch_gram<float>(P, A2, pa, B, qb, out2));
   if (out32) {
@@ -1242,36 +1256,98 @@ template ks_status batch_convert<float, float>(Batch &, int, int);
 template ks_status launch_gram<double>(Problem &, const double *, int, const double *, int,
                                        double *);
 template ks_status launch_gram<float>(Problem &, const float *, int, const float *, int, double *);
-// Pipelined form of combine_ts_kernel for 16-byte-aligned operands (every k
-// a multiple of 4 and every A base 16-byte aligned): the A stages are copied
-// global -> shared by cp.async (16 bytes per copy, zero-filled past the last
-// row and past K) three stages ahead, row-major with a 4-float pad, so no
-// registers hold staged data and three stages of loads are in flight per
-// block.  A thread reads, per 4 K-values, one float4 of each of its 8 rows
-// and one float4 of C per K-value: 128 FMAs per 12 vector loads.  The FMA
-// chains and the final step are those of combine_ts_kernel (K ascending).
-constexpr int kTaStages = 3, kTaLd = kTsK + 4;
+// Warp form of the tall-skinny update (combine_wa_kernel below).
+constexpr int kWaStages = 3, kWaR = 8, kWaRows = 4 * kWaR, kWaK = 32, kWaLd = kWaK + 4;
+constexpr int kWaWarps = 12;
 
-size_t combine_ta_smem(int K) {
-  const int nst = (K + kTsK - 1) / kTsK;
-  return ((size_t)nst * kTsK * kTile + (size_t)kTaStages * kTsRows * kTaLd) * sizeof(float);
+// Half h of the epilogue for one lane: rows row0 + 4 i, columns 32 h + 4 tx ..
+// + 3 of out = alpha acc + beta Bm and out2 = add2 + out; `staged` holds this
+// half of Bm or add2 in shared memory (row stride kWaLd).  dsum[i] gathers
+// the row's density increment (ts_epilogue).
+__device__ __forceinline__ void wa_half(long long n, int q, long long row0, int tx, int h,
+                                        f2_t (&acc)[kWaR][4], float alpha, float beta,
+                                        const float *staged, bool with_b, float *__restrict__ out,
+                                        float *__restrict__ out2, bool vec, bool dens,
+                                        float (&dsum)[kWaR]) {
+  const int col0 = 32 * h + 4 * tx;
+#pragma unroll
+  for (int i = 0; i < kWaR; ++i) {
+    const long long row = row0 + 4 * i, o = row * q + col0;
+    const float4 s4 = staged ? *reinterpret_cast<const float4 *>(staged + 4 * i * kWaLd)
+                             : make_float4(0.f, 0.f, 0.f, 0.f);
+    const float s[4] = {s4.x, s4.y, s4.z, s4.w};
+    float v[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      float lo, hi;
+      f2_split(acc[i][2 * h + (j >> 1)], lo, hi);
+      v[j] = alpha * ((j & 1) ? hi : lo);
+      if (with_b) v[j] = fmaf(beta, s[j], v[j]);
+    }
+    if (row < n && vec && col0 + 3 < q && KS_IN(o + 3, n * q)) {
+      *reinterpret_cast<float4 *>(out + o) = make_float4(v[0], v[1], v[2], v[3]);
+      if (out2)
+        *reinterpret_cast<float4 *>(out2 + o) =
+            make_float4(s[0] + v[0], s[1] + v[1], s[2] + v[2], s[3] + v[3]);
+    } else if (row < n) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (col0 + j < q && KS_IN(o + j, n * q)) {
+          out[o + j] = v[j];
+          if (out2) out2[o + j] = s[j] + v[j];
+        }
+    }
+    if (dens)
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (col0 + j < q) dsum[i] = fmaf(v[j], fmaf(2.f, s[j], v[j]), dsum[i]);
+  }
 }
 
+// Pipelined form of combine_ts_kernel for 16-byte-aligned operands (every k
+// a multiple of 4 and every A base 16-byte aligned).  FP32 FMAs bound it
+// (6.4 GFLOP against 336 MB for the retraction at 64^3 x 64), and next to them
+// shared memory, which delivers 128 bytes per clock against 128 FMAs: an
+// 8 x 4 block of outputs per thread reads 1.5 bytes per FMA, the 8 x 8 block
+// per lane here one.  Each warp runs alone on tiles of 32 rows, with its own
+// ring of kWaStages stages (32 rows x kWaK K-values, cp.async 16 bytes per copy,
+// zero-filled past the last row and past K) and no block barrier, so one warp's
+// epilogue overlaps the others' products.  The epilogue's operand (Bm or
+// add2) follows the K stages through the ring as two more stages: read from
+// global memory in the epilogue, its 16 loads per lane waited one by one.  A
+// lane owns rows ty + 4 i (i < 8) and columns 4 tx .. + 3 and 32 + 4 tx .. + 3
+// (ty = lane / 8, tx = lane % 8).  The coefficient image (K x 64, zero padded)
+// is shared by the block's warps, and the FMAs are packed pairs of columns
+// (f2_fma: the scalar outer product stops at 49 of 76 TF/s).  Update with Bm at
+// 64^3, K = 128: 134 us for the block-synchronous 8 x 4 form (32 TF/s), 107 us
+// here (40 TF/s); 16 x 8 per lane (8 warps) took 168 us.
+// The FMA chains and the final step are those of combine_ts_kernel (K
+// ascending).
 
-__global__ void __launch_bounds__(256, 2) combine_ta_kernel(
+size_t combine_wa_smem(int K) {
+  const int nst = (K + kWaK - 1) / kWaK;
+  return ((size_t)nst * kWaK * kTile + (size_t)kWaWarps * kWaStages * kWaRows * kWaLd) *
+         sizeof(float);
+}
+
+__global__ void __launch_bounds__(32 * kWaWarps, 1) combine_wa_kernel(
     long long n, int q, const float *__restrict__ A1, int k1, const float *__restrict__ c1,
     const float *__restrict__ A2, int k2, const float *__restrict__ c2,
     const float *__restrict__ A3, int k3, const float *__restrict__ c3, float alpha, float beta,
     const float *__restrict__ Bm, float *__restrict__ out, const float *__restrict__ add2,
     float *__restrict__ out2, long long ntiles, TsDensity dn) {
-  extern __shared__ __align__(16) float ta_smem[];
+  extern __shared__ __align__(16) float wa_smem[];
   const int k12 = k1 + (A2 ? k2 : 0);
   const int K = k12 + (A3 ? k3 : 0);
-  const int nst = (K + kTsK - 1) / kTsK;
-  float *Cs = ta_smem;                                  // [nst * kTsK][64]
-  float *As = ta_smem + (size_t)nst * kTsK * kTile;     // [kTaStages][kTsRows][kTaLd]
-  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-  for (int e = tid; e < nst * kTsK * kTile; e += 256) {
+  const int nst = (K + kWaK - 1) / kWaK;
+  // the epilogue's operand: at most one of Bm (added) and add2 (to out2)
+  const float *Es = Bm ? Bm : add2;
+  const int ntot = nst + (Es ? 2 : 0);
+  float *Cs = wa_smem;                                  // [nst * kWaK][64]
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, ty = lane >> 3, tx = lane & 7;
+  constexpr int kRing = kWaStages * kWaRows * kWaLd;
+  float *As = wa_smem + (size_t)nst * kWaK * kTile + (size_t)warp * kRing;
+  for (int e = threadIdx.x; e < nst * kWaK * kTile; e += 32 * kWaWarps) {
     const int r = e / kTile, c = e % kTile;
     float v = 0.f;
     if (c < q) {
@@ -1281,22 +1357,47 @@ __global__ void __launch_bounds__(256, 2) combine_ta_kernel(
     }
     Cs[e] = v;
   }
-  const long long mine = ntiles > blockIdx.x ? (ntiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
-  const long long W = mine * nst;
-  // stage w: 128 rows x 32 K-values = 1024 16-byte copies, 4 per thread
-  auto issue = [&](long long w) {
-    const long long tile = blockIdx.x + (w / nst) * gridDim.x;
-    const int k0 = (int)(w % nst) * kTsK;
-    float *dst = As + (size_t)(w % kTaStages) * kTsRows * kTaLd;
+  // this warp's tiles: (warp + kWaWarps j) gridDim + block, so that the tiles
+  // spread evenly over the blocks
+  const long long first = (long long)warp * gridDim.x + blockIdx.x;
+  const long long step = (long long)kWaWarps * gridDim.x;
+  const long long mine = ntiles > first ? (ntiles - first + step - 1) / step : 0;
+  const long long W = mine * ntot;
+  int istage = 0;                                       // K stage and tile of the next issue
+  long long itile = first;
+  int ibuf = 0;
+  // widths that are multiples of kWaK (p = 64): a stage lies in one operand
+  const bool whole = k1 % kWaK == 0 && k12 % kWaK == 0 && K % kWaK == 0 && q % kWaK == 0;
+  auto issue = [&]() {
+    const int k0 = istage * kWaK;
+    float *dst = As + ibuf * (kWaRows * kWaLd);
+    if (whole) {
+      const float *M = Es;
+      int ld = q, kc = k0 - K;
+      if (k0 < k1) { M = A1; ld = k1; kc = k0; }
+      else if (k0 < k12) { M = A2; ld = k2; kc = k0 - k1; }
+      else if (k0 < K) { M = A3; ld = k3; kc = k0 - k12; }
+      const long long row0 = itile * kWaRows + (lane >> 3);
+      const float *src = M + row0 * ld + kc + (lane & 7) * 4;
+      const uint32_t d0 = smem_addr(dst + (lane >> 3) * kWaLd + (lane & 7) * 4);
 #pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      const int idx = tid + t * 256;
-      const int rr = idx >> 3, kq = (idx & 7) * 4;
-      const long long row = tile * kTsRows + rr;
+      for (int t = 0; t < kWaRows / 4; ++t) {
+        const bool in = row0 + 4 * t < n &&
+                        KS_IN((row0 + 4 * t) * ld + kc + (lane & 7) * 4 + 3, n * ld);
+        cp_async16(d0 + t * 4 * kWaLd * 4, in ? src + (long long)4 * t * ld : M, in ? 16u : 0u);
+      }
+    } else
+#pragma unroll
+    for (int t = 0; t < kWaRows * kWaK / 128; ++t) {
+      const int rr = (lane >> 3) + 4 * t, kq = (lane & 7) * 4;
+      const long long row = itile * kWaRows + rr;
       const int k = k0 + kq;
       const float *src = A1;
       uint32_t bytes = 0;
-      if (row < n) {
+      if (istage >= nst) {
+        const int c = (istage - nst) * kWaK + kq;
+        if (row < n && c < q && KS_IN(row * q + c + 3, n * q)) { src = Es + row * q + c; bytes = 16; }
+      } else if (row < n) {
         if (k < k1) {
           if (KS_IN(row * k1 + k + 3, n * k1)) { src = A1 + row * k1 + k; bytes = 16; }
         } else if (k < k12) {
@@ -1305,49 +1406,87 @@ __global__ void __launch_bounds__(256, 2) combine_ta_kernel(
           if (KS_IN(row * k3 + (k - k12) + 3, n * k3)) { src = A3 + row * k3 + (k - k12); bytes = 16; }
         }
       }
-      const long long di = (long long)(w % kTaStages) * kTsRows * kTaLd + rr * kTaLd + kq;
-      if (KS_IN(di + 3, (long long)kTaStages * kTsRows * kTaLd))
-        cp_async16(smem_addr(dst + rr * kTaLd + kq), src, bytes);
+      cp_async16(smem_addr(dst + rr * kWaLd + kq), src, bytes);
     }
+    if (++istage == ntot) {
+      istage = 0;
+      itile += step;
+    }
+    if (++ibuf == kWaStages) ibuf = 0;
   };
-  float acc[8][4];
+  f2_t acc[kWaR][4];
+  float dsum[kWaR];
 #pragma unroll
-  for (int i = 0; i < 8; ++i)
+  for (int i = 0; i < kWaR; ++i) dsum[i] = 0.f;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-  for (int st = 0; st < kTaStages - 1; ++st) {
-    if (st < W) issue(st);
+  for (int i = 0; i < kWaR; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
+  for (int st = 0; st < kWaStages - 1; ++st) {
+    if (st < W) issue();
     cp_async_commit();
   }
   __syncthreads();                                      // C staged
+  int stage = 0, buf = 0;
+  long long tile = first;
   for (long long w = 0; w < W; ++w) {
-    asm volatile("cp.async.wait_group %0;\n" ::"n"(kTaStages - 2) : "memory");  // stage w landed
-    __syncthreads();                                    // ... everyone's; stage w-1 consumed
-    if (w + kTaStages - 1 < W) issue(w + kTaStages - 1);
+    asm volatile("cp.async.wait_group %0;\n" ::"n"(kWaStages - 2) : "memory");  // stage w landed
+    __syncwarp();                                       // ... every lane's; stage w - 1 consumed
+    if (w + kWaStages - 1 < W) issue();
     cp_async_commit();
-    const int k0 = (int)(w % nst) * kTsK;
-    const float *Ab = As + (size_t)(w % kTaStages) * kTsRows * kTaLd + (size_t)8 * ty * kTaLd;
-#pragma unroll 2
-    for (int kq = 0; kq < kTsK; kq += 4) {
-      float4 a[8];
+    const float *Ab = As + buf * (kWaRows * kWaLd) + ty * kWaLd;
+    if (stage < nst) {
+      const float *Cb = Cs + (size_t)stage * kWaK * kTile + 4 * tx;
+#pragma unroll 1
+      for (int kq = 0; kq < kWaK; kq += 4) {
+        float4 a[kWaR];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) a[i] = *reinterpret_cast<const float4 *>(Ab + i * kTaLd + kq);
+        for (int i = 0; i < kWaR; ++i)
+          a[i] = *reinterpret_cast<const float4 *>(Ab + 4 * i * kWaLd + kq);
 #pragma unroll
-      for (int kk = 0; kk < 4; ++kk) {
-        const float4 cv = *reinterpret_cast<const float4 *>(Cs + (size_t)(k0 + kq + kk) * kTile +
-                                                            4 * tx);
-        const float cc[4] = {cv.x, cv.y, cv.z, cv.w};
+        for (int kk = 0; kk < 4; ++kk) {
+          const ulonglong2 lo = *reinterpret_cast<const ulonglong2 *>(Cb + (kq + kk) * kTile);
+          const ulonglong2 hi = *reinterpret_cast<const ulonglong2 *>(Cb + (kq + kk) * kTile + 32);
+          const f2_t cc[4] = {lo.x, lo.y, hi.x, hi.y};
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const float av = kk == 0 ? a[i].x : kk == 1 ? a[i].y : kk == 2 ? a[i].z : a[i].w;
+          for (int i = 0; i < kWaR; ++i) {
+            const f2_t av = f2_dup(kk == 0 ? a[i].x : kk == 1 ? a[i].y : kk == 2 ? a[i].z : a[i].w);
 #pragma unroll
-          for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av, cc[j], acc[i][j]);
+            for (int j = 0; j < 4; ++j) acc[i][j] = f2_fma(av, cc[j], acc[i][j]);
+          }
         }
       }
     }
-    if (w % nst == nst - 1) {
-      const long long tile = blockIdx.x + (w / nst) * gridDim.x;
-      ts_epilogue(n, q, tile * kTsRows + 8 * ty, tx, acc, alpha, beta, Bm, out, add2, out2, dn);
+    const long long row0 = tile * kWaRows + ty;
+    if (Es ? stage >= nst : stage == nst - 1) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+        if (!Es || stage == nst + h)
+          wa_half(n, q, row0, tx, h, acc, alpha, beta, Es ? Ab + 4 * tx : nullptr, Bm != nullptr,
+                  out, out2, dn.vec != 0, dn.rho != nullptr, dsum);
+    }
+    if (++buf == kWaStages) buf = 0;
+    if (++stage == ntot) {
+      if (dn.rho) {
+        // the eight lanes of a row; lane tx keeps row row0 + 4 tx, so the FP64 tail
+        // is one instruction per tile
+        float mine_ = 0.f;
+#pragma unroll
+        for (int i = 0; i < kWaR; ++i) {
+#pragma unroll
+          for (int s = 4; s > 0; s >>= 1) dsum[i] += __shfl_xor_sync(0xffffffffu, dsum[i], s);
+          if (tx == i) mine_ = dsum[i];
+          dsum[i] = 0.f;
+        }
+        const long long row = row0 + 4 * tx;
+        if (row < n) dn.rho[row] = dn.rho_b[row] + dn.occ * (double)mine_;
+      }
+#pragma unroll
+      for (int i = 0; i < kWaR; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
+      stage = 0;
+      tile += step;
     }
   }
   asm volatile("cp.async.wait_all;\n" ::: "memory");
@@ -1370,15 +1509,20 @@ static void launch_ts(Problem &P, int q, const float *A1, int k1, const float *c
   auto al16 = [](const void *ptr) { return reinterpret_cast<uintptr_t>(ptr) % 16 == 0; };
   dn.vec = q % 4 == 0 && al16(out) && al16(Bm) && al16(add2) && al16(out2) ? 1 : 0;
   const int K = k1 + (A2 ? k2 : 0) + (A3 ? k3 : 0);
+  // (the staged epilogue operand: one of Bm and add2, in 16-byte copies)
+  const float *es = Bm ? Bm : add2;
+  if (ta_aligned(A1, k1, A2, k2, A3, k3) && !(Bm && add2) && ta_aligned(es, q, es, q, es, q)) {
+    const long long ntiles = (P.n + kWaRows - 1) / kWaRows;
+    const long long nb = ntiles < P.sms ? ntiles : P.sms;
+    combine_wa_kernel<<<(int)nb, 32 * kWaWarps, combine_wa_smem(K), P.stream>>>(
+        P.n, q, A1, k1, c1, A2, k2, c2, A3, k3, c3, alpha, beta, Bm, out, add2, out2, ntiles, dn);
+    return;
+  }
   const long long ntiles = (P.n + kTsRows - 1) / kTsRows;
   long long nb = 2LL * P.sms;
   if (nb > ntiles) nb = ntiles;
-  if (ta_aligned(A1, k1, A2, k2, A3, k3))
-    combine_ta_kernel<<<(int)nb, 256, combine_ta_smem(K), P.stream>>>(
-        P.n, q, A1, k1, c1, A2, k2, c2, A3, k3, c3, alpha, beta, Bm, out, add2, out2, ntiles, dn);
-  else
-    combine_ts_kernel<<<(int)nb, 256, combine_ts_smem(K), P.stream>>>(
-        P.n, q, A1, k1, c1, A2, k2, c2, A3, k3, c3, alpha, beta, Bm, out, add2, out2, ntiles, dn);
+  combine_ts_kernel<<<(int)nb, 256, combine_ts_smem(K), P.stream>>>(
+      P.n, q, A1, k1, c1, A2, k2, c2, A3, k3, c3, alpha, beta, Bm, out, add2, out2, ntiles, dn);
 }
 
 // out = A1 C1 + A2 C2 + A3 C3 and out2 = add2 + out in one pass of the
@@ -1435,16 +1579,16 @@ ks_status launch_combine3_f32(Problem &P, const float *A1, int k1, const double 
 // Dynamic shared memory of the tall-skinny update beyond the default 48 KiB
 // (on the current device; called when a problem is created).
 ks_status configure_blas_kernels() {
-  KS_CUDA_TRY(cudaFuncSetAttribute(gram2_ta_kernel<true>,
+  KS_CUDA_TRY(cudaFuncSetAttribute(gram2_wa_kernel<true>,
                                    cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)gram_ta_smem<true>()));
-  KS_CUDA_TRY(cudaFuncSetAttribute(gram2_ta_kernel<false>,
+                                   (int)gram_wa_smem()));
+  KS_CUDA_TRY(cudaFuncSetAttribute(gram2_wa_kernel<false>,
                                    cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)gram_ta_smem<false>()));
+                                   (int)gram_wa_smem()));
   KS_CUDA_TRY(cudaFuncSetAttribute(combine_ts_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    (int)combine_ts_smem(kTsMaxK)));
-  KS_CUDA_TRY(cudaFuncSetAttribute(combine_ta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)combine_ta_smem(kTsMaxK)));
+  KS_CUDA_TRY(cudaFuncSetAttribute(combine_wa_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)combine_wa_smem(kTsMaxK)));
   return KS_OK;
 }
 

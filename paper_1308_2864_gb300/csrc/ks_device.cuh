@@ -164,6 +164,43 @@ __device__ __forceinline__ bool grid_barrier(GridBarrier *bar, int *status) {
   return grid_barrier_n(bar, status, gridDim.x * gridDim.y * gridDim.z);
 }
 
+// Packed FP32 pairs (two lanes of one 64-bit register pair): each lane rounds
+// like the scalar instruction.  On GB300 an outer-product loop of scalar FMAs
+// reaches 49 TFLOP/s (two operands per FMA from the register file stall its
+// dispatch) and the same loop of packed ones 76, the pipe's peak, also when
+// one factor is duplicated into a pair per use.
+using f2_t = unsigned long long;
+__device__ __forceinline__ f2_t f2_add(f2_t a, f2_t b) {
+  f2_t d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ f2_t f2_mul(f2_t a, f2_t b) {
+  f2_t d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ f2_t f2_fma(f2_t a, f2_t b, f2_t c) {
+  f2_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ f2_t f2_dup(float x) {
+  f2_t d;
+  asm("mov.b64 %0, {%1, %1};" : "=l"(d) : "f"(x));
+  return d;
+}
+// a - b (one rounding)
+__device__ __forceinline__ f2_t f2_sub(f2_t a, f2_t b) { return f2_fma(b, f2_dup(-1.f), a); }
+__device__ __forceinline__ void f2_split(f2_t a, float &x, float &y) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(a));
+}
+__device__ __forceinline__ double f2_sum(f2_t a) {
+  float x, y;
+  f2_split(a, x, y);
+  return (double)x + (double)y;
+}
+
 // 27-point Q1 stencil coefficient classes (see the stiffness/mass
 // construction in ks_stencil.cu): centre, face (6), edge (12), corner (8).
 struct StencilCoef {

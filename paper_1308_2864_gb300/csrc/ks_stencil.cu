@@ -637,35 +637,6 @@ struct StF2 {
   static_assert(kStThreads == PC / 2 * TX * (TY / R), "one thread per orbital pair and column");
 };
 
-using f2_t = unsigned long long;
-__device__ __forceinline__ f2_t f2_add(f2_t a, f2_t b) {
-  f2_t d;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ f2_t f2_mul(f2_t a, f2_t b) {
-  f2_t d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ f2_t f2_fma(f2_t a, f2_t b, f2_t c) {
-  f2_t d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-__device__ __forceinline__ f2_t f2_dup(float x) {
-  f2_t d;
-  asm("mov.b64 %0, {%1, %1};" : "=l"(d) : "f"(x));
-  return d;
-}
-// a - b (one rounding)
-__device__ __forceinline__ f2_t f2_sub(f2_t a, f2_t b) { return f2_fma(b, f2_dup(-1.f), a); }
-__device__ __forceinline__ double f2_sum(f2_t a) {
-  float x, y;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(a));
-  return (double)x + (double)y;
-}
-
 template <int Kind>
 constexpr size_t st_f2_smem() {
   return (size_t)kStStages * (StF2::BOX + st_naux<float, Kind>() * StF2::AUX) * sizeof(float) + 128;
