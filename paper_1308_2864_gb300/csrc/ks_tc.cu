@@ -285,21 +285,29 @@ __global__ void __launch_bounds__(kTcThreads, 1) gram_tc_kernel(long long n, int
   tc_teardown(tmem);
 }
 
+// Byte offset of element (r, k) of an R x KS K-major tile (core matrices of 8
+// rows x 16 bytes, K-adjacent ones 128 bytes apart, row groups 32 KS apart).
+template <int KS>
+__device__ __forceinline__ int kmajor_offset_of(int r, int k) {
+  return (r >> 3) * (32 * KS) + (k >> 2) * 128 + (r & 7) * 16 + (k & 3) * 4;
+}
+
 // Coefficient image of the update: for column tile ct (256 columns of
-// q) and stage s (K-values 32 s .. 32 s + 31 of [C1; C2]), the hi and lo
+// q) and stage s (K-values KS s .. KS s + KS - 1 of [C1; C2]), the hi and lo
 // K-major tiles exactly as a stage buffer holds them, so a block copies
-// each stage's 64 KiB with cp.async.
+// each stage as one contiguous piece.
+template <int KS>
 __global__ void combine_image_kernel(int q, int k1, const double *__restrict__ C1, int k2,
                                      const double *__restrict__ C2, int stages, float *img) {
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const long long per_stage = (long long)kTcN * kTcK;
+  const long long per_stage = (long long)kTcN * KS;
   const long long total = (long long)((q + kTcN - 1) / kTcN) * stages * per_stage;
   if (e >= total) return;
   const int within = (int)(e % per_stage);
   const long long ts = e / per_stage;             // ct * stages + s
   const int s = (int)(ts % stages), ct = (int)(ts / stages);
-  const int c = within / kTcK, k = within % kTcK;
-  const int kk = s * kTcK + k, col = ct * kTcN + c;
+  const int c = within / KS, k = within % KS;
+  const int kk = s * KS + k, col = ct * kTcN + c;
   double x = 0.0;
   if (col < q) {
     if (kk < k1) x = C1[(long long)kk * q + col];
@@ -308,9 +316,9 @@ __global__ void combine_image_kernel(int q, int k1, const double *__restrict__ C
   float hi, lo;
   split_tf32((float)x, hi, lo);
   unsigned char *base = (unsigned char *)(img + ts * 2 * per_stage);
-  const int off = kmajor_offset(c, k);
+  const int off = kmajor_offset_of<KS>(c, k);
   *(float *)(base + off) = hi;
-  *(float *)(base + kTileBBytes + off) = lo;
+  *(float *)(base + kTcN * KS * 4 + off) = lo;
 }
 
 __device__ __forceinline__ void cp_async16(void *dst, const void *src) {
@@ -417,6 +425,232 @@ __global__ void __launch_bounds__(kTcThreads, 1) combine_tc_kernel(
     }
   }
   tc_teardown(tmem);
+}
+
+// Bounded wait on a phase of an mbarrier that also gives up once another
+// role of the block has set *abort; a wait that runs out sets it.
+__device__ __forceinline__ bool role_wait(uint64_t *bar, uint32_t parity, volatile int *abort) {
+  const uint32_t a = smem_u32(bar);
+  for (long long spins = 0; spins < kSpinLimit; ++spins) {
+    uint32_t done;
+    asm volatile("{\n.reg .pred q;\nmbarrier.try_wait.parity.shared::cta.b64 q, [%1], %2;\n"
+                 "selp.u32 %0, 1, 0, q;\n}\n"
+                 : "=r"(done) : "r"(a), "r"(parity) : "memory");
+    if (done) return true;
+    if (*abort) return false;
+  }
+  *abort = 1;
+  return false;
+}
+
+__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(smem_u32(bar)) : "memory");
+}
+
+// ---------------------------------------------------------------- wide updates
+// out = alpha (A1 C1 + A2 C2) + beta Bm, pipelined by warp role, for operands
+// whose rows allow 16-byte loads.  The MMAs bound it when nothing waits (three
+// TF32 products: 116 GFLOP of 48^3 x 512 are 0.36 ms at half the measured BF16
+// rate); next to them L2, which delivers the coefficient image to every row
+// tile.  So a block owns 256 rows x 256 columns, two 128-row accumulators that
+// share each coefficient stage (half the image traffic of 128-row tiles), and
+// K advances in stages of 16 through a ring of kWSlots slots:
+//   warps 0-7  load A two stages ahead in registers, split it into TF32 hi and
+//              lo (kmajor_offset_of<16>), then read the accumulators out;
+//   warp 8     (one thread) issues 2 K-steps x 2 row halves x (hi.hi + hi.lo +
+//              lo.hi) per stage; its commits release the slot;
+//   warp 9     (one thread) copies the stage's hi and lo coefficients, 32 KiB in
+//              one bulk copy.
+// Roles meet on mbarriers only.  (The block-synchronous kernel above copies
+// 64 KiB of image per stage, then waits for them before its MMAs: 1.11 ms at 48^3
+// x 512, K = 1024, against 0.48 ms here, 240 TF/s of useful products.)  The MMA
+// order per accumulator is that kernel's, so the results are too.  It stays for
+// operands without 16-byte rows.  Every wait is bounded; a role that gives up sets the
+// block's abort flag, the others stop at their next poll, copies and MMAs in
+// flight get a bounded wait, and the block records KS_ETIMEOUT.
+constexpr int kWM = 256, kWK = 16, kWSlots = 3;
+constexpr int kWTile = 256 * kWK * 4;                       // 16 KiB: hi or lo of A or B
+constexpr int kWStage = 4 * kWTile;                         // A hi, A lo, B hi, B lo
+constexpr int kWSmem = kWSlots * kWStage + 1024;
+constexpr int kWThreads = 320, kWCols = 512;
+static_assert(kWSlots * kWStage >= 8 * 64 * 33 * 4, "the read-out tiles reuse the ring");
+
+__device__ __forceinline__ uint64_t smem_desc16(uint32_t saddr) {
+  uint64_t d = (uint64_t)((saddr >> 4) & 0x3FFF);
+  d |= (uint64_t)(128 >> 4) << 16;                          // K-adjacent core matrices
+  d |= (uint64_t)(512 >> 4) << 32;                          // row groups of 8
+  d |= (uint64_t)1 << 46;
+  return d;
+}
+
+__device__ __forceinline__ void bulk_copy(void *dst, const void *src, uint32_t bytes,
+                                          uint64_t *bar) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::
+          "r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar))
+      : "memory");
+}
+
+__global__ void __launch_bounds__(kWThreads, 1) combine_tcw_kernel(
+    long long n, int q, const float *__restrict__ A1, int k1, const float *__restrict__ A2, int k2,
+    const float *__restrict__ img, int stages, int ncol, float alpha, float beta,
+    const float *__restrict__ Bm, float *__restrict__ out, int *status) {
+  extern __shared__ __align__(1024) unsigned char dyn_raw[];
+  unsigned char *ring = (unsigned char *)(((uintptr_t)dyn_raw + 1023) & ~(uintptr_t)1023);
+  __shared__ __align__(8) uint64_t full[kWSlots], empty[kWSlots], accdone;
+  __shared__ uint32_t tmem_slot;
+  __shared__ int abort_s;
+  volatile int *abort = &abort_s;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const long long row0 = (long long)(blockIdx.x / ncol) * kWM;
+  const int ct = blockIdx.x % ncol, c0 = ct * kTcN;
+  const int K = k1 + (A2 ? k2 : 0);
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                 :: "r"(smem_u32(&tmem_slot)), "r"(kWCols));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  if (tid == 0) {
+    abort_s = 0;
+    for (int s = 0; s < kWSlots; ++s) {
+      mbar_init(&full[s], 9);                               // eight A warps, the copy
+      mbar_init(&empty[s], 1);
+    }
+    mbar_init(&accdone, 1);
+    fence_barrier_init();
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;");
+  const uint32_t tmem = tmem_slot;
+  int copied = 0;
+  if (warp < 8) {
+    // lane: row lane % 8 of a group of 8, K-values 4 (lane / 8) .. + 3 of the stage;
+    // groups warp + 8 i.  An 8-lane phase of a 16-byte store covers a core matrix.
+    const int r = lane & 7, kc = lane >> 3;
+    float4 va[4], vb[4];
+    auto load = [&](int s, float4 (&v)[4]) {
+      const int k = s * kWK + 4 * kc;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const long long row = row0 + (warp + 8 * i) * 8 + r;
+        v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (row < n && k < K && s < stages) {
+          if (k < k1) {
+            if (KS_IN(row * k1 + k + 3, n * k1)) v[i] = *reinterpret_cast<const float4 *>(A1 + row * k1 + k);
+          } else if (KS_IN(row * k2 + k - k1 + 3, n * k2)) {
+            v[i] = *reinterpret_cast<const float4 *>(A2 + row * k2 + (k - k1));
+          }
+        }
+      }
+    };
+    auto put = [&](int s, const float4 (&v)[4]) -> bool {
+      const int slot = s % kWSlots, u = s / kWSlots;
+      if (u > 0 && !role_wait(&empty[slot], (uint32_t)((u - 1) & 1), abort)) return false;
+      unsigned char *st = ring + slot * kWStage;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        float4 hi, lo;
+        split_tf32(v[i].x, hi.x, lo.x);
+        split_tf32(v[i].y, hi.y, lo.y);
+        split_tf32(v[i].z, hi.z, lo.z);
+        split_tf32(v[i].w, hi.w, lo.w);
+        const int off = (warp + 8 * i) * (32 * kWK) + kc * 128 + r * 16;
+        *reinterpret_cast<float4 *>(st + off) = hi;
+        *reinterpret_cast<float4 *>(st + kWTile + off) = lo;
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&full[slot]);
+      return true;
+    };
+    load(0, va);
+    load(1, vb);
+    for (int s = 0; s < stages; s += 2) {
+      if (!put(s, va)) break;
+      load(s + 2, va);
+      if (s + 1 < stages) {
+        if (!put(s + 1, vb)) break;
+        load(s + 3, vb);
+      }
+    }
+    if (role_wait(&accdone, 0u, abort) && !*abort) {
+      asm volatile("tcgen05.fence::after_thread_sync;");
+      // accumulator -> the warp's own transposed tile in the (now idle) ring, 64
+      // columns at a time, then row-contiguous stores
+      const int half = warp >> 2, quad = warp & 3;
+      float *T = reinterpret_cast<float *>(ring) + warp * 64 * 33;
+      const long long rbase = row0 + half * 128 + quad * 32;
+#pragma unroll 1
+      for (int cb = 0; cb < kTcN; cb += 64) {
+        uint32_t v[64];
+        tmem_ld64(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(half * kTcN + cb), v);
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < 64; ++j) T[j * 33 + lane] = __uint_as_float(v[j]);
+        __syncwarp();
+#pragma unroll 4
+        for (int rr = 0; rr < 32; ++rr) {
+          const long long row = rbase + rr;
+          if (row >= n) break;
+#pragma unroll
+          for (int w = 0; w < 2; ++w) {
+            const int col = c0 + cb + lane + 32 * w;
+            if (col >= q || !KS_IN(row * q + col, n * q)) continue;
+            float y = alpha * T[(lane + 32 * w) * 33 + rr];
+            if (Bm) y = fmaf(beta, Bm[row * q + col], y);
+            out[row * q + col] = y;
+          }
+        }
+      }
+    }
+  } else if (warp == 8 && lane == 0) {
+    int s = 0;
+    for (; s < stages; ++s) {
+      const int slot = s % kWSlots;
+      if (!role_wait(&full[slot], (uint32_t)((s / kWSlots) & 1), abort)) break;
+      asm volatile("tcgen05.fence::after_thread_sync;");
+      const uint32_t sa = smem_u32(ring + slot * kWStage), sb = sa + 2 * kWTile;
+#pragma unroll
+      for (int ks = 0; ks < kWK / 8; ++ks)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          // 128 rows are 16 groups of 512 bytes; a K-step is two core matrices
+          const uint32_t ah = sa + h * 8192 + ks * 256, bh = sb + ks * 256;
+          const uint32_t d = tmem + (uint32_t)(h * kTcN);
+          mma_tf32(d, smem_desc16(ah), smem_desc16(bh), (s > 0 || ks > 0) ? 1u : 0u);
+          mma_tf32(d, smem_desc16(ah), smem_desc16(bh + kWTile), 1u);
+          mma_tf32(d, smem_desc16(ah + kWTile), smem_desc16(bh), 1u);
+        }
+      commit(&empty[slot]);
+    }
+    commit(&accdone);                                       // MMAs in flight, also after an abort
+    mbar_wait(smem_u32(&accdone), 0u);
+  } else if (warp == 9 && lane == 0) {
+    for (int s = 0; s < stages; ++s) {
+      const int slot = s % kWSlots, u = s / kWSlots;
+      if (u > 0 && !role_wait(&empty[slot], (uint32_t)((u - 1) & 1), abort)) break;
+      mbar_arrive_expect_tx(&full[slot], 2 * kWTile);
+      bulk_copy(ring + slot * kWStage + 2 * kWTile,
+                reinterpret_cast<const unsigned char *>(img) +
+                    ((long long)ct * stages + s) * (2 * kWTile),
+                2 * kWTile, &full[slot]);
+      copied = s + 1;
+    }
+  }
+  __syncthreads();
+  if (*abort) {
+    if (tid == 0) atomicCAS(status, 0, (int)KS_ETIMEOUT);
+    // copies still in flight write the ring: a bounded wait for each slot's last
+    // one (a slot whose A warps gave up never completes)
+    if (warp == 9 && lane == 0)
+      for (int s = copied > kWSlots ? copied - kWSlots : 0; s < copied; ++s)
+        mbar_wait(smem_u32(&full[s % kWSlots]), (uint32_t)((s / kWSlots) & 1));
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;");
+  __syncthreads();
+  if (warp == 0)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(kWCols));
 }
 
 // ---------------------------------------------------------------- narrow updates
@@ -558,26 +792,6 @@ __global__ void combine_image64_kernel(int q, Img64 im, int stages, float *__res
   const int off = sw128_offset(c, k);
   *(float *)(base + off) = hi;
   *(float *)(base + kNImgBytes / 2 + off) = lo;
-}
-
-// Bounded wait on a phase of an mbarrier that also gives up once another
-// role of the block has set *abort; a wait that runs out sets it.
-__device__ __forceinline__ bool role_wait(uint64_t *bar, uint32_t parity, volatile int *abort) {
-  const uint32_t a = smem_u32(bar);
-  for (long long spins = 0; spins < kSpinLimit; ++spins) {
-    uint32_t done;
-    asm volatile("{\n.reg .pred q;\nmbarrier.try_wait.parity.shared::cta.b64 q, [%1], %2;\n"
-                 "selp.u32 %0, 1, 0, q;\n}\n"
-                 : "=r"(done) : "r"(a), "r"(parity) : "memory");
-    if (done) return true;
-    if (*abort) return false;
-  }
-  *abort = 1;
-  return false;
-}
-
-__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(smem_u32(bar)) : "memory");
 }
 
 // Epilogue of 32 accumulator columns c0 .. c0 + 31 of one row: out, and with
@@ -791,6 +1005,8 @@ ks_status configure_tc_kernels() {
                                    kTcSmem));
   KS_CUDA_TRY(cudaFuncSetAttribute(combine_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    kTcSmem));
+  KS_CUDA_TRY(cudaFuncSetAttribute(combine_tcw_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   kWSmem));
   return KS_OK;
 }
 
@@ -802,23 +1018,39 @@ ks_status launch_combine_tc(Problem &P, const float *A1, int k1, const double *C
                             const float *A2, int k2, const double *C2, double alpha, double beta,
                             const float *Bm, float *out, int q) {
   const int K = k1 + (A2 ? k2 : 0);
-  const int stages = (K + kTcK - 1) / kTcK;
-  const long long img_len = (long long)((q + kTcN - 1) / kTcN) * stages * 2 * kTcN * kTcK;
+  // 16-byte loads of A: every width a multiple of 4, aligned bases
+  const bool wide = k1 % 4 == 0 && (!A2 || k2 % 4 == 0) &&
+                    reinterpret_cast<uintptr_t>(A1) % 16 == 0 &&
+                    reinterpret_cast<uintptr_t>(A2) % 16 == 0;
+  const int ks = wide ? kWK : kTcK;
+  const int stages = (K + ks - 1) / ks, ncol = (q + kTcN - 1) / kTcN;
+  const long long img_len = (long long)ncol * stages * 2 * kTcN * ks;
   if ((size_t)img_len > P.tc_img_len) return set_error(KS_EINVAL, "combine_tc: image too large");
   {
     ProfScope ps_(P.stream, KP_REDUCE);
-    const long long elems = img_len / 2;
-    combine_image_kernel<<<(int)((elems + 255) / 256), 256, 0, P.stream>>>(
-        q, k1, C1, A2 ? k2 : 0, C2, stages, P.tc_img);
+    const int nb = (int)((img_len / 2 + 255) / 256);
+    if (wide)
+      combine_image_kernel<kWK><<<nb, 256, 0, P.stream>>>(q, k1, C1, A2 ? k2 : 0, C2, stages,
+                                                          P.tc_img);
+    else
+      combine_image_kernel<kTcK><<<nb, 256, 0, P.stream>>>(q, k1, C1, A2 ? k2 : 0, C2, stages,
+                                                           P.tc_img);
   }
   KS_CUDA_TRY(cudaGetLastError());
-  dim3 grid((unsigned)((P.n + kTcM - 1) / kTcM), (unsigned)((q + kTcN - 1) / kTcN));
   {
     ProfScope ps_(P.stream, KP_COMBINE, 2.0 * P.n * q * K,
                   (double)P.n * (K + q * (Bm ? 2 : 1)) * sizeof(float));
-    combine_tc_kernel<<<grid, kTcThreads, kTcSmem, P.stream>>>(
-        P.n, q, A1, k1, A2, A2 ? k2 : 0, P.tc_img, stages, (float)alpha, (float)beta, Bm, out,
-        P.dstatus);
+    if (wide) {
+      const unsigned nb = (unsigned)((P.n + kWM - 1) / kWM) * (unsigned)ncol;
+      combine_tcw_kernel<<<nb, kWThreads, kWSmem, P.stream>>>(
+          P.n, q, A1, k1, A2, A2 ? k2 : 0, P.tc_img, stages, ncol, (float)alpha, (float)beta, Bm,
+          out, P.dstatus);
+    } else {
+      const dim3 grid((unsigned)((P.n + kTcM - 1) / kTcM), (unsigned)ncol);
+      combine_tc_kernel<<<grid, kTcThreads, kTcSmem, P.stream>>>(
+          P.n, q, A1, k1, A2, A2 ? k2 : 0, P.tc_img, stages, (float)alpha, (float)beta, Bm, out,
+          P.dstatus);
+    }
   }
   KS_CUDA_TRY(cudaGetLastError());
   return KS_OK;

@@ -85,3 +85,28 @@ def test_cayley_factor_sizes(p):
     for tau in (1e-3, 0.5):
         got = P.retract(ks.KS_CAYLEY, dev(X), dev(pt.ev.EX), tau).cpu().numpy()
         assert_rel(got, ost.retract_cayley(model, pt, tau), 1e-11, f"tau {tau}")
+
+
+@pytest.mark.parametrize("N,k1,k2,q", [(4, 36, 36, 33), (7, 40, 36, 260), (7, 256, 256, 256),
+                                       (8, 300, 260, 300), (10, 260, 4, 257), (12, 512, 512, 512)])
+def test_wide_fp32_update_on_tensor_cores(N, k1, k2, q):
+    # widths that are multiples of 4 (the pipelined form): K of 72 .. 1024 in
+    # stages of 16 with a ragged last one, fewer rows than a tile (4^3) and ragged
+    # row and column tiles; the bound of the general tensor-core update test
+    import paper_1308_2864_gb300 as ks
+    s = ki.small_system(N=N, L=7.0, natoms=2, p=max(k1, k2, q), Z=4.0, seed=4)
+    P = ks.Problem.from_system(s)
+    P.set_tensor_cores(2)
+    rng = np.random.default_rng(29)
+    A1 = rng.standard_normal((s.n, k1)).astype(np.float32)
+    A2 = rng.standard_normal((s.n, k2)).astype(np.float32)
+    Bm = rng.standard_normal((s.n, q)).astype(np.float32)
+    C1, C2 = rng.standard_normal((k1, q)), rng.standard_normal((k2, q))
+    t = lambda a: torch.from_numpy(a).cuda()
+    A1d, A2d = A1.astype(np.float64), A2.astype(np.float64)
+    for bm, beta in ((None, 0.0), (Bm, 2.0)):
+        got = P.step_combine_f32(t(A1), t(C1), t(A2), t(C2), alpha=-0.5, beta=beta,
+                                 Bm=None if bm is None else t(bm)).cpu().numpy()
+        want = -0.5 * (A1d @ C1 + A2d @ C2) + beta * Bm
+        bound = 0.5 * (np.abs(A1d) @ np.abs(C1) + np.abs(A2d) @ np.abs(C2)) + beta * np.abs(Bm)
+        assert np.all(np.abs(got - want) <= 4e-6 * bound + 1e-12)
