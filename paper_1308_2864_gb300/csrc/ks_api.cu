@@ -10,8 +10,10 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <utility>
+#include <vector>
 
 #include "ks_internal.cuh"
 
@@ -98,6 +100,49 @@ ks_status validate_desc(const ks_problem_desc *d) {
   return KS_OK;
 }
 
+// Pinned host slots for the problems' scalar mirrors.  A copy into pageable
+// memory makes the host wait for the stream inside each call, so the two copies
+// of every line-search decision cost some 20 us; one copy into a pinned slot
+// takes one round trip.  Pinning per problem would cost more than it saves
+// for short-lived problems (and freeing it would wait for the device), so
+// slots come from slabs that live as long as the process: at most as many as
+// problems were alive at once, rounded up to a slab.  Any thread may take or
+// return a slot.
+namespace {
+constexpr size_t kSlotBytes = 256;
+constexpr int kSlabSlots = 64;
+static_assert((SC_COUNT + 1) * sizeof(double) <= kSlotBytes, "scalars and status fit a slot");
+std::mutex g_slot_mu;
+std::vector<void *> g_slots;
+
+ks_status take_slot(double **out) {
+  std::lock_guard<std::mutex> lk(g_slot_mu);
+  if (!g_slots.empty()) {
+    // a device reset in this process releases pinned memory: such slots are stale
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, g_slots.back()) != cudaSuccess ||
+        at.type != cudaMemoryTypeHost) {
+      cudaGetLastError();
+      g_slots.clear();
+    }
+  }
+  if (g_slots.empty()) {
+    void *slab = nullptr;
+    KS_CUDA_TRY(cudaHostAlloc(&slab, kSlotBytes * kSlabSlots, cudaHostAllocPortable));
+    for (int i = kSlabSlots - 1; i >= 0; --i) g_slots.push_back((char *)slab + i * kSlotBytes);
+  }
+  *out = static_cast<double *>(g_slots.back());
+  g_slots.pop_back();
+  std::memset(*out, 0, kSlotBytes);
+  return KS_OK;
+}
+
+void return_slot(double *slot) {
+  std::lock_guard<std::mutex> lk(g_slot_mu);
+  g_slots.push_back(slot);
+}
+}  // namespace
+
 // Device memory is stream-ordered (cudaMallocAsync / cudaFreeAsync on the
 // problem's stream), so creating and destroying problems does not
 // synchronise the device while other problems run on other streams.
@@ -107,12 +152,10 @@ static void free_problem(Problem &P) {
   f(P.vext); f(P.rho); f(P.vH); f(P.veff); f(P.rho_b); f(P.veff_b); f(P.zero_n); f(P.cg_r); f(P.cg_pa); f(P.cg_pb); f(P.cg_q);
   f(P.cg_z); f(P.cg_rho_prev); f(P.cg_t1); f(P.cg_t2); f(P.dst_phi); f(P.dst_kap); f(P.dst_mu);
   for (auto &b : P.blk) f(b);
-  f(P.pp); f(P.cf); f(P.rt32); f(P.tc_img); f(P.oz_emax); f(P.oz_img); f(P.oz_rowexp); f(P.partials); f(P.scal); f(P.atoms_dev); f(P.thomas_w); f(P.bar); f(P.red_counter); f(P.dstatus);
-  delete[] P.scal_host;
-  delete[] P.dstatus_host;
-  P.scal_host = nullptr;
-  P.dstatus_host = nullptr;
+  f(P.pp); f(P.cf); f(P.rt32); f(P.tc_img); f(P.oz_emax); f(P.oz_img); f(P.oz_rowexp); f(P.partials); f(P.scal); f(P.atoms_dev); f(P.thomas_w); f(P.bar); f(P.red_counter);
   if (s) cudaStreamSynchronize(s);
+  if (P.scal_host) return_slot(P.scal_host);      // no copy into it is in flight any more
+  P.scal_host = nullptr;
   cudaGetLastError();
   if (P.own_stream && P.stream) cudaStreamDestroy(P.stream);
 }
@@ -128,14 +171,17 @@ static ks_status dalloc(T **ptr, size_t count, Problem &P) {
 
 static double *sm(Problem &P, int which) { return P.pp + (size_t)which * P.p * P.p; }
 
-// Copy device scalars and the status word to the host and wait.
-static ks_status sync_scalars(Problem &P) {
-  KS_CUDA_TRY(cudaMemcpyAsync(P.scal_host, P.scal, SC_COUNT * sizeof(double),
+ks_status read_scalars(Problem &P) {
+  KS_CUDA_TRY(cudaMemcpyAsync(P.scal_host, P.scal, (SC_COUNT + 1) * sizeof(double),
                               cudaMemcpyDeviceToHost, P.stream));
-  KS_CUDA_TRY(cudaMemcpyAsync(P.dstatus_host, P.dstatus, sizeof(int), cudaMemcpyDeviceToHost,
-                              P.stream));
   KS_CUDA_TRY(cudaStreamSynchronize(P.stream));
   prof_collect();
+  return KS_OK;
+}
+
+// Copy device scalars and the status word to the host and wait.
+static ks_status sync_scalars(Problem &P) {
+  KS_TRY(read_scalars(P));
   const int st = *P.dstatus_host;
   if (st != KS_OK) {
     KS_CUDA_TRY(cudaMemsetAsync(P.dstatus, 0, sizeof(int), P.stream));
@@ -1111,24 +1157,21 @@ ks_status ks_problem_create(const ks_problem_desc *d, ks_problem **out) {
   if ((size_t)4 * P.cg_blocks > part) part = (size_t)4 * P.cg_blocks;
   P.partials_len = part;
   ALLOC(P.partials, part);
-  ALLOC(P.scal, SC_COUNT);
+  ALLOC(P.scal, SC_COUNT + 1);
+  P.dstatus = reinterpret_cast<int *>(P.scal + SC_COUNT);
   ALLOC(P.atoms_dev, P.atoms_host.size());
   ALLOC(P.thomas_w, (size_t)P.N);
   ALLOC(P.bar, 1);
   ALLOC(P.red_counter, 1);
-  ALLOC(P.dstatus, 1);
 #undef ALLOC
-  P.scal_host = new (std::nothrow) double[SC_COUNT];
-  P.dstatus_host = new (std::nothrow) int[1];
-  if (!P.scal_host || !P.dstatus_host) return fail(set_error(KS_ENOMEM, "host allocation failed"));
+  if ((st = take_slot(&P.scal_host)) != KS_OK) return fail(st);
+  P.dstatus_host = reinterpret_cast<int *>(P.scal_host + SC_COUNT);
   e = cudaMemcpyAsync(P.atoms_dev, P.atoms_host.data(), P.atoms_host.size() * sizeof(double),
                       cudaMemcpyHostToDevice, P.stream);
   if (e != cudaSuccess) return fail(cuda_error(e, "copy atoms"));
-  e = cudaMemsetAsync(P.scal, 0, SC_COUNT * sizeof(double), P.stream);
+  e = cudaMemsetAsync(P.scal, 0, (SC_COUNT + 1) * sizeof(double), P.stream);
   if (e != cudaSuccess) return fail(cuda_error(e, "memset"));
   e = cudaMemsetAsync(P.red_counter, 0, sizeof(unsigned int), P.stream);
-  if (e != cudaSuccess) return fail(cuda_error(e, "memset"));
-  e = cudaMemsetAsync(P.dstatus, 0, sizeof(int), P.stream);
   if (e != cudaSuccess) return fail(cuda_error(e, "memset"));
   e = cudaMemsetAsync(P.vH, 0, n * sizeof(double), P.stream);
   if (e != cudaSuccess) return fail(cuda_error(e, "memset"));

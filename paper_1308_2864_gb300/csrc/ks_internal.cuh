@@ -135,13 +135,13 @@ struct Problem {
   double *partials = nullptr;      // Gram partial tiles and block partial sums
   size_t partials_len = 0;
   double *scal = nullptr;          // device scalars (SC_*)
-  double *scal_host = nullptr;     // pinned mirror
+  double *scal_host = nullptr;     // pinned mirror of scal and the status word
   double *atoms_dev = nullptr;
   double *thomas_w = nullptr;      // N pivots of the 1-D mass solve
   GridBarrier *bar = nullptr;
   unsigned int *red_counter = nullptr;  // last-block reduction counter (rests at 0)
-  int *dstatus = nullptr;          // device status word
-  int *dstatus_host = nullptr;     // pinned mirror
+  int *dstatus = nullptr;          // device status word (after the scalars: one copy reads both)
+  int *dstatus_host = nullptr;     // its place in scal_host
 
   // State of the last ConOptM phase (for ks_state_save / resume): slot
   // indices of the current/previous/trial blocks and the line-search scalars.
@@ -174,6 +174,8 @@ struct Problem {
   size_t bytes = 0;
 };
 
+// Device scalars and status word to their host mirror, waiting for the stream.
+ks_status read_scalars(Problem &P);
 size_t problem_bytes(int N, int p, int sms);
 // Checks every field of a problem description on the host (no device call);
 // KS_EINVAL with the reason recorded, else KS_OK.

@@ -7,12 +7,10 @@ using namespace ks;
 
 namespace {
 
+// Waits for the step; its device status, with the scalars in P.scal_host.
 ks_status finish(Problem &P) {
-  int st = 0;
-  KS_CUDA_TRY(cudaMemcpyAsync(P.dstatus_host, P.dstatus, sizeof(int), cudaMemcpyDeviceToHost,
-                              P.stream));
-  KS_CUDA_TRY(cudaStreamSynchronize(P.stream));
-  st = *P.dstatus_host;
+  KS_TRY(read_scalars(P));
+  const int st = *P.dstatus_host;
   if (st != KS_OK) {
     KS_CUDA_TRY(cudaMemsetAsync(P.dstatus, 0, sizeof(int), P.stream));
     KS_CUDA_TRY(cudaStreamSynchronize(P.stream));
@@ -21,10 +19,10 @@ ks_status finish(Problem &P) {
   return KS_OK;
 }
 
-ks_status read_scalars(Problem &P, int first, int count, double *out) {
-  KS_CUDA_TRY(cudaMemcpyAsync(out, P.scal + first, count * sizeof(double), cudaMemcpyDeviceToHost,
-                              P.stream));
-  return finish(P);
+ks_status finish_scalars(Problem &P, int first, int count, double *out) {
+  KS_TRY(finish(P));
+  for (int i = 0; i < count; ++i) out[i] = P.scal_host[first + i];
+  return KS_OK;
 }
 
 }  // namespace
@@ -41,7 +39,7 @@ ks_status ks_step_vext(ks_problem *kp, double *vext) {
 
 ks_status ks_step_eii(ks_problem *kp, double *eii) {
   if (!kp || !eii) return set_error(KS_EINVAL, "null argument");
-  return read_scalars(kp->P, SC_EII, 1, eii);
+  return finish_scalars(kp->P, SC_EII, 1, eii);
 }
 
 ks_status ks_step_density(ks_problem *kp, const double *X, double *rho) {
@@ -57,11 +55,8 @@ ks_status ks_step_hartree(ks_problem *kp, const double *rho, double *vH, int war
   double *r = resid ? resid : P.cg_r;
   KS_TRY(launch_cg(P, rho, vH, r, warm != 0));
   P.cg_inc_ok = false;     // the caller's vH and residual, not the loop's
-  double it = 0;
-  KS_CUDA_TRY(cudaMemcpyAsync(&it, P.scal + SC_CG_ITERS, sizeof(double), cudaMemcpyDeviceToHost,
-                              P.stream));
   ks_status st = finish(P);
-  if (iters) *iters = (int)it;
+  if (iters) *iters = (int)P.scal_host[SC_CG_ITERS];
   return st;
 }
 
@@ -76,7 +71,7 @@ ks_status ks_step_potential(ks_problem *kp, const double *rho, const double *vH,
   }
   KS_TRY(launch_potential(P, rho, vH, r, veff, true));
   double e[4];
-  KS_TRY(read_scalars(P, SC_EEXT, 4, e));
+  KS_TRY(finish_scalars(P, SC_EEXT, 4, e));
   if (energies)
     for (int i = 0; i < 4; ++i) energies[i] = e[i];
   return KS_OK;
@@ -88,7 +83,7 @@ ks_status ks_step_hamiltonian(ks_problem *kp, const double *X, const double *vef
   Problem &P = kp->P;
   KS_TRY(launch_hamiltonian(P, X, veff, EX, MX, P.scal + SC_EKIN));
   double k = 0;
-  KS_TRY(read_scalars(P, SC_EKIN, 1, &k));
+  KS_TRY(finish_scalars(P, SC_EKIN, 1, &k));
   if (kinetic) *kinetic = k;
   return KS_OK;
 }
@@ -99,7 +94,7 @@ ks_status ks_step_hamiltonian_f32(ks_problem *kp, const float *X, const double *
   Problem &P = kp->P;
   KS_TRY(launch_hamiltonian<float>(P, X, veff, EX, MX, P.scal + SC_EKIN));
   double k = 0;
-  KS_TRY(read_scalars(P, SC_EKIN, 1, &k));
+  KS_TRY(finish_scalars(P, SC_EKIN, 1, &k));
   if (kinetic) *kinetic = k;
   return KS_OK;
 }
