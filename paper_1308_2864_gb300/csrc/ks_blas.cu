@@ -183,6 +183,33 @@ __global__ void gram_reduce_kernel(int chunks, long long len, const double *__re
 // partial.
 constexpr int kSmallPQ = 8;
 
+// Sums v[0 .. V) over the 32 lanes, the results spread over them: each round
+// a lane keeps half of its values and gets its partner's share of that half, so
+// 16 values take 16 FP64 adds (a butterfly per value: 80) and 64 take 62.  Lane
+// holds the sum of index i (returned) in v[0] (V = 16; both lanes of a pair) or
+// of i and i + 1 in v[0], v[1] (V = 64).
+template <int V>
+__device__ __forceinline__ int warp_scatter_sum(double (&v)[V], int lane) {
+  int idx = 0, m = V / 2;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    if (m >= 1) {
+      const bool up = (lane & o) != 0;
+#pragma unroll
+      for (int i = 0; i < V / 2; ++i)
+        if (i < m) {
+          const double keep = up ? v[i + m] : v[i], send = up ? v[i] : v[i + m];
+          v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+      if (up) idx += m;
+      m >>= 1;
+    } else {
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+    }
+  }
+  return idx;
+}
+
 template <typename T>
 __device__ __forceinline__ void gram_small_body(long long n, int pa, int qb, long long rows_per,
                                                 const T *__restrict__ A, const T *__restrict__ B,
@@ -213,17 +240,23 @@ __device__ __forceinline__ void gram_small_body(long long n, int pa, int qb, lon
     }
   }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (pa <= 4 && qb <= 4) {
+    double v[16];
 #pragma unroll
-  for (int a = 0; a < kSmallPQ; ++a) {
-    if (a >= pa) break;
+    for (int a = 0; a < 4; ++a)
 #pragma unroll
-    for (int b = 0; b < kSmallPQ; ++b) {
-      if (b >= qb) break;
-      double v = (double)acc[a][b];
+      for (int b = 0; b < 4; ++b) v[4 * a + b] = (double)acc[a][b];
+    const int i = warp_scatter_sum<16>(v, lane);
+    if ((lane & 1) == 0) red[warp][(i >> 2) * kSmallPQ + (i & 3)] = v[0];
+  } else {
+    double v[64];
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (lane == 0) red[warp][a * kSmallPQ + b] = v;
-    }
+    for (int a = 0; a < 8; ++a)
+#pragma unroll
+      for (int b = 0; b < 8; ++b) v[8 * a + b] = (double)acc[a][b];
+    const int i = warp_scatter_sum<64>(v, lane);
+    red[warp][i] = v[0];
+    red[warp][i + 1] = v[1];
   }
   __syncthreads();
   for (int e = threadIdx.x; e < pa * qb; e += blockDim.x) {
@@ -310,13 +343,39 @@ __global__ void __launch_bounds__(256) gram_mid_kernel(long long n, int pa, int 
   gram_mid_body<T>(n, pa, qb, rows_per, A, B, part, blockIdx.x);
 }
 
+// out (null: left to the reduction kernel): the last block to finish sums the
+// chunks, in chunk order, and re-arms the counter.
 template <typename T>
 __global__ void __launch_bounds__(256) gram_small_kernel(long long n, int pa, int qb,
                                                          long long rows_per,
                                                          const T *__restrict__ A,
                                                          const T *__restrict__ B,
-                                                         double *__restrict__ part) {
+                                                         double *__restrict__ part,
+                                                         double *__restrict__ out,
+                                                         unsigned int *counter) {
   gram_small_body<T>(n, pa, qb, rows_per, A, B, part, blockIdx.x);
+  if (!out) return;
+  __shared__ int s_last;
+  __shared__ double sums[256];
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(counter, 1u) == gridDim.x - 1u;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  constexpr int kLen = kSmallPQ * kSmallPQ, kSubs = 256 / kLen;
+  const int e = threadIdx.x % kLen, sub = threadIdx.x / kLen, len = pa * qb;
+  double v = 0.0;
+  if (e < len)
+    for (int c = sub; c < (int)gridDim.x; c += kSubs) v += ldcg(part + (long long)c * len + e);
+  sums[threadIdx.x] = v;
+  __syncthreads();
+  if (sub == 0 && e < len) {
+#pragma unroll
+    for (int s = 1; s < kSubs; ++s) v += sums[s * kLen + e];
+    out[e] = v;
+  }
+  if (threadIdx.x == 0) *counter = 0u;
 }
 
 // Pipelined FP32 Grams for 32 < max(pa, qb) <= 64 and 16-byte-aligned
@@ -549,10 +608,14 @@ ks_status launch_gram(Problem &P, const T *A, int pa, const T *B, int qb, double
   const size_t need = (size_t)chunks * pa * qb;
   if (need > P.partials_len)
     return set_error(KS_EINVAL, "gram: partial buffer too small (%zu > %zu)", need, P.partials_len);
+  // few chunks of a small Gram are summed by the last block (a launch less);
+  // many take too long in one block
+  const bool tail = pa <= kSmallPQ && qb <= kSmallPQ && chunks <= 128;
   {
     ProfScope ps_(P.stream, KP_GRAM, 2.0 * P.n * pa * qb, (double)P.n * (pa + qb) * sizeof(T));
     if (pa <= kSmallPQ && qb <= kSmallPQ)
-      gram_small_kernel<T><<<chunks, 256, 0, P.stream>>>(P.n, pa, qb, rows_per, A, B, P.partials);
+      gram_small_kernel<T><<<chunks, 256, 0, P.stream>>>(P.n, pa, qb, rows_per, A, B, P.partials,
+                                                         tail ? out : nullptr, P.red_counter);
     else if (pa <= kMidPQ && qb <= kMidPQ)
       gram_mid_kernel<T><<<chunks, 256, 0, P.stream>>>(P.n, pa, qb, rows_per, A, B, P.partials);
     else
@@ -560,6 +623,7 @@ ks_status launch_gram(Problem &P, const T *A, int pa, const T *B, int qb, double
                                                                 P.partials);
   }
   KS_CUDA_TRY(cudaGetLastError());
+  if (tail) return KS_OK;
   const long long len = (long long)pa * qb;
   {
     ProfScope ps_(P.stream, KP_REDUCE);

@@ -671,7 +671,7 @@ __device__ __forceinline__ double defect_update(const CgArgs &a, bool first, dou
 // still in r (a.incr) forms the new one without a stencil, r = r_old + (b -
 // b_old), from the right-hand side of the last solve (rho_prev).
 __device__ void cg_body(const CgArgs &a) {
-  __shared__ double smem[33];
+  __shared__ double smem[2 * 33];
   const int nb = a.vnb;
   unsigned int epoch = 0;
   double *partA = a.part, *partB = a.part + nb, *partC = a.part + 2 * nb, *partD = a.part + 3 * nb;
@@ -707,14 +707,18 @@ __device__ void cg_body(const CgArgs &a) {
     rr_l = fma(rk, rk, rr_l);
     bb_l = fma(b, b, bb_l);
   }
-  {
-    const double s1 = block_sum(rr_l, smem);
-    const double s2 = block_sum(bb_l, smem);
-    if (threadIdx.x == 0) { partB[a.vb] = s1; partD[a.vb] = s2; }
-  }
+  double rb[2] = {rr_l, bb_l};
+  block_sum_n<2>(rb, smem);
+  if (threadIdx.x == 0) { partB[a.vb] = rb[0]; partD[a.vb] = rb[1]; }
   if (!cg_barrier(a, epoch)) return;
-  double rr = block_sum_array(partB, nb, smem);
-  const double bb = block_sum_array(partD, nb, smem);
+  rb[0] = rb[1] = 0.0;
+  for (int i = threadIdx.x; i < nb; i += blockDim.x) {
+    rb[0] += ldcg(partB + i);
+    rb[1] += ldcg(partD + i);
+  }
+  block_sum_n<2>(rb, smem);
+  double rr = rb[0];
+  const double bb = rb[1];
   const double thr = a.tol * a.tol * bb;
   // a non-finite right-hand side or start makes every comparison below false
   bool bad = !isfinite(rr) || !isfinite(bb);

@@ -76,6 +76,34 @@ __device__ __forceinline__ double block_sum(double v, double *smem /* >= 33 */) 
   return r;
 }
 
+// The same for C <= 4 channels at once (blockDim.x >= 32 C; smem >= 33 C):
+// one exchange through shared memory instead of C, each channel summed in
+// block_sum's order.
+template <int C>
+__device__ __forceinline__ void block_sum_n(double (&v)[C], double *smem) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+    for (int c = 0; c < C; ++c) v[c] += __shfl_xor_sync(0xffffffffu, v[c], o);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int nw = blockDim.x >> 5;
+  __syncthreads();
+  if (lane == 0)
+#pragma unroll
+    for (int c = 0; c < C; ++c) smem[33 * c + warp] = v[c];
+  __syncthreads();
+  if (warp < C) {
+    double w = lane < nw ? smem[33 * warp + lane] : 0.0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+    if (lane == 0) smem[33 * warp + 32] = w;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int c = 0; c < C; ++c) v[c] = smem[33 * c + 32];
+  __syncthreads();
+}
+
 // Sum nb values src[0..nb) in a fixed order by the whole block (strided
 // partial sums in index order, then block_sum).  src may have been written
 // by other blocks of this launch, so it is read through L2.
@@ -85,14 +113,16 @@ __device__ __forceinline__ double block_sum_array(const double *src, int nb, dou
   return block_sum(acc, smem);
 }
 
-// Last-block reduction: every block has written its nchan partial sums to
+// Last-block reduction: every block has written its C partial sums to
 // part[c * nb + blockIdx.x] (thread 0); the block that arrives last sums
 // each channel over all blocks in index order (the same order whichever
 // block is last, so the result is deterministic), writes scale * sum to
-// out[c] and re-arms the counter for the next launch on the stream.
-__device__ __forceinline__ void grid_reduce_tail(const double *part, int nb, int nchan,
-                                                 double *out, double scale,
-                                                 unsigned int *counter, double *smem) {
+// out[c] and re-arms the counter for the next launch on the stream.  smem: 33 C
+// doubles.
+template <int C>
+__device__ __forceinline__ void grid_reduce_tail(const double *part, int nb, double *out,
+                                                 double scale, unsigned int *counter,
+                                                 double *smem) {
   __shared__ int s_last;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -103,11 +133,18 @@ __device__ __forceinline__ void grid_reduce_tail(const double *part, int nb, int
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  for (int c = 0; c < nchan; ++c) {
-    const double sacc = block_sum_array(part + (long long)c * nb, nb, smem);
-    if (threadIdx.x == 0) out[c] = scale * sacc;
+  double s[C];
+#pragma unroll
+  for (int c = 0; c < C; ++c) s[c] = 0.0;
+  for (int i = threadIdx.x; i < nb; i += blockDim.x)
+#pragma unroll
+    for (int c = 0; c < C; ++c) s[c] += ldcg(part + (long long)c * nb + i);
+  block_sum_n<C>(s, smem);
+  if (threadIdx.x == 0) {
+#pragma unroll
+    for (int c = 0; c < C; ++c) out[c] = scale * s[c];
+    *counter = 0u;
   }
-  if (threadIdx.x == 0) *counter = 0u;
 }
 
 // Polls of a grid-barrier wait before the waiting thread starts to sleep.

@@ -232,7 +232,7 @@ template <typename T, int PC, int Kind>
 __device__ __forceinline__ void stencil_plain_body(const StArgs &a, int vb) {
   using Tl = StTile<PC>;
   __shared__ T tile[Tl::HY * Tl::HX * PC];
-  __shared__ double smem[33];
+  __shared__ double smem[Kind == SK_MASS_BB ? 4 * 33 : 33];
   const int N = a.N, p = a.p;
   // block -> (tile x, tile y, orbital chunk, z segment)
   int b = vb;
@@ -351,21 +351,19 @@ __device__ __forceinline__ void stencil_plain_body(const StArgs &a, int vb) {
   }
   if (Kind == SK_MASS) return;
   if (Kind == SK_HAM && StCols<T, Kind>::kNew) acc0 *= cf.ke;
-  const double s0 =
-      block_sum(Kind == SK_HAM_INC ? (double)acc0 - (double)acc1 : (double)acc0, smem);
-  if (threadIdx.x == 0) a.part[vb] = s0;
-  if (Kind == SK_MASS_BB) {
-    const double s1 = block_sum((double)acc1, smem);
-    const double s2 = block_sum((double)acc2, smem);
-    const double s3 = block_sum((double)acc3, smem);
-    if (threadIdx.x == 0) {
-      a.part[a.nb + vb] = s1;
-      a.part[2 * a.nb + vb] = s2;
-      a.part[3 * a.nb + vb] = s3;
-    }
+  if constexpr (Kind == SK_MASS_BB) {
+    double s[4] = {(double)acc0, (double)acc1, (double)acc2, (double)acc3};
+    block_sum_n<4>(s, smem);
+    if (threadIdx.x == 0)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) a.part[i * a.nb + vb] = s[i];
+  } else {
+    const double s0 =
+        block_sum(Kind == SK_HAM_INC ? (double)acc0 - (double)acc1 : (double)acc0, smem);
+    if (threadIdx.x == 0) a.part[vb] = s0;
   }
-  grid_reduce_tail(a.part, a.nb, Kind == SK_MASS_BB ? 4 : 1, a.red_out, a.red_scale, a.counter,
-                   smem);
+  grid_reduce_tail<Kind == SK_MASS_BB ? 4 : 1>(a.part, a.nb, a.red_out, a.red_scale, a.counter,
+                                               smem);
 }
 
 template <typename T, int PC, int Kind>
@@ -419,7 +417,7 @@ __global__ void __launch_bounds__(kStThreads, 2) stencil_tma_kernel(const __grid
   // SK_HAM_INC: V_b and V - V_b (formed in FP64) of the same planes
   __shared__ T vbs[Kind == SK_HAM_INC ? 3 : 1][Kind == SK_HAM_INC ? TXY : 1];
   __shared__ T dvs[Kind == SK_HAM_INC ? 3 : 1][Kind == SK_HAM_INC ? TXY : 1];
-  __shared__ double smem[33];
+  __shared__ double smem[Kind == SK_MASS_BB ? 4 * 33 : 33];
   const StArgs &a = ta.a;
   const int N = a.N, p = a.p;
   int b = blockIdx.x;
@@ -603,21 +601,19 @@ __global__ void __launch_bounds__(kStThreads, 2) stencil_tma_kernel(const __grid
   }
   if (Kind == SK_MASS) return;
   if (Kind == SK_HAM && StCols<T, Kind>::kNew) acc0 *= cf.ke;
-  const double s0 =
-      block_sum(Kind == SK_HAM_INC ? (double)acc0 - (double)acc1 : (double)acc0, smem);
-  if (threadIdx.x == 0) a.part[blockIdx.x] = s0;
-  if (Kind == SK_MASS_BB) {
-    const double s1 = block_sum((double)acc1, smem);
-    const double s2 = block_sum((double)acc2, smem);
-    const double s3 = block_sum((double)acc3, smem);
-    if (threadIdx.x == 0) {
-      a.part[a.nb + blockIdx.x] = s1;
-      a.part[2 * a.nb + blockIdx.x] = s2;
-      a.part[3 * a.nb + blockIdx.x] = s3;
-    }
+  if constexpr (Kind == SK_MASS_BB) {
+    double s[4] = {(double)acc0, (double)acc1, (double)acc2, (double)acc3};
+    block_sum_n<4>(s, smem);
+    if (threadIdx.x == 0)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) a.part[i * a.nb + blockIdx.x] = s[i];
+  } else {
+    const double s0 =
+        block_sum(Kind == SK_HAM_INC ? (double)acc0 - (double)acc1 : (double)acc0, smem);
+    if (threadIdx.x == 0) a.part[blockIdx.x] = s0;
   }
-  grid_reduce_tail(a.part, a.nb, Kind == SK_MASS_BB ? 4 : 1, a.red_out, a.red_scale, a.counter,
-                   smem);
+  grid_reduce_tail<Kind == SK_MASS_BB ? 4 : 1>(a.part, a.nb, a.red_out, a.red_scale, a.counter,
+                                               smem);
 }
 
 // ---------------------------------------------------------------- FP32, p >= 32
@@ -656,7 +652,7 @@ __global__ void __launch_bounds__(kStThreads, Kind == SK_MASS_BB ? 1 : 2)
   __shared__ float vs[kHam ? 3 : 1][kHam ? TXY : 1];
   __shared__ float vbs[Kind == SK_HAM_INC ? 3 : 1][Kind == SK_HAM_INC ? TXY : 1];
   __shared__ float dvs[Kind == SK_HAM_INC ? 3 : 1][Kind == SK_HAM_INC ? TXY : 1];
-  __shared__ double smem[33];
+  __shared__ double smem[Kind == SK_MASS_BB ? 4 * 33 : 33];
   const StArgs &a = ta.a;
   const int N = a.N, p = a.p;
   int b = blockIdx.x;
@@ -838,18 +834,21 @@ __global__ void __launch_bounds__(kStThreads, Kind == SK_MASS_BB ? 1 : 2)
     for (int i = 0; i < 4; ++i) acc[i] = 0ull;
   }
   if (Kind == SK_MASS) return;
-  const double s0 = block_sum(
-      Kind == SK_HAM_INC ? f2_sum(acc[0]) - f2_sum(acc[1]) : f2_sum(acc[0]), smem);
-  if (threadIdx.x == 0) a.part[blockIdx.x] = s0;
-  if (Kind == SK_MASS_BB) {
+  if constexpr (Kind == SK_MASS_BB) {
+    double s[4];
 #pragma unroll
-    for (int i = 1; i < 4; ++i) {
-      const double s = block_sum(f2_sum(acc[i]), smem);
-      if (threadIdx.x == 0) a.part[i * a.nb + blockIdx.x] = s;
-    }
+    for (int i = 0; i < 4; ++i) s[i] = f2_sum(acc[i]);
+    block_sum_n<4>(s, smem);
+    if (threadIdx.x == 0)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) a.part[i * a.nb + blockIdx.x] = s[i];
+  } else {
+    const double s0 = block_sum(
+        Kind == SK_HAM_INC ? f2_sum(acc[0]) - f2_sum(acc[1]) : f2_sum(acc[0]), smem);
+    if (threadIdx.x == 0) a.part[blockIdx.x] = s0;
   }
-  grid_reduce_tail(a.part, a.nb, Kind == SK_MASS_BB ? 4 : 1, a.red_out, a.red_scale, a.counter,
-                   smem);
+  grid_reduce_tail<Kind == SK_MASS_BB ? 4 : 1>(a.part, a.nb, a.red_out, a.red_scale, a.counter,
+                                               smem);
 }
 
 // Geometry of a launch: tiles, orbital chunks and z segments; the number of

@@ -3,6 +3,8 @@
 // h^3 sum rho eps_xc(rho), and V_eff = Vext + vH + v_xc with
 // v_xc = d(rho eps_xc)/d rho.  LDA = Slater exchange, optionally with the
 // Perdew-Zunger (1981) correlation of the unpolarised electron gas.
+#include <algorithm>
+
 #include "ks_device.cuh"
 
 namespace ks {
@@ -138,8 +140,8 @@ __device__ __forceinline__ void tf_point(double rho_d, R z, R ctf, R vtf, R &e, 
   e = ctf * rho * r23;
 }
 
-// Channels of the block partials: 0 = E_ext, 1 = E_H, 2 = E_xc and, when
-// ctf != 0 (orbital-free model), 3 = E_TF, with v_TF added to V_eff.  Block
+// Channels of the block partials: 0 = E_ext, 1 = E_H, 2 = E_xc, 3 = E_TF (0
+// unless ctf != 0, the orbital-free model, with v_TF added to V_eff).  Block
 // vb of vnb (grid-stride over the n nodes); the last block to finish sums
 // the partials in block order.
 template <typename R>
@@ -152,7 +154,7 @@ __device__ __forceinline__ void potential_body(long long n, double h3, int xc, i
                                                double *__restrict__ veff, double *__restrict__ part,
                                                double *__restrict__ out, unsigned int *counter,
                                                int vb, int vnb) {
-  __shared__ double smem[33];
+  __shared__ double smem[4 * 33];
   const double inv8pi = 1.0 / (8.0 * M_PI);
   const R ctf_r = (R)ctf, vtf_r = (R)(ctf * (5.0 / 3.0));
   double e_ext = 0.0, e_h = 0.0, e_xc = 0.0, e_tf = 0.0;
@@ -178,18 +180,12 @@ __device__ __forceinline__ void potential_body(long long n, double h3, int xc, i
     }
     veff[k] = v;
   }
-  const double s0 = block_sum(e_ext, smem);
-  const double s1 = block_sum(e_h, smem);
-  const double s2 = block_sum(e_xc, smem);
-  const int nchan = ctf != 0.0 ? 4 : 3;
-  const double s3 = nchan == 4 ? block_sum(e_tf, smem) : 0.0;
-  if (threadIdx.x == 0) {
-    part[vb] = s0;
-    part[vnb + vb] = s1;
-    part[2 * vnb + vb] = s2;
-    if (nchan == 4) part[3 * vnb + vb] = s3;
-  }
-  grid_reduce_tail(part, vnb, nchan, out, 1.0, counter, smem);
+  double s[4] = {e_ext, e_h, e_xc, e_tf};
+  block_sum_n<4>(s, smem);
+  if (threadIdx.x == 0)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) part[c * vnb + vb] = s[c];
+  grid_reduce_tail<4>(part, vnb, out, 1.0, counter, smem);
 }
 
 template <typename R>
@@ -258,7 +254,10 @@ ks_status launch_reduce(Problem &P, const double *partials, int nchan, int nb, d
 
 ks_status launch_potential(Problem &P, const double *rho, const double *vH, const double *r,
                            double *veff, bool with_hartree, bool fp32_xc) {
-  const int nb = reduce_blocks(P, P.n);
+  // at most two blocks per SM: a block ends in four FP64 sums, as much work for
+  // the FP64 pipe as a third of a node per thread, and the last one sums all
+  // blocks' partials (1024 blocks of one node per thread took 53 us at 64^3)
+  const int nb = std::min(reduce_blocks(P, P.n), 2 * P.sms);
   const double h3 = P.h * P.h * P.h;
   {
     ProfScope ps_(P.stream, KP_POTENTIAL, 40.0 * P.n, 40.0 * P.n);
