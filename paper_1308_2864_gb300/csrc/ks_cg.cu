@@ -23,7 +23,8 @@
 // passes.  What bounds a solve is the chain of phases: a barrier costs 2.5 to
 // 4 us, a transform phase its loads' latency, the update the FP64 pipe.
 // Measured, PCG with full transforms -> this form: warm solve at 64^3 172 ->
-// 106 us, at 105^3 519 -> 299 us; cold at 81^3 463 -> 180 us; 24^3 80 -> 63 us.
+// 104 us, at 105^3 519 -> 293 us; cold at 81^3 463 -> 177 us; 24^3 80 -> 63 us
+// (of which packed FMAs in the transforms' tiles 2 to 6 us).
 //
 // Each step's reductions are partial sums written per block and summed by
 // every block in the same order, so all blocks take identical branch
@@ -312,20 +313,39 @@ __device__ __forceinline__ void ldv(const float *p, float (&v)[TT]) {
   }
 }
 
-// acc[u][v] += sum_k A[k][m0 + u] B[k][n0 + v] (row strides lda, ldb)
+// acc[u][v] = sum_k A[k][m0 + u] B[k][n0 + v] (row strides lda, ldb); packed
+// FMAs over the columns (f2_fma), each a chain over ascending k.
 template <int TT>
 __device__ __forceinline__ void tile_fma(const float *A, int lda, const float *B, int ldb, int K,
                                          float (&acc)[TT][TT]) {
+  f2_t c[TT][TT / 2];
+#pragma unroll
+  for (int u = 0; u < TT; ++u)
+#pragma unroll
+    for (int v = 0; v < TT / 2; ++v) c[u][v] = 0ull;
 #pragma unroll 4
   for (int k = 0; k < K; ++k) {
-    float av[TT], bv[TT];
+    float av[TT];
+    f2_t bv[TT / 2];
     ldv<TT>(A + k * lda, av);
-    ldv<TT>(B + k * ldb, bv);
+    if constexpr (TT == 4) {
+      const ulonglong2 q = *reinterpret_cast<const ulonglong2 *>(B + k * ldb);
+      bv[0] = q.x;
+      bv[1] = q.y;
+    } else {
+      bv[0] = *reinterpret_cast<const f2_t *>(B + k * ldb);
+    }
 #pragma unroll
-    for (int u = 0; u < TT; ++u)
+    for (int u = 0; u < TT; ++u) {
+      const f2_t a2 = f2_dup(av[u]);
 #pragma unroll
-      for (int v = 0; v < TT; ++v) acc[u][v] = fmaf(av[u], bv[v], acc[u][v]);
+      for (int v = 0; v < TT / 2; ++v) c[u][v] = f2_fma(a2, bv[v], c[u][v]);
+    }
   }
+#pragma unroll
+  for (int u = 0; u < TT; ++u)
+#pragma unroll
+    for (int v = 0; v < TT / 2; ++v) f2_split(c[u][v], acc[u][2 * v], acc[u][2 * v + 1]);
 }
 
 // out(m0, n0, acc) for every TT x TT tile of C = A^T B (M x Nn, K terms), both
@@ -339,10 +359,6 @@ __device__ __forceinline__ void tile_gemm(int M, int Nn, int K, const float *A, 
     const int m0 = t / tn * TT, n0 = t % tn * TT;
     if (!KS_IN(m0 + TT - 1, lda) || !KS_IN(n0 + TT - 1, ldb)) continue;
     float acc[TT][TT];
-#pragma unroll
-    for (int u = 0; u < TT; ++u)
-#pragma unroll
-      for (int v = 0; v < TT; ++v) acc[u][v] = 0.f;
     tile_fma<TT>(A + m0, lda, B + n0, ldb, K, acc);
     out(m0, n0, acc);
   }
@@ -358,10 +374,6 @@ __device__ __forceinline__ void tile_gemm2(int M, int Nn, int K1, const float *A
     const int m0 = t / tn * TT, n0 = t % tn * TT;
     if (!KS_IN(m0 + TT - 1, lda) || !KS_IN(n0 + TT - 1, ldb)) continue;
     float e[TT][TT], o[TT][TT];
-#pragma unroll
-    for (int u = 0; u < TT; ++u)
-#pragma unroll
-      for (int v = 0; v < TT; ++v) e[u][v] = o[u][v] = 0.f;
     tile_fma<TT>(A1 + m0, lda, B1 + n0, ldb, K1, e);
     tile_fma<TT>(A2 + m0, lda, B2 + n0, ldb, K2, o);
     out(m0, n0, e, o);
@@ -553,10 +565,6 @@ __device__ __forceinline__ void fused_pass_c(const CgArgs &a, const float *in, d
     for (int t = threadIdx.x; t < tiles; t += kCgThreads) {
       const int m0 = t / tn * TT, n0 = t % tn * TT;
       float e[TT][TT], o[TT][TT];
-#pragma unroll
-      for (int u = 0; u < TT; ++u)
-#pragma unroll
-        for (int v = 0; v < TT; ++v) e[u][v] = o[u][v] = 0.f;
       tile_fma<TT>(Yt + m0, ldy, d.ie + n0, hp, d.h1, e);
       tile_fma<TT>(Yt + d.h1 * ldy + m0, ldy, d.io + n0, hp, d.h0, o);
 #pragma unroll
