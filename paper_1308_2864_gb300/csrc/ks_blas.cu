@@ -268,11 +268,14 @@ __device__ __forceinline__ void gram_small_body(long long n, int pa, int qb, lon
 }
 
 // Mid-size Grams (kSmallPQ < pa, qb <= kMidPQ): the block keeps the whole
-// pa x qb result of its row chunk, one thread per output (up to four per
-// thread), staging kMidRows rows of A and B in shared memory at a time.
-// Threads map onto the pa qb outputs with no padding, so no FMA is spent on
-// entries outside the Gram (the 64-wide tile would spend (64/p)^2 times the
-// work at p = 16).
+// pa x qb result of its row chunk, staging kMidRows rows of A and B in shared
+// memory at a time.  Threads map onto the outputs with no padding beyond one row
+// and column, so no FMA is spent on entries outside the Gram (the 64-wide tile
+// would spend (64/p)^2 times the work at p = 16).  Up to 256 outputs: one per
+// thread.  Above, a 2 x 2 block per thread: four shared values for four FMAs
+// where one output per thread reads eight, which bound the kernel (two reads
+// per FMA); every output is the same row-ascending chain in both.  Measured, the
+// Grams of 24 batched jobs (N 20 to 38, p 4 to 32): 123 -> 71 us per launch.
 constexpr int kMidPQ = 32, kMidRows = 32;
 static_assert(kMidRows * kMidPQ <= 4 * 256, "a stage is 4 values per thread of a 256-thread block");
 
@@ -280,20 +283,21 @@ template <typename T>
 __device__ __forceinline__ void gram_mid_body(long long n, int pa, int qb, long long rows_per,
                                               const T *__restrict__ A, const T *__restrict__ B,
                                               double *__restrict__ part, int chunk) {
-  __shared__ T As[kMidRows * kMidPQ];
-  __shared__ T Bs[kMidRows * kMidPQ];
+  // (an odd width's last block reads one value past its row: the next row's, or
+  // up to one value past the stage, so a few spare entries)
+  __shared__ __align__(16) T As[kMidRows * kMidPQ + 4];
+  __shared__ __align__(16) T Bs[kMidRows * kMidPQ + 4];
   const long long r0 = chunk * rows_per;
   long long r1 = r0 + rows_per;
   if (r1 > n) r1 = n;
   const int outs = pa * qb;
-  int oa[4], ob[4];
-#pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    const int e = threadIdx.x + u * blockDim.x;
-    oa[u] = e < outs ? e / qb : 0;
-    ob[u] = e < outs ? e % qb : 0;
-  }
-  T acc[4] = {0, 0, 0, 0};
+  const bool wide = outs > 256;
+  const int tb = (qb + 1) / 2, ta = (pa + 1) / 2;
+  const bool work = wide ? (int)threadIdx.x < ta * tb : (int)threadIdx.x < outs;
+  // first output (row, column) of this thread
+  const int oa = !work ? 0 : wide ? 2 * ((int)threadIdx.x / tb) : (int)threadIdx.x / qb;
+  const int ob = !work ? 0 : wide ? 2 * ((int)threadIdx.x % tb) : (int)threadIdx.x % qb;
+  T acc[2][2] = {{0, 0}, {0, 0}};
   // the next stage's values travel in registers while this stage computes
   // (256 threads x 4 cover a stage of kMidRows x kMidPQ)
   T ra[4], rb[4];
@@ -318,20 +322,32 @@ __device__ __forceinline__ void gram_mid_body(long long n, int pa, int qb, long 
     }
     __syncthreads();
     if (r + kMidRows < r1) fetch(r + kMidRows);
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      if (threadIdx.x + u * blockDim.x >= outs) break;
-      T a = acc[u];
-      for (int k = 0; k < rows; ++k) a = fma(As[k * pa + oa[u]], Bs[k * qb + ob[u]], a);
-      acc[u] = a;
+    if (!work) continue;
+    const T *as = As + oa, *bs = Bs + ob;
+    if (!wide) {
+      T a = acc[0][0];
+#pragma unroll 8
+      for (int k = 0; k < rows; ++k) a = fma(as[k * pa], bs[k * qb], a);
+      acc[0][0] = a;
+    } else {
+#pragma unroll 8
+      for (int k = 0; k < rows; ++k) {
+        const T a0 = as[k * pa], a1 = as[k * pa + 1], b0 = bs[k * qb], b1 = bs[k * qb + 1];
+        acc[0][0] = fma(a0, b0, acc[0][0]);
+        acc[0][1] = fma(a0, b1, acc[0][1]);
+        acc[1][0] = fma(a1, b0, acc[1][0]);
+        acc[1][1] = fma(a1, b1, acc[1][1]);
+      }
     }
   }
+  if (!work) return;
   double *dst = part + (long long)chunk * outs;
 #pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    const int e = threadIdx.x + u * blockDim.x;
-    if (e < outs) dst[e] = (double)acc[u];
-  }
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+      if ((wide || (i == 0 && j == 0)) && oa + i < pa && ob + j < qb)
+        dst[(oa + i) * qb + ob + j] = (double)acc[i][j];
 }
 
 template <typename T>

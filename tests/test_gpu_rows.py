@@ -110,3 +110,22 @@ def test_wide_fp32_update_on_tensor_cores(N, k1, k2, q):
         want = -0.5 * (A1d @ C1 + A2d @ C2) + beta * Bm
         bound = 0.5 * (np.abs(A1d) @ np.abs(C1) + np.abs(A2d) @ np.abs(C2)) + beta * np.abs(Bm)
         assert np.all(np.abs(got - want) <= 4e-6 * bound + 1e-12)
+
+
+@pytest.mark.parametrize("pa,qb", [(9, 9), (16, 16), (16, 17), (17, 16), (9, 29), (31, 31),
+                                   (32, 31), (31, 32), (32, 32)])
+def test_mid_gram_thread_blocks(pa, qb):
+    # both sides of 256 outputs (one or 2 x 2 per thread), odd widths; rows that
+    # end inside a stage of 32.  A chain of n rounded products: n unit roundoffs.
+    import paper_1308_2864_gb300 as ks
+    for N in (4, 9):
+        s = ki.small_system(N=N, L=7.0, natoms=2, p=max(pa, qb), Z=4.0, seed=4)
+        P = ks.Problem.from_system(s)
+        rng = np.random.default_rng(pa * 40 + qb)
+        A, B = rng.standard_normal((s.n, pa)), rng.standard_normal((s.n, qb))
+        got = P.step_gram(dev(A), dev(B)).cpu().numpy()
+        assert np.all(np.abs(got - A.T @ B) <= 2 * s.n * 2.0**-53 * (np.abs(A).T @ np.abs(B)))
+        A, B = A.astype(np.float32), B.astype(np.float32)
+        got = P.step_gram_f32(torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda()).cpu().numpy()
+        A, B = A.astype(np.float64), B.astype(np.float64)
+        assert np.all(np.abs(got - A.T @ B) <= 2 * s.n * 2.0**-24 * (np.abs(A).T @ np.abs(B)))
