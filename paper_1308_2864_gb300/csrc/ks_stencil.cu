@@ -227,7 +227,12 @@ struct StCols {
 
 // Plain-load form of one block (vb = the block's index in the system's
 // launch geometry); the single-system kernel and the batched kernel of a
-// job table both run it.
+// job table both run it.  Latency of the walk bounds it, so everything a plane
+// reads from memory is in flight before its sums: the next halo box and the
+// node-local inputs, which (left at their use, behind the stores of the node
+// before) waited four times per plane.  Measured, FP32 stencils of 24 batched
+// jobs (N 20 to 38, p 4 to 32): E_X 48 -> 34 us per launch, M D with the BB traces and
+// the mass products 79 -> 53 us; M x of 105^3 x 1 in FP64 51 -> 37 us.
 template <typename T, int PC, int Kind>
 __device__ __forceinline__ void stencil_plain_body(const StArgs &a, int vb) {
   using Tl = StTile<PC>;
@@ -260,19 +265,22 @@ __device__ __forceinline__ void stencil_plain_body(const StArgs &a, int vb) {
   constexpr int kBox = Tl::HY * Tl::HX * PC;
   constexpr int kPf = (kBox + kStThreads - 1) / kStThreads;
   T pf[kPf];
+  // where each of them lies within a plane (-1: outside the grid), formed once
+  // instead of in every plane
+  int off[kPf];
+#pragma unroll
+  for (int i = 0; i < kPf; ++i) {
+    const int t = threadIdx.x + i * kStThreads;
+    const int l = t % PC, hn = t / PC;
+    const int gx = x0 + hn % Tl::HX - 1, gy = y0 + hn / Tl::HX - 1, go = oc * PC + l;
+    off[i] = t < kBox && gx >= 0 && gx < N && gy >= 0 && gy < N && go < p
+                 ? (gy * N + gx) * p + go : -1;
+  }
   auto fetch = [&](int zp) {
+    const T *Az = A + (long long)zp * N * N * p;
     const bool zok = zp >= 0 && zp < N;
 #pragma unroll
-    for (int i = 0; i < kPf; ++i) {
-      const int t = threadIdx.x + i * kStThreads;
-      const int l = t % PC, hn = t / PC;
-      const int hx = hn % Tl::HX, hy = hn / Tl::HX;
-      const int gx = x0 + hx - 1, gy = y0 + hy - 1, go = oc * PC + l;
-      T v = 0;
-      if (t < kBox && zok && gx >= 0 && gx < N && gy >= 0 && gy < N && go < p)
-        v = __ldg(A + (((long long)zp * N + gy) * N + gx) * p + go);
-      pf[i] = v;
-    }
+    for (int i = 0; i < kPf; ++i) pf[i] = zok && off[i] >= 0 ? __ldg(Az + off[i]) : (T)0;
   };
   auto plane = [&]() {
     __syncthreads();
@@ -299,29 +307,56 @@ __device__ __forceinline__ void stencil_plain_body(const StArgs &a, int vb) {
   if (z0 < z1) fetch(z0 + 1);
 
   T acc0 = 0, acc1 = 0, acc2 = 0, acc3 = 0;
+  // this thread's entries within a plane (-1: none)
+  int ent[kStNodesPerThread];
+#pragma unroll
+  for (int r = 0; r < kStNodesPerThread; ++r) {
+    const int gx = x0 + lx[r], gy = y0 + ly[r];
+    ent[r] = ovalid && gx < N && gy < N ? gy * N + gx : -1;
+  }
 
   for (int z = z0; z < z1; ++z) {
+    const long long zb = (long long)z * N * N, nodes = (long long)N * N * N;
+    // the node-local inputs of plane z, all in flight at once: left at their use
+    // they would wait for each other behind the stores of the node before
+    double va[kStNodesPerThread];
+    T bb[6][kStNodesPerThread];
+    auto locals = [&]() {
+#pragma unroll
+      for (int r = 0; r < kStNodesPerThread; ++r) {
+        const long long k = zb + ent[r], idx = k * p + o;
+        const bool in = ent[r] >= 0 && KS_IN(k, nodes) && KS_IN(idx, nodes * p);
+        if (Kind == SK_HAM || Kind == SK_HAM_INC) va[r] = in ? a.veff[k] : 0.0;
+        if (Kind == SK_MASS_BB) {
+          bb[0][r] = in ? ((const T *)a.X)[idx] : (T)0;
+          bb[1][r] = in ? ((const T *)a.Xp)[idx] : (T)0;
+          bb[2][r] = in ? ((const T *)a.MX)[idx] : (T)0;
+          bb[3][r] = in ? ((const T *)a.MXp)[idx] : (T)0;
+          bb[4][r] = in ? ((const T *)a.Dp)[idx] : (T)0;
+          bb[5][r] = in ? ((const T *)a.MDp)[idx] : (T)0;
+        }
+      }
+    };
+    constexpr bool kEarly = sizeof(T) == 4;        // FP64: registers
+    if (kEarly) locals();
     plane();                                       // plane z + 1
     if (z + 1 < z1) fetch(z + 2);                  // in flight during the outputs of plane z
+    if (!kEarly) locals();
 #pragma unroll
     for (int r = 0; r < kStNodesPerThread; ++r) {
-      const int gx = x0 + lx[r], gy = y0 + ly[r];
       const T centre = sc.c_mid[r];
-      const long long nodes = (long long)N * N * N;
-      if (ovalid && gx < N && gy < N && KS_IN(((long long)z * N + gy) * N + gx, nodes) &&
-          KS_IN((((long long)z * N + gy) * N + gx) * p + o, nodes * p)) {
-        const long long k = ((long long)z * N + gy) * N + gx;
-        const long long idx = k * p + o;
+      const long long k = zb + ent[r], idx = k * p + o;
+      if (ent[r] >= 0 && KS_IN(k, nodes) && KS_IN(idx, nodes * p)) {
         const T m = want_m ? sc.mass(r, cf) : (T)0;
         if (Kind == SK_HAM) {
           const T kx = sc.stiff(r, cf);
-          if (sizeof(T) == 4 || a.out1) ((T *)a.out1)[idx] = fma(cf.kin, kx, cf.vscale * (T)a.veff[k] * centre);
+          if (sizeof(T) == 4 || a.out1) ((T *)a.out1)[idx] = fma(cf.kin, kx, cf.vscale * (T)va[r] * centre);
           if (a.out2) ((T *)a.out2)[idx] = m;
           acc0 = fma(centre, kx, acc0);
         } else if (Kind == SK_HAM_INC) {
           const T kx = sc.stiff(r, cf);
           const T xb = ((const T *)a.X)[idx], eb = ((const T *)a.MX)[idx];
-          const T v = (T)a.veff[k], vb = (T)a.veff_b[k], dv = (T)(a.veff[k] - a.veff_b[k]);
+          const T v = (T)va[r], vb = (T)a.veff_b[k], dv = (T)(va[r] - a.veff_b[k]);
           ((T *)a.out1)[idx] = cf.kin * kx + cf.vscale * (dv * xb + v * centre);
           if (a.out2) ((T *)a.out2)[idx] = m;
           // compensated sum of delta . (2 f K X_b + f K delta); acc1 holds the
@@ -336,10 +371,10 @@ __device__ __forceinline__ void stencil_plain_body(const StArgs &a, int vb) {
           if (Kind != SK_MASS_DOT || sizeof(T) == 4 || a.out1) ((T *)a.out1)[idx] = m;
           if (Kind >= SK_MASS_DOT) acc0 = fma(centre, m, acc0);
           if (Kind == SK_MASS_BB) {
-            const T dx = ((const T *)a.X)[idx] - ((const T *)a.Xp)[idx];
-            const T dmx = ((const T *)a.MX)[idx] - ((const T *)a.MXp)[idx];
-            const T dd = centre - ((const T *)a.Dp)[idx];
-            const T dmd = m - ((const T *)a.MDp)[idx];
+            const T dx = bb[0][r] - bb[1][r];
+            const T dmx = bb[2][r] - bb[3][r];
+            const T dd = centre - bb[4][r];
+            const T dmd = m - bb[5][r];
             acc1 = fma(dx, dmx, acc1);
             acc2 = fma(dx, dmd, acc2);
             acc3 = fma(dd, dmd, acc3);
@@ -366,8 +401,16 @@ __device__ __forceinline__ void stencil_plain_body(const StArgs &a, int vb) {
                                                smem);
 }
 
+// Resident blocks that the plain-load kernels are compiled for: the walk over
+// the planes is latency, and FP64 at one block per SM (over 128 registers) or
+// the short FP32 kinds at two leave the SM idle between a plane's loads and use.
+template <typename T, int Kind>
+constexpr int st_min_blocks() {
+  return sizeof(T) == 4 && (Kind == SK_MASS || Kind == SK_MASS_DOT) ? 3 : 2;
+}
+
 template <typename T, int PC, int Kind>
-__global__ void __launch_bounds__(kStThreads) stencil_kernel(StArgs a) {
+__global__ void __launch_bounds__(kStThreads, (st_min_blocks<T, Kind>())) stencil_kernel(StArgs a) {
   stencil_plain_body<T, PC, Kind>(a, blockIdx.x);
 }
 
@@ -1115,7 +1158,7 @@ struct StSlots {
 };
 
 template <typename T, int PC, int Kind>
-__global__ void __launch_bounds__(kStThreads) stencil_batch_kernel(
+__global__ void __launch_bounds__(kStThreads, (st_min_blocks<T, Kind>())) stencil_batch_kernel(
     const BJob *__restrict__ jobs, const int *__restrict__ start, int J,
     const unsigned char *__restrict__ active, StSlots sl) {
   const int j = batch_job_of(start, J, blockIdx.x);
