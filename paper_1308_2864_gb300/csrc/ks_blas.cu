@@ -794,17 +794,153 @@ __global__ void __launch_bounds__(256) combine_kernel(long long n, int q, const 
                            blockIdx.y);
 }
 
-// Narrow updates (q <= kNarrowQ): one thread per output entry, the small
-// C matrices in shared memory, no padded arithmetic.
+// Narrow updates (q <= kNarrowQ): a thread takes 4 consecutive columns, the small
+// C matrices in shared memory, no padded arithmetic.  FP64, bound by its pipe:
+// one row per thread, A read from L1.  FP32: combine_rows_body.
 constexpr int kNarrowQ = 32;
 constexpr int kNarrowK = 2 * kNarrowQ;
 constexpr int kNarrowCols = 4;                     // output columns per thread
+
+// FP32 form: 4 rows x 4 columns per thread.  A tile's rows (as many as the
+// threads cover; 144 at q = 26) are staged up to 32 columns at a time, read and
+// written as contiguous memory; four k of A and of C are one 16-byte shared read
+// each, 8 reads for 64 FMAs (one row per thread and scalar reads: 5 per 4), and
+// the rounding of C to FP32, on the FP64 pipe, is per tile of rows instead of per
+// 1024 outputs.  Rows of a thread lie `groups` apart: a warp's groups read
+// consecutive rows, whose odd multiple of 16 bytes misses no bank.  Every output
+// keeps its chain over k and its last step.  Measured, 24 batched jobs (N 20 to
+// 38, p 4 to 32): 119 -> 93 us per update of one or two blocks.  What is left is
+// latency: a tile loads, computes and writes in turn, four blocks to an SM.
+constexpr int kNrK = 32;                           // columns of A per stage
+constexpr int kNrStage = 6144;                     // floats of a stage: 1024 rows x 4 .. 128 x 36
+
+__device__ __forceinline__ int nr_pitch(int kc) {  // odd multiple of 4 floats
+  const int v = (kc + 3) / 4;
+  return 4 * (v | 1);
+}
+
+__device__ __forceinline__ void combine_rows_body(
+    long long n, int q, const float *__restrict__ A1, int k1, const double *__restrict__ C1,
+    const float *__restrict__ A2, int k2, const double *__restrict__ C2, float alpha, float beta,
+    const float *__restrict__ Bm, float *__restrict__ out, int vb, int vnb) {
+  __shared__ __align__(16) float Cs[2 * kNarrowK * kNarrowQ];
+  __shared__ __align__(16) float As[kNrStage];
+  const int K = k1 + (A2 ? k2 : 0);
+  const int ncg = (q + 3) / 4, ldc = 4 * ncg;
+  const int groups = min(256 / ncg, kNrStage / (4 * nr_pitch(min(max(k1, A2 ? k2 : 0), kNrK))));
+  const int tr = 4 * groups;                       // rows of a tile
+  const long long ntiles = (n + tr - 1) / tr;
+  if (vb >= ntiles) return;
+  for (int e = threadIdx.x; e < K * ldc; e += blockDim.x) {
+    const int k = e / ldc, c = e - k * ldc;
+    Cs[e] = c >= q ? 0.f : (float)(k < k1 ? C1[k * q + c] : C2[(k - k1) * q + c]);
+  }
+  const int g = threadIdx.x / ncg, col0 = 4 * (threadIdx.x % ncg);
+  const bool work = g < groups;
+  for (long long t = vb; t < ntiles; t += vnb) {
+    const long long r0 = t * tr;
+    const int rows = (int)min((long long)tr, n - r0);
+    float acc[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int u = 0; u < 4; ++u) acc[i][u] = 0.f;
+    for (int s = 0; s < (A2 ? 2 : 1); ++s) {
+      const int ks = s ? k2 : k1;
+      const float *A = (s ? A2 : A1) + r0 * ks;
+      for (int kb = 0; kb < ks; kb += kNrK) {
+        const int kc = min(kNrK, ks - kb), ld = nr_pitch(kc);
+        __syncthreads();                           // (the stage, and Cs the first time)
+        // element e = row kc + k of the stage, advanced without a division
+        const int dr = 256 / kc, dk = 256 - dr * kc;
+        int row = threadIdx.x / kc, k = threadIdx.x - row * kc;
+        const int cnt = rows * kc;
+        for (int e0 = threadIdx.x; e0 < cnt; e0 += 8 * 256) {
+          float v[8];
+          int at[8];
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            const bool in = e0 + u * 256 < cnt;
+            at[u] = in ? row * ld + k : -1;
+            v[u] = in ? A[(long long)row * ks + kb + k] : 0.f;
+            row += dr;
+            k += dk;
+            if (k >= kc) {
+              k -= kc;
+              ++row;
+            }
+          }
+#pragma unroll
+          for (int u = 0; u < 8; ++u)
+            if (at[u] >= 0) As[at[u]] = v[u];
+        }
+        __syncthreads();
+        if (work) {
+          const float *a0 = As + g * ld;
+          const float *c0 = Cs + ((s ? k1 : 0) + kb) * ldc + col0;
+          int kk = 0;
+          for (; kk + 4 <= kc; kk += 4) {
+            float a[4][4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const float4 w = *reinterpret_cast<const float4 *>(a0 + i * groups * ld + kk);
+              a[i][0] = w.x; a[i][1] = w.y; a[i][2] = w.z; a[i][3] = w.w;
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const float4 c = *reinterpret_cast<const float4 *>(c0 + (kk + j) * ldc);
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                acc[i][0] = fma(a[i][j], c.x, acc[i][0]);
+                acc[i][1] = fma(a[i][j], c.y, acc[i][1]);
+                acc[i][2] = fma(a[i][j], c.z, acc[i][2]);
+                acc[i][3] = fma(a[i][j], c.w, acc[i][3]);
+              }
+            }
+          }
+          for (; kk < kc; ++kk) {
+            const float4 c = *reinterpret_cast<const float4 *>(c0 + kk * ldc);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const float a = a0[i * groups * ld + kk];
+              acc[i][0] = fma(a, c.x, acc[i][0]);
+              acc[i][1] = fma(a, c.y, acc[i][1]);
+              acc[i][2] = fma(a, c.z, acc[i][2]);
+              acc[i][3] = fma(a, c.w, acc[i][3]);
+            }
+          }
+        }
+      }
+    }
+    // the tile's outputs leave through the stage: contiguous rows x q
+    __syncthreads();
+    if (work)
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (col0 + u < q) As[(g + i * groups) * q + col0 + u] = acc[i][u];
+    __syncthreads();
+    const long long o0 = r0 * q;
+#pragma unroll 4
+    for (int e = threadIdx.x; e < rows * q; e += 256) {
+      float v = alpha * As[e];
+      if (Bm) v = fma(beta, Bm[o0 + e], v);
+      out[o0 + e] = v;
+    }
+  }
+}
 
 template <typename T>
 __device__ __forceinline__ void combine_narrow_body(
     long long n, int q, const T *__restrict__ A1, int k1, const double *__restrict__ C1,
     const T *__restrict__ A2, int k2, const double *__restrict__ C2, double alpha_d,
     double beta_d, const T *__restrict__ Bm, T *__restrict__ out, int vb, int vnb) {
+  if constexpr (sizeof(T) == 4) {
+    combine_rows_body(n, q, A1, k1, C1, A2, k2, C2, (float)alpha_d, (float)beta_d, Bm, out, vb,
+                      vnb);
+    return;
+  } else {
   __shared__ T Cs[2][kNarrowK * kNarrowQ];
   for (int e = threadIdx.x; e < k1 * q; e += blockDim.x) Cs[0][e] = (T)C1[e];
   if (A2)
@@ -848,6 +984,7 @@ __device__ __forceinline__ void combine_narrow_body(
       if (Bm) v = fma(beta, Bm[o], v);
       out[o] = v;
     }
+  }
   }
 }
 
@@ -1208,11 +1345,12 @@ __global__ void coef_batch_kernel(const BJob *__restrict__ jobs, const int *__re
   else if (smC2 >= 0 && e < 2 * len) b.cf[e] = (float)b.pp[(size_t)smC2 * len + e - len];
 }
 
-template <typename T>
+// (two kernels, so that each form has its own registers and shared memory)
+template <typename T, bool Narrow>
 __global__ void __launch_bounds__(256) combine_batch_kernel(const BJob *__restrict__ jobs,
                                                             const int *__restrict__ start, int J,
                                                             const unsigned char *__restrict__ active,
-                                                            CombSlots sl, int narrow) {
+                                                            CombSlots sl) {
   const int j = batch_job_of(start, J, blockIdx.x);
   if (!active[j]) return;
   const BJob &b = jobs[j];
@@ -1225,7 +1363,7 @@ __global__ void __launch_bounds__(256) combine_batch_kernel(const BJob *__restri
   T *out = (T *)b.blk[sl.out];
   const double *C1 = b.pp + (size_t)sl.c1 * len;
   const double *C2 = sl.c2 >= 0 ? b.pp + (size_t)sl.c2 * len : nullptr;
-  if (narrow) {
+  if constexpr (Narrow) {
     combine_narrow_body<T>(b.n, p, A1, p, C1, A2, p, C2, sl.alpha, sl.beta, Bm, out, vb,
                            b.comb_nb);
   } else {
@@ -1258,8 +1396,12 @@ ks_status batch_combine(Batch &B, int sA1, int smC1, int sA2, int smC2, double a
     if (nb == 0) continue;
     {
       ProfScope ps_(B.stream, KP_COMBINE);
-      combine_batch_kernel<T><<<nb, 256, 0, B.stream>>>(B.jobs_dev, B.map(m), B.J, B.active_dev,
-                                                        sl, narrow);
+      if (narrow)
+        combine_batch_kernel<T, true><<<nb, 256, 0, B.stream>>>(B.jobs_dev, B.map(m), B.J,
+                                                                B.active_dev, sl);
+      else
+        combine_batch_kernel<T, false><<<nb, 256, 0, B.stream>>>(B.jobs_dev, B.map(m), B.J,
+                                                                 B.active_dev, sl);
     }
     KS_CUDA_TRY(cudaGetLastError());
   }

@@ -129,3 +129,29 @@ def test_mid_gram_thread_blocks(pa, qb):
         got = P.step_gram_f32(torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda()).cpu().numpy()
         A, B = A.astype(np.float64), B.astype(np.float64)
         assert np.all(np.abs(got - A.T @ B) <= 2 * s.n * 2.0**-24 * (np.abs(A).T @ np.abs(B)))
+
+
+@pytest.mark.parametrize("k1,k2,q", [(1, 0, 1), (4, 4, 4), (5, 5, 5), (8, 8, 8), (17, 17, 17),
+                                     (26, 26, 26), (31, 30, 29), (32, 32, 32), (33, 64, 3),
+                                     (64, 63, 32)])
+def test_narrow_fp32_update_tiles(k1, k2, q):
+    # column groups with and without a remainder, K in one stage, two and a stage
+    # of one; rows that end inside a tile.  Each output is one chain of k1 + k2 FMAs
+    # and two more roundings, of operands rounded once.
+    import paper_1308_2864_gb300 as ks
+    for N in (4, 12):
+        s = ki.small_system(N=N, L=7.0, natoms=2, p=max(k1, k2, q), Z=4.0, seed=4)
+        P = ks.Problem.from_system(s)
+        rng = np.random.default_rng(k1 + 100 * q)
+        t = lambda a: torch.from_numpy(a).cuda()
+        f32 = lambda k: rng.standard_normal((s.n, k)).astype(np.float32)
+        A1, A2, Bm = f32(k1), f32(k2), f32(q)
+        C1, C2 = rng.standard_normal((k1, q)), rng.standard_normal((k2, q))
+        for bm, beta in ((None, 0.0), (Bm, 2.0)):
+            two = (t(A2), t(C2)) if k2 else (None, None)
+            got = P.step_combine_f32(t(A1), t(C1), *two, alpha=-0.5, beta=beta,
+                                     Bm=None if bm is None else t(bm)).cpu().numpy()
+            want = -0.5 * (A1.astype(float) @ C1 + A2.astype(float) @ C2) + beta * Bm
+            bound = 0.5 * (np.abs(A1).astype(float) @ np.abs(C1)
+                           + np.abs(A2).astype(float) @ np.abs(C2)) + beta * np.abs(Bm)
+            assert np.all(np.abs(got - want) <= (k1 + k2 + 4) * 2.0**-23 * bound)
