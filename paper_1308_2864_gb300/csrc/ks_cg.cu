@@ -58,38 +58,8 @@ struct CgArgs {
   int vb, vnb;                // this block's index among the vnb blocks that solve this system
 };
 
-// Grid barrier of the solver: one counter that only grows (zeroed before
-// the launch), `epoch` the arrivals expected so far (compared modulo 2^32).
-// Arrival is a release, the poll an acquire, so a phase costs one atomic
-// round trip and a poll; a wait that runs out records KS_ETIMEOUT and
-// adds 2^30 to the counter, which ends every other block's wait at its next
-// poll.
 __device__ __forceinline__ bool cg_barrier(const CgArgs &a, unsigned int &epoch) {
-  __shared__ int s_ok;
-  epoch += (unsigned int)a.vnb;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    unsigned int *cnt = &a.bar->count;
-    unsigned int v;
-    asm volatile("atom.add.release.gpu.global.u32 %0, [%1], 1;" : "=r"(v) : "l"(cnt) : "memory");
-    long long spins = 0;
-    unsigned int ns = 32;
-    while ((int)((v = ld_acquire_gpu(cnt)) - epoch) < 0) {
-      if (++spins > kSpinLimit) {
-        atomicCAS(a.status, 0, (int)KS_ETIMEOUT);
-        v = epoch + (1u << 30);
-        atomicAdd(cnt, 1u << 30);
-        break;
-      }
-      if (spins > kSpinFree) {
-        __nanosleep(ns);
-        if (ns < 256) ns <<= 1;
-      }
-    }
-    s_ok = v - epoch < (1u << 29);
-  }
-  __syncthreads();
-  return s_ok != 0;
+  return grid_barrier_n(a.bar, a.status, (unsigned int)a.vnb, epoch);
 }
 
 // (K v)_k for v = a + beta * b (b ignored when UseB is false), Dirichlet.

@@ -116,26 +116,25 @@ __global__ void __launch_bounds__(256) density_row_kernel(int n, int p, double o
 
 template <typename T>
 ks_status launch_density(Problem &P, const T *X, double *rho) {
-  if (P.p >= 32 && sizeof(T) == 8) {
+  if (P.p < 32) {
+    ProfScope ps_(P.stream, KP_DENSITY, 2.0 * P.n * P.p, (double)P.n * P.p * sizeof(T) + 8.0 * P.n);
+    density_thread_kernel<T><<<(P.n + kThreads - 1) / kThreads, kThreads, 0, P.stream>>>(
+        P.n, P.p, P.occ, X, rho);
+  } else if constexpr (sizeof(T) == 8) {
     const long long rows = 32 / kDenLanes * kDenSteps * (kThreads / 32);
     long long blocks = (P.n + rows - 1) / rows;
     if (blocks > 32LL * P.sms) blocks = 32LL * P.sms;
-    const double *Xd = reinterpret_cast<const double *>(X);
     ProfScope ps_(P.stream, KP_DENSITY, 2.0 * P.n * P.p, (double)P.n * P.p * sizeof(T) + 8.0 * P.n);
     if (P.p % 2 == 0 && reinterpret_cast<uintptr_t>(X) % 16 == 0)
-      density_row_kernel<true><<<(int)blocks, kThreads, 0, P.stream>>>(P.n, P.p, P.occ, Xd, rho);
+      density_row_kernel<true><<<(int)blocks, kThreads, 0, P.stream>>>(P.n, P.p, P.occ, X, rho);
     else
-      density_row_kernel<false><<<(int)blocks, kThreads, 0, P.stream>>>(P.n, P.p, P.occ, Xd, rho);
-  } else if (P.p >= 32) {
+      density_row_kernel<false><<<(int)blocks, kThreads, 0, P.stream>>>(P.n, P.p, P.occ, X, rho);
+  } else {
     const long long warps = (P.n + 31) / 32;
     long long blocks = (warps * 32 + kThreads - 1) / kThreads;
     if (blocks > 64LL * P.sms) blocks = 64LL * P.sms;
     ProfScope ps_(P.stream, KP_DENSITY, 2.0 * P.n * P.p, (double)P.n * P.p * sizeof(T) + 8.0 * P.n);
     density_warp_kernel<T><<<(int)blocks, kThreads, 0, P.stream>>>(P.n, P.p, P.occ, X, rho);
-  } else {
-    ProfScope ps_(P.stream, KP_DENSITY, 2.0 * P.n * P.p, (double)P.n * P.p * sizeof(T) + 8.0 * P.n);
-    density_thread_kernel<T><<<(P.n + kThreads - 1) / kThreads, kThreads, 0, P.stream>>>(
-        P.n, P.p, P.occ, X, rho);
   }
   KS_CUDA_TRY(cudaGetLastError());
   return KS_OK;

@@ -157,48 +157,41 @@ __device__ __forceinline__ unsigned int ld_acquire_gpu(const unsigned int *p) {
 }
 
 // Barrier of the nb blocks that share `bar` inside a cooperative launch (all
-// blocks of the launch co-resident; nb = the whole grid, or the blocks of one
-// system in a batched launch).
-// Every wait is bounded: a block that spins longer than kSpinLimit records
-// KS_ETIMEOUT in *status and leaves the barrier.  Returns false when the
-// status word holds an error, so that callers can return together.
-__device__ __forceinline__ bool grid_barrier_n(GridBarrier *bar, int *status, unsigned int nb) {
+// blocks of the launch co-resident): one counter that only grows (zeroed before
+// the launch), `epoch` the arrivals expected so far (compared modulo 2^32).
+// Arrival is a release, the poll an acquire, so a phase costs one atomic
+// round trip and a poll.  Every wait is bounded: one that runs out records
+// KS_ETIMEOUT in *status and adds 2^30 to the counter, which ends every other
+// block's wait at its next poll; false then.
+__device__ __forceinline__ bool grid_barrier_n(GridBarrier *bar, int *status, unsigned int nb,
+                                               unsigned int &epoch) {
   __shared__ int s_ok;
+  epoch += nb;
   __syncthreads();
   if (threadIdx.x == 0) {
-    const unsigned int gen = ld_acquire_gpu(&bar->gen);
-    __threadfence();
-    const unsigned int arrived = atomicAdd(&bar->count, 1u);
-    if (arrived == nb - 1) {
-      atomicExch(&bar->count, 0u);
-      __threadfence();
-      atomicAdd(&bar->gen, 1u);
-    } else {
-      // poll without sleeping first (a barrier between short phases is
-      // usually released within a few microseconds), then back off
-      long long spins = 0;
-      unsigned int ns = 32;
-      while (ld_acquire_gpu(&bar->gen) == gen) {
-        if (++spins > kSpinLimit) {
-          atomicCAS(status, 0, (int)KS_ETIMEOUT);
-          break;
-        }
-        if (spins > kSpinFree) {
-          __nanosleep(ns);
-          if (ns < 256) ns <<= 1;
-        }
+    unsigned int *cnt = &bar->count;
+    unsigned int v;
+    asm volatile("atom.add.release.gpu.global.u32 %0, [%1], 1;" : "=r"(v) : "l"(cnt) : "memory");
+    // poll without sleeping first (a barrier between short phases is
+    // usually released within a few microseconds), then back off
+    long long spins = 0;
+    unsigned int ns = 32;
+    while ((int)((v = ld_acquire_gpu(cnt)) - epoch) < 0) {
+      if (++spins > kSpinLimit) {
+        atomicCAS(status, 0, (int)KS_ETIMEOUT);
+        v = epoch + (1u << 30);
+        atomicAdd(cnt, 1u << 30);
+        break;
+      }
+      if (spins > kSpinFree) {
+        __nanosleep(ns);
+        if (ns < 256) ns <<= 1;
       }
     }
-    __threadfence();
-    s_ok = (*(volatile int *)status == 0);
+    s_ok = v - epoch < (1u << 29);
   }
   __syncthreads();
   return s_ok != 0;
-}
-
-// The same over the whole grid of the launch.
-__device__ __forceinline__ bool grid_barrier(GridBarrier *bar, int *status) {
-  return grid_barrier_n(bar, status, gridDim.x * gridDim.y * gridDim.z);
 }
 
 // Packed FP32 pairs (two lanes of one 64-bit register pair): each lane rounds

@@ -45,7 +45,6 @@ constexpr long long kSpinLimit = 1LL << 22;
 // Workspace of the software grid barrier used by cooperative kernels.
 struct GridBarrier {
   unsigned int count;
-  unsigned int gen;
 };
 
 // Launch geometry of the cooperative CG kernel.

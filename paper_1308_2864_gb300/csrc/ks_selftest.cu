@@ -18,7 +18,8 @@ namespace ks {
 namespace {
 
 __global__ void wait_timeout_probe_kernel(GridBarrier *bar, int *status) {
-  grid_barrier_n(bar, status, 2u);
+  unsigned int epoch = 0;
+  grid_barrier_n(bar, status, 2u, epoch);
 }
 
 struct ProbeState {
