@@ -60,11 +60,11 @@ C4_TTS_JOBS = (1, 2, 4, 5)
 MAXIT = 400000
 # DRAM bytes (read + write) per launch of a class's kernel, from one ncu
 # capture of the current kernels on this workload (profiles/c2_mixed_kernels_ncu.md):
-# the update's two launches of an iteration, 201 + 43 MB (D) and 212 + 97 MB
+# the update's two launches of an iteration, 201 + 39 MB (D) and 206 + 92 MB
 # (retraction), averaged.  To be retaken whenever the kernel changes.
 CLASS_TRAFFIC = {
-    "combine": (276.6e6, "ncu dram__bytes_read.sum + dram__bytes_write.sum per launch of "
-                         "combine_ta_kernel, mean of its two launches per iteration"),
+    "combine": (269.1e6, "ncu dram__bytes_read.sum + dram__bytes_write.sum per launch of "
+                         "combine_wa_kernel, mean of its two launches per iteration"),
 }
 GOLDEN_C1 = os.path.join(ROOT, "tests", "golden", "c1_converged.json")
 

@@ -27,8 +27,10 @@ ks_status ks_step_eii(ks_problem *prob, double *eii);
  * X: DEVICE n x p; rho: DEVICE n. */
 ks_status ks_step_density(ks_problem *prob, const double *X, double *rho);
 
-/* Hartree potential by conjugate gradients on K vH = 4 pi h^3 rho (the
- * discrete L^+ rho of Sec. 2.3), stopping at ||r|| <= cg_tol ||b||.
+/* Hartree potential from K vH = 4 pi h^3 rho (the discrete L^+ rho of
+ * Sec. 2.3) by defect correction with the FP32 sine-basis inverse, or by
+ * conjugate gradients where that stalls or is switched off, stopping at
+ * ||r|| <= cg_tol ||b||.
  *   rho    DEVICE n
  *   vH     DEVICE n, in/out: the start vector when warm != 0, else ignored
  *   resid  DEVICE n or NULL, receives r = 4 pi h^3 rho - K vH
