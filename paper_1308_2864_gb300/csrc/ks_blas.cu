@@ -1536,8 +1536,8 @@ __device__ __forceinline__ void wa_half(long long n, int q, long long row0, int 
 // zero-filled past the last row and past K) and no block barrier, so one warp's
 // epilogue overlaps the others' products.  The epilogue's operand (Bm or
 // add2) follows the K stages through the ring as two more stages: read from
-// global memory in the epilogue, its 16 loads per lane waited one by one.  A
-// lane owns rows ty + 4 i (i < 8) and columns 4 tx .. + 3 and 32 + 4 tx .. + 3
+// global memory in the epilogue, its 16 loads per lane waited one by one (one
+// stage where q <= kWaK).  A lane owns rows ty + 4 i (i < 8) and columns 4 tx .. + 3 and 32 + 4 tx .. + 3
 // (ty = lane / 8, tx = lane % 8).  The coefficient image (K x 64, zero padded)
 // is shared by the block's warps, and the FMAs are packed pairs of columns
 // (f2_fma: the scalar outer product stops at 49 of 76 TF/s).  Update with Bm at
@@ -1564,7 +1564,9 @@ __global__ void __launch_bounds__(32 * kWaWarps, 1) combine_wa_kernel(
   const int nst = (K + kWaK - 1) / kWaK;
   // the epilogue's operand: at most one of Bm (added) and add2 (to out2)
   const float *Es = Bm ? Bm : add2;
-  const int ntot = nst + (Es ? 2 : 0);
+  // one stage per kWaK of its q columns: for q <= kWaK a second one would lie
+  // past its rows
+  const int ntot = nst + (Es ? (q + kWaK - 1) / kWaK : 0);
   float *Cs = wa_smem;                                  // [nst * kWaK][64]
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, ty = lane >> 3, tx = lane & 7;
   constexpr int kRing = kWaStages * kWaRows * kWaLd;
@@ -1588,7 +1590,7 @@ __global__ void __launch_bounds__(32 * kWaWarps, 1) combine_wa_kernel(
   int istage = 0;                                       // K stage and tile of the next issue
   long long itile = first;
   int ibuf = 0;
-  // widths that are multiples of kWaK (p = 64): a stage lies in one operand
+  // widths that are multiples of kWaK (q = 32 or 64): a stage lies in one operand
   const bool whole = k1 % kWaK == 0 && k12 % kWaK == 0 && K % kWaK == 0 && q % kWaK == 0;
   auto issue = [&]() {
     const int k0 = istage * kWaK;
@@ -1604,8 +1606,7 @@ __global__ void __launch_bounds__(32 * kWaWarps, 1) combine_wa_kernel(
       const uint32_t d0 = smem_addr(dst + (lane >> 3) * kWaLd + (lane & 7) * 4);
 #pragma unroll
       for (int t = 0; t < kWaRows / 4; ++t) {
-        const bool in = row0 + 4 * t < n &&
-                        KS_IN((row0 + 4 * t) * ld + kc + (lane & 7) * 4 + 3, n * ld);
+        const bool in = row0 + 4 * t < n && KS_IN(kc + (lane & 7) * 4 + 3, ld);
         cp_async16(d0 + t * 4 * kWaLd * 4, in ? src + (long long)4 * t * ld : M, in ? 16u : 0u);
       }
     } else
