@@ -47,9 +47,10 @@ __device__ __forceinline__ double inv_of(double x) {
   return fma(y, fma(e, e, e), y);
 }
 
-// ln x for normal x > 0: x = 2^k m with m in [sqrt(1/2), sqrt(2)), and the
-// area-tangent series ln m = 2 (s + s^3/3 + s^5/5 + ...), s = (m - 1)/(m + 1),
-// |s| <= 0.1716: the terms through s^21 leave 2 s^23/23 < 3e-19.
+// ln x: x = 2^k m with m in [sqrt(1/2), sqrt(2)), and the area-tangent series
+// ln m = 2 (s + s^3/3 + s^5/5 + ...), s = (m - 1)/(m + 1), |s| <= 0.1716: the
+// terms through s^21 leave 2 s^23/23 < 3e-19.  -inf at 0: r_s of a density beyond
+// the FP32 range, whose start of rho^(-1/3) is 0, must not pass for a number.
 __device__ __forceinline__ double ln_series(double x) {
   const long long bits = __double_as_longlong(x);
   // exponent of x / sqrt(1/2), by its high word (sqrt(1/2) = 0x3fe6a09e...)
@@ -69,6 +70,7 @@ __device__ __forceinline__ double ln_series(double x) {
   t = fma(t, q, 0.2);
   t = fma(t, q, 1.0 / 3.0);
   const double s2 = s + s;
+  if (bits <= 0) return __longlong_as_double(0xfff0000000000000ll);
   return fma((double)k, 0.69314718055994530942, fma(s2 * q, t, s2));
 }
 
