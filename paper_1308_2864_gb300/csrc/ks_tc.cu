@@ -466,8 +466,9 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
 // x 512, K = 1024, against 0.48 ms here, 240 TF/s of useful products.)  The MMA
 // order per accumulator is that kernel's, so the results are too.  It stays for
 // operands without 16-byte rows.  Every wait is bounded; a role that gives up sets the
-// block's abort flag, the others stop at their next poll, copies and MMAs in
-// flight get a bounded wait, and the block records KS_ETIMEOUT.
+// block's abort flag, the others stop at their next poll (a warp by vote: its
+// lanes may see the flag at different polls, and what follows a wait is for whole
+// warps), copies and MMAs in flight get a bounded wait, and the block records KS_ETIMEOUT.
 constexpr int kWM = 256, kWK = 16, kWSlots = 3;
 constexpr int kWTile = 256 * kWK * 4;                       // 16 KiB: hi or lo of A or B
 constexpr int kWStage = 4 * kWTile;                         // A hi, A lo, B hi, B lo
@@ -546,7 +547,8 @@ __global__ void __launch_bounds__(kWThreads, 1) combine_tcw_kernel(
     };
     auto put = [&](int s, const float4 (&v)[4]) -> bool {
       const int slot = s % kWSlots, u = s / kWSlots;
-      if (u > 0 && !role_wait(&empty[slot], (uint32_t)((u - 1) & 1), abort)) return false;
+      const bool ok = u == 0 || role_wait(&empty[slot], (uint32_t)((u - 1) & 1), abort);
+      if (!__all_sync(0xffffffffu, ok)) return false;       // the warp leaves as a whole
       unsigned char *st = ring + slot * kWStage;
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
@@ -574,7 +576,8 @@ __global__ void __launch_bounds__(kWThreads, 1) combine_tcw_kernel(
         load(s + 3, vb);
       }
     }
-    if (role_wait(&accdone, 0u, abort) && !*abort) {
+    const bool done = role_wait(&accdone, 0u, abort) && !*abort;
+    if (__all_sync(0xffffffffu, done)) {
       asm volatile("tcgen05.fence::after_thread_sync;");
       // accumulator -> the warp's own transposed tile in the (now idle) ring, 64
       // columns at a time, then row-contiguous stores
