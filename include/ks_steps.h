@@ -135,13 +135,15 @@ ks_status ks_step_combine(ks_problem *prob, const double *A1, int k1, const doub
  * library (the software grid barrier of the cooperative kernels, the
  * mbarrier waits of the TMA and tensor-core pipelines) gives up after a fixed
  * number of polls, records KS_ETIMEOUT in the launch's status word and
- * returns.  The probe runs the grid barrier in a one-block launch while the
- * barrier expects two blocks, so its wait expires.
+ * returns.  The probe runs the grid barrier in a launch of four blocks while
+ * the barrier expects five, so their waits expire about together, then lets a
+ * fifth block arrive late; all five must be told of the failure.
  *   stream   cudaStream_t, or NULL for the legacy default stream
  *   status   HOST, receives the status the probe recorded (KS_ETIMEOUT when
  *            the bound works)
  *   seconds  HOST or NULL, wall time of the call (about a second)
- * Returns KS_OK when the probe ran and the context is still usable. */
+ * Returns KS_OK when the probe ran, the failure reached every block and the
+ * context is still usable. */
 ks_status ks_selftest_wait_timeout(void *stream, int *status, double *seconds);
 
 /* Peak-rate probe of the FMA pipes, the denominator of the roofline of the

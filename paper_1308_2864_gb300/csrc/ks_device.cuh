@@ -150,37 +150,40 @@ __device__ __forceinline__ void grid_reduce_tail(const double *part, int nb, dou
 // Polls of a grid-barrier wait before the waiting thread starts to sleep.
 constexpr long long kSpinFree = 1 << 14;
 
-__device__ __forceinline__ unsigned int ld_acquire_gpu(const unsigned int *p) {
-  unsigned int v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+__device__ __forceinline__ unsigned long long ld_acquire_gpu(const unsigned long long *p) {
+  unsigned long long v;
+  asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
   return v;
 }
 
 // Barrier of the nb blocks that share `bar` inside a cooperative launch (all
 // blocks of the launch co-resident): one counter that only grows (zeroed before
-// the launch), `epoch` the arrivals expected so far (compared modulo 2^32).
-// Arrival is a release, the poll an acquire, so a phase costs one atomic
-// round trip and a poll.  Every wait is bounded: one that runs out records
-// KS_ETIMEOUT in *status and adds 2^30 to the counter, which ends every other
-// block's wait at its next poll; false then.
+// the launch), `epoch` the arrivals expected so far.  Arrival is a release, the
+// poll an acquire, so a phase costs one atomic round trip and a poll.  Every wait
+// is bounded: one that runs out records KS_ETIMEOUT in *status and sets the
+// counter's top bit, which no number of arrivals or of further marks undoes.  It
+// ends every other block's wait at its next poll, and every later one's; false
+// then.
 __device__ __forceinline__ bool grid_barrier_n(GridBarrier *bar, int *status, unsigned int nb,
-                                               unsigned int &epoch) {
+                                               unsigned long long &epoch) {
   __shared__ int s_ok;
   epoch += nb;
   __syncthreads();
   if (threadIdx.x == 0) {
-    unsigned int *cnt = &bar->count;
-    unsigned int v;
-    asm volatile("atom.add.release.gpu.global.u32 %0, [%1], 1;" : "=r"(v) : "l"(cnt) : "memory");
+    unsigned long long *word = &bar->word;
+    unsigned long long v;
+    asm volatile("atom.add.release.gpu.global.u64 %0, [%1], 1;"
+                 : "=l"(v) : "l"(word) : "memory");
     // poll without sleeping first (a barrier between short phases is
     // usually released within a few microseconds), then back off
     long long spins = 0;
     unsigned int ns = 32;
-    while ((int)((v = ld_acquire_gpu(cnt)) - epoch) < 0) {
+    // (the mark makes v larger than any epoch)
+    while ((v = ld_acquire_gpu(word)) < epoch) {
       if (++spins > kSpinLimit) {
         atomicCAS(status, 0, (int)KS_ETIMEOUT);
-        v = epoch + (1u << 30);
-        atomicAdd(cnt, 1u << 30);
+        atomicOr(word, kBarrierFailed);
+        v = kBarrierFailed;
         break;
       }
       if (spins > kSpinFree) {
@@ -188,7 +191,7 @@ __device__ __forceinline__ bool grid_barrier_n(GridBarrier *bar, int *status, un
         if (ns < 256) ns <<= 1;
       }
     }
-    s_ok = v - epoch < (1u << 29);
+    s_ok = v < kBarrierFailed;
   }
   __syncthreads();
   return s_ok != 0;

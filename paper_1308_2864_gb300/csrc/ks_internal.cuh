@@ -42,10 +42,12 @@ constexpr int kStallWindow = 500;
 constexpr long long kSpinLimit = 1LL << 22;
 
 // ---------------------------------------------------------------- grid
-// Workspace of the software grid barrier used by cooperative kernels.
+// Workspace of the software grid barrier used by cooperative kernels: arrivals
+// in the low 63 bits, the failure mark (kBarrierFailed) in the top one.
 struct GridBarrier {
-  unsigned int count;
+  unsigned long long word;
 };
+constexpr unsigned long long kBarrierFailed = 1ull << 63;
 
 // Launch geometry of the cooperative CG kernel.
 constexpr int kCgThreads = 256;

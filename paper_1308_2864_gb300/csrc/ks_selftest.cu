@@ -5,10 +5,13 @@
 // KS_ETIMEOUT in the launch's status word and returns, so a wait that cannot
 // complete leaves the context usable and reaches the host as an error.
 //
-// The probe runs the library's own grid barrier in a launch of one block
-// while the barrier expects two: the second arrival never comes, the
-// waiting thread gives up after kSpinLimit polls (about a second with the
-// back-off), and the kernel returns with KS_ETIMEOUT recorded.
+// The probe runs the library's own grid barrier in a launch of kProbeBlocks
+// blocks while the barrier expects one more: the last arrival never comes, the
+// waiting threads give up after kSpinLimit polls (about a second with the
+// back-off), all about together, and the kernel returns with KS_ETIMEOUT
+// recorded.  A second launch is the late block: its arrival completes the count,
+// and it must be told of the failure all the same, or it would go on with what
+// the departed blocks never wrote.
 #include <chrono>
 
 #include "ks_device.cuh"
@@ -17,14 +20,18 @@
 namespace ks {
 namespace {
 
-__global__ void wait_timeout_probe_kernel(GridBarrier *bar, int *status) {
-  unsigned int epoch = 0;
-  grid_barrier_n(bar, status, 2u, epoch);
+constexpr unsigned int kProbeBlocks = 4;
+
+// told: blocks that left the barrier with its failure.
+__global__ void wait_timeout_probe_kernel(GridBarrier *bar, int *status, int *told) {
+  unsigned long long epoch = 0;
+  const bool ok = grid_barrier_n(bar, status, kProbeBlocks + 1u, epoch);
+  if (threadIdx.x == 0 && !ok) atomicAdd(told, 1);
 }
 
 struct ProbeState {
   GridBarrier bar;
-  int status;
+  int status, told;
 };
 
 }  // namespace
@@ -45,8 +52,9 @@ ks_status ks_selftest_wait_timeout(void *stream, int *status, double *seconds) {
   cudaError_t e = cudaMemsetAsync(d, 0, sizeof(ProbeState), s);
   if (e == cudaSuccess) {
     {
-      ProfScope ps_(s, KP_OTHER);
-      wait_timeout_probe_kernel<<<1, 32, 0, s>>>(&d->bar, &d->status);
+      ProfScope ps_(s, KP_OTHER, 0.0, 0.0, 2);
+      wait_timeout_probe_kernel<<<kProbeBlocks, 32, 0, s>>>(&d->bar, &d->status, &d->told);
+      wait_timeout_probe_kernel<<<1, 32, 0, s>>>(&d->bar, &d->status, &d->told);
     }
     e = cudaGetLastError();
   }
@@ -55,6 +63,9 @@ ks_status ks_selftest_wait_timeout(void *stream, int *status, double *seconds) {
   if (e != cudaSuccess) st = cuda_error(e, "wait-timeout probe");
   cudaFree(d);
   if (st != KS_OK) return st;
+  if (h.status == KS_ETIMEOUT && h.told != (int)kProbeBlocks + 1)
+    return set_error(KS_ECUDA, "wait-timeout probe: %d of %d blocks were told of the failure",
+                     h.told, (int)kProbeBlocks + 1);
   *status = h.status;
   if (seconds)
     *seconds = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
