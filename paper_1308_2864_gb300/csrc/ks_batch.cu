@@ -57,14 +57,14 @@ ks_status upload(Batch &B, void *dst, const void *src, size_t bytes) {
   return KS_OK;
 }
 
-// Device scalars, status words and the CG's remaining-job count to the
+// Device scalars, status words and the CG's remaining-job counts to the
 // pinned host mirrors (capturable: fixed addresses, no synchronisation).
 ks_status copy_scalars(Batch &B) {
   KS_CUDA_TRY(cudaMemcpyAsync(B.scal_host, B.scal_dev, sizeof(double) * SC_COUNT * B.J,
                               cudaMemcpyDeviceToHost, B.stream));
   KS_CUDA_TRY(cudaMemcpyAsync(B.status_host, B.status_dev, sizeof(int) * B.J,
                               cudaMemcpyDeviceToHost, B.stream));
-  KS_CUDA_TRY(cudaMemcpyAsync(B.cg_remaining_host, B.cg_remaining_dev, sizeof(int),
+  KS_CUDA_TRY(cudaMemcpyAsync(B.cg_remaining_host, B.cg_remaining_dev, 2 * sizeof(int),
                               cudaMemcpyDeviceToHost, B.stream));
   return KS_OK;
 }
@@ -634,13 +634,13 @@ ks_status ks_batch_create(const ks_problem_desc *descs, int njobs, void *stream,
   BALLOC(B.status_dev, sizeof(int) * njobs);
   BALLOC(B.active_dev, (size_t)njobs);
   BALLOC(B.tau_dev, sizeof(double) * njobs);
-  BALLOC(B.cg_remaining_dev, sizeof(int));
+  BALLOC(B.cg_remaining_dev, 2 * sizeof(int));
   HALLOC(B.scal_host, sizeof(double) * SC_COUNT * njobs);
   HALLOC(B.status_host, sizeof(int) * njobs);
   HALLOC(B.active_host, (size_t)njobs);
   HALLOC(B.tau_host, sizeof(double) * njobs);
   HALLOC(B.cg_tolw_host, sizeof(double) * 2 * njobs);
-  HALLOC(B.cg_remaining_host, sizeof(int));
+  HALLOC(B.cg_remaining_host, 2 * sizeof(int));
   B.ring_bytes = (size_t)64 * (((size_t)njobs * sizeof(double) + 255) / 256 * 256);
   HALLOC(B.ring_host, B.ring_bytes);
   if ((e = cudaMemsetAsync(B.scal_dev, 0, sizeof(double) * SC_COUNT * njobs, B.stream)) != cudaSuccess ||

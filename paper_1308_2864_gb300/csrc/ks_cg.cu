@@ -870,15 +870,17 @@ ks_status launch_cg(Problem &P, const double *rho, double *v, double *r, bool wa
 //   init     r = b - K x (x = 0 when cold), r.r, b.b, tolerance
 //   A/B/C    the fused sine-basis transforms, one block per (job, plane)
 //            resp. (job, ky); C writes z
-//   update   x += z, r -= K z, r.r -> convergence
-//   it1, it2 a CG iteration, for jobs without the preconditioner only
-//            (launched when there is such a job): p = r + beta p_old, q = K p,
-//            p.q -> alpha; x += alpha p, r -= alpha q, r.r
+//   update   x += z, r -= K z, r.r -> convergence, or a step that did not halve
+//            the residual: the job is handed to the CG iterations (as in cg_body)
+//   it1, it2 a CG iteration, for jobs without the preconditioner and those handed
+//            over (launched when there is such a job): p = r + beta p_old,
+//            q = K p, p.q -> alpha; x += alpha p, r -= alpha q, r.r
 // A job that has converged (or failed) skips every later phase.  The host
-// reads the number of jobs still iterating once per iteration.
+// reads the number of jobs still iterating, and of those in CG, once per iteration.
 struct CgState {
   double rr, bb, thr, rho, beta, alpha;
   int it, done, maxit, precond;
+  int cg_it;                       // CG iterations done
 };
 
 // Last block of one job's nb blocks: sums of the nchan partial channels
@@ -960,6 +962,7 @@ __global__ void __launch_bounds__(kCgThreads) cg_b_init(CgBatchView v) {
     t.rho = s[0];
     t.beta = 0.0;
     t.it = 0;
+    t.cg_it = 0;
     t.maxit = a.maxit;
     t.precond = a.precond;
     t.done = t.rr <= t.thr ? 1 : 0;
@@ -1018,7 +1021,15 @@ __global__ void __launch_bounds__(kCgThreads) cg_b_update(CgBatchView v) {
   if (threadIdx.x == 0) a.part[vb] = sum;
   double s[1];
   if (!job_tail(a.part, nb, 1, v.counters + j, smem, s)) return;
-  if (threadIdx.x == 0) cg_step_done(a, v.st[j], s[0]);
+  if (threadIdx.x == 0) {
+    CgState &u = v.st[j];
+    const bool slow = s[0] > 0.25 * u.rr;
+    cg_step_done(a, u, s[0]);
+    if (slow && !u.done) {
+      u.precond = 0;
+      u.rho = s[0];
+    }
+  }
 }
 
 __global__ void __launch_bounds__(kCgThreads) cg_b_it1(CgBatchView v) {
@@ -1031,14 +1042,14 @@ __global__ void __launch_bounds__(kCgThreads) cg_b_it1(CgBatchView v) {
   const int N = a.N;
   const long long NN = (long long)N * N;
   const double *s_vec = a.r;
-  double *pold = (t.it % 2 == 0) ? a.pb : a.pa, *pnew = (t.it % 2 == 0) ? a.pa : a.pb;
+  double *pold = (t.cg_it % 2 == 0) ? a.pb : a.pa, *pnew = (t.cg_it % 2 == 0) ? a.pa : a.pb;
   double pq_l = 0.0;
   for (long long k = (long long)vb * blockDim.x + threadIdx.x; k < a.n;
        k += (long long)nb * blockDim.x) {
     const int ix = (int)(k % N), iy = (int)((k / N) % N), iz = (int)(k / NN);
     double pk;
-    const double qk = t.it == 0 ? stiff_apply<false>(s_vec, nullptr, 0.0, N, ix, iy, iz, a.c, &pk)
-                                : stiff_apply<true>(s_vec, pold, t.beta, N, ix, iy, iz, a.c, &pk);
+    const double qk = t.cg_it == 0 ? stiff_apply<false>(s_vec, nullptr, 0.0, N, ix, iy, iz, a.c, &pk)
+                                   : stiff_apply<true>(s_vec, pold, t.beta, N, ix, iy, iz, a.c, &pk);
     pnew[k] = pk;
     a.q[k] = qk;
     pq_l = fma(pk, qk, pq_l);
@@ -1065,7 +1076,7 @@ __global__ void __launch_bounds__(kCgThreads) cg_b_it2(CgBatchView v) {
   const CgArgs &a = v.args[j];
   const CgState t = v.st[j];
   if (t.precond) return;
-  const double *p = (t.it % 2 == 0) ? a.pa : a.pb;
+  const double *p = (t.cg_it % 2 == 0) ? a.pa : a.pb;
   double rl = 0.0;
   for (long long k = (long long)vb * blockDim.x + threadIdx.x; k < a.n;
        k += (long long)nb * blockDim.x) {
@@ -1081,21 +1092,27 @@ __global__ void __launch_bounds__(kCgThreads) cg_b_it2(CgBatchView v) {
   if (threadIdx.x == 0) {
     CgState &u = v.st[j];
     cg_step_done(a, u, s[0]);
+    ++u.cg_it;
     u.beta = s[0] / u.rho;
     u.rho = s[0];
   }
 }
 
-// Number of active jobs still iterating.
+// Active jobs still iterating: out[0] all of them, out[1] those in CG.
 __global__ void cg_b_count(const CgState *st, const unsigned char *active, int J, int *out) {
-  __shared__ int cnt;
-  if (threadIdx.x == 0) cnt = 0;
+  __shared__ int cnt[2];
+  if (threadIdx.x < 2) cnt[threadIdx.x] = 0;
   __syncthreads();
-  int c = 0;
-  for (int j = threadIdx.x; j < J; j += blockDim.x) c += active[j] && !st[j].done;
-  atomicAdd(&cnt, c);
+  int c = 0, g = 0;
+  for (int j = threadIdx.x; j < J; j += blockDim.x)
+    if (active[j] && !st[j].done) {
+      ++c;
+      g += !st[j].precond;
+    }
+  atomicAdd(&cnt[0], c);
+  atomicAdd(&cnt[1], g);
   __syncthreads();
-  if (threadIdx.x == 0) *out = cnt;
+  if (threadIdx.x < 2) out[threadIdx.x] = cnt[threadIdx.x];
 }
 
 ks_status batch_cg_setup(Batch &B) {
@@ -1191,12 +1208,10 @@ static ks_status cg_precond_launch(Batch &B) {
 }
 
 // One step of every job still iterating: correction of the preconditioned
-// jobs, CG iteration of the others (none in the usual batch).
-static ks_status cg_iteration_launch(Batch &B) {
+// jobs (pre), CG iteration of the others (plain; none in the usual batch).
+static ks_status cg_iteration_launch(Batch &B, bool pre, bool plain) {
   const CgBatchView nodes = cg_view(B, BM_CG_NODES);
   const int nn = B.total(BM_CG_NODES);
-  bool plain = false, pre = false;
-  for (int j = 0; j < B.J; ++j) (B.probs[j]->P.cg_precond ? pre : plain) = true;
   ProfScope ps_(B.stream, KP_CG, 0.0, 0.0, (pre ? 4 : 0) + (plain ? 2 : 0));
   if (pre) {
     KS_TRY(cg_precond_launch(B));
@@ -1236,7 +1251,10 @@ ks_status batch_cg_launch(Batch &B, int iters) {
     cg_b_init<<<B.total(BM_CG_NODES), kCgThreads, 0, B.stream>>>(nodes);
     KS_CUDA_TRY(cudaGetLastError());
   }
-  for (int it = 0; it < iters; ++it) KS_TRY(cg_iteration_launch(B));
+  // (a job handed over to CG in these steps goes on in batch_cg_continue)
+  bool plain = false, pre = false;
+  for (int j = 0; j < B.J; ++j) (B.probs[j]->P.cg_precond ? pre : plain) = true;
+  for (int it = 0; it < iters; ++it) KS_TRY(cg_iteration_launch(B, pre, plain));
   return cg_count_launch(B);
 }
 
@@ -1245,11 +1263,12 @@ ks_status batch_cg_continue(Batch &B) {
   for (int j = 0; j < B.J; ++j)
     if (B.active_host[j] && B.probs[j]->P.cg_maxit > maxit) maxit = B.probs[j]->P.cg_maxit;
   for (int it = 0; it < maxit; ++it) {
-    KS_CUDA_TRY(cudaMemcpyAsync(B.cg_remaining_host, B.cg_remaining_dev, sizeof(int),
+    KS_CUDA_TRY(cudaMemcpyAsync(B.cg_remaining_host, B.cg_remaining_dev, 2 * sizeof(int),
                                 cudaMemcpyDeviceToHost, B.stream));
     KS_CUDA_TRY(cudaStreamSynchronize(B.stream));
-    if (*B.cg_remaining_host == 0) break;
-    KS_TRY(cg_iteration_launch(B));
+    const int left = B.cg_remaining_host[0], plain = B.cg_remaining_host[1];
+    if (left == 0) break;
+    KS_TRY(cg_iteration_launch(B, left > plain, plain > 0));
     KS_TRY(cg_count_launch(B));
   }
   return KS_OK;

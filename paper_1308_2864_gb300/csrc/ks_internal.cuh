@@ -464,7 +464,7 @@ struct Batch {
   void *cg_state_dev = nullptr;    // J per-job PCG scalars
   double *cg_tolw_dev = nullptr, *cg_tolw_host = nullptr;   // per job (tolerance, warm)
   unsigned int *cg_counters = nullptr;                      // per-job last-block counters
-  int *cg_remaining_dev = nullptr, *cg_remaining_host = nullptr;
+  int *cg_remaining_dev = nullptr, *cg_remaining_host = nullptr;   // jobs iterating, in CG
   std::vector<unsigned char> warm; // per job: a previous Hartree potential exists
   char *ring_host = nullptr;       // pinned staging ring of the small uploads
   size_t ring_bytes = 0, ring_used = 0;

@@ -33,3 +33,32 @@ def test_hartree_parity_transforms(N):
     w = torch.from_numpy(0.9 * exact + 0.01 * rho).cuda()
     w, _, _ = P.step_hartree(torch.from_numpy(rho).cuda(), w, warm=True)
     assert np.abs(w.cpu().numpy() - exact).max() <= 1e-8 * np.abs(exact).max()
+
+
+@pytest.mark.parametrize("graphs", [True, False])
+def test_stalled_correction_goes_on_as_conjugate_gradients(graphs):
+    # at a node spacing of 3e19 the products of two 1-D eigenvalues overflow FP32
+    # for half of the modes: the sine-basis inverse leaves them out, the
+    # correction stalls, and both paths finish with CG.  A job table holds such a
+    # job beside an ordinary one.  Energies at the Hartree tolerance (1e-10 of the
+    # residual): 1e-8, as the potential above.
+    import paper_1308_2864_gb300 as ks
+    from oracle import energy as oe
+    wide = ki.small_system(N=9, L=3e20, natoms=1, p=1, Z=2.0, seed=3)
+    usual = ki.small_system(N=10, L=7.0, natoms=2, p=2, Z=1.0, seed=7)
+    P = ks.Problem.from_system(wide)
+    # (x0() is bound to the atom; norms near 1, as the factor's FP32 starts need)
+    x0 = np.random.default_rng(5).standard_normal((wide.n, 1)) / math.sqrt(wide.n * wide.h ** 3)
+    X = torch.from_numpy(x0).cuda()
+    P.orthonormalize(X)
+    rho = P.step_density(X)
+    _, _, it = P.step_hartree(rho)
+    assert 4 < it < 200
+    E = P.energy_grad(X)[0]
+    assert E == pytest.approx(oe.evaluate(oe.Model.from_system(wide), X.cpu().numpy()).E, rel=1e-8)
+    B = ks.Batch([usual, wide])
+    B.set_graphs(graphs)
+    res, _ = B.minimize([usual.x0(), x0], gtol=1e30, maxit=1)
+    assert [r["status"] for r in res] == [0, 0]
+    assert res[1]["E"] == pytest.approx(E, rel=1e-8)
+    assert res[1]["cg_iters_total"] < 200
