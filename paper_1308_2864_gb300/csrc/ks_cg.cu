@@ -58,7 +58,7 @@ struct CgArgs {
   int vb, vnb;                // this block's index among the vnb blocks that solve this system
 };
 
-__device__ __forceinline__ bool cg_barrier(const CgArgs &a, unsigned long long &epoch) {
+__device__ __forceinline__ bool cg_barrier(const CgArgs &a, unsigned int &epoch) {
   return grid_barrier_n(a.bar, a.status, (unsigned int)a.vnb, epoch);
 }
 
@@ -202,7 +202,7 @@ constexpr size_t kTiledSmem = (size_t)(kTK * kTCPad + kTK * kTJ) * sizeof(float)
 
 // z = P r (six tiled passes, a grid barrier after each of the first five);
 // false when a barrier failed.
-__device__ bool apply_precond(const CgArgs &a, unsigned long long &epoch) {
+__device__ bool apply_precond(const CgArgs &a, unsigned int &epoch) {
   extern __shared__ float dyn[];
   tiled_pass<0>(a, a.r32, a.t1, nullptr, 0, dyn);
   if (!cg_barrier(a, epoch)) return false;
@@ -561,7 +561,7 @@ __device__ __forceinline__ void fused_pass_c(const CgArgs &a, const float *in, d
 __device__ __forceinline__ bool small_tiles(int N) { return half_pad(N) <= 32; }
 
 // z = P r of the fused form: three phases, a barrier after the first two.
-__device__ bool apply_precond_fused(const CgArgs &a, unsigned long long &epoch) {
+__device__ bool apply_precond_fused(const CgArgs &a, unsigned int &epoch) {
   extern __shared__ float dyn[];
   const bool s = small_tiles(a.N);
   if (s) fused_pass_a<2>(a, a.r32, a.t1, dyn); else fused_pass_a<4>(a, a.r32, a.t1, dyn);
@@ -651,7 +651,7 @@ __device__ __forceinline__ double defect_update(const CgArgs &a, bool first, dou
 __device__ void cg_body(const CgArgs &a) {
   __shared__ double smem[2 * 33];
   const int nb = a.vnb;
-  unsigned long long epoch = 0;
+  unsigned int epoch = 0;
   double *partA = a.part, *partB = a.part + nb, *partC = a.part + 2 * nb, *partD = a.part + 3 * nb;
   const long long tid = (long long)a.vb * blockDim.x + threadIdx.x;
   const long long stride = (long long)a.vnb * blockDim.x;

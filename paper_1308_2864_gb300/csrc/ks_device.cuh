@@ -158,19 +158,20 @@ __device__ __forceinline__ unsigned long long ld_acquire_gpu(const unsigned long
 
 // Barrier of the nb blocks that share `bar` inside a cooperative launch (all
 // blocks of the launch co-resident): one counter that only grows (zeroed before
-// the launch), `epoch` the arrivals expected so far.  Arrival is a release, the
+// the launch), `epoch` the barriers passed so far.  Arrival is a release, the
 // poll an acquire, so a phase costs one atomic round trip and a poll.  Every wait
 // is bounded: one that runs out records KS_ETIMEOUT in *status and sets the
 // counter's top bit, which no number of arrivals or of further marks undoes.  It
 // ends every other block's wait at its next poll, and every later one's; false
 // then.
 __device__ __forceinline__ bool grid_barrier_n(GridBarrier *bar, int *status, unsigned int nb,
-                                               unsigned long long &epoch) {
+                                               unsigned int &epoch) {
   __shared__ int s_ok;
-  epoch += nb;
+  ++epoch;
   __syncthreads();
   if (threadIdx.x == 0) {
     unsigned long long *word = &bar->word;
+    const unsigned long long all = (unsigned long long)epoch * nb;
     unsigned long long v;
     asm volatile("atom.add.release.gpu.global.u64 %0, [%1], 1;"
                  : "=l"(v) : "l"(word) : "memory");
@@ -178,8 +179,8 @@ __device__ __forceinline__ bool grid_barrier_n(GridBarrier *bar, int *status, un
     // usually released within a few microseconds), then back off
     long long spins = 0;
     unsigned int ns = 32;
-    // (the mark makes v larger than any epoch)
-    while ((v = ld_acquire_gpu(word)) < epoch) {
+    // (the mark makes v larger than any count)
+    while ((v = ld_acquire_gpu(word)) < all) {
       if (++spins > kSpinLimit) {
         atomicCAS(status, 0, (int)KS_ETIMEOUT);
         atomicOr(word, kBarrierFailed);

@@ -24,7 +24,7 @@ constexpr unsigned int kProbeBlocks = 4;
 
 // told: blocks that left the barrier with its failure.
 __global__ void wait_timeout_probe_kernel(GridBarrier *bar, int *status, int *told) {
-  unsigned long long epoch = 0;
+  unsigned int epoch = 0;
   const bool ok = grid_barrier_n(bar, status, kProbeBlocks + 1u, epoch);
   if (threadIdx.x == 0 && !ok) atomicAdd(told, 1);
 }
