@@ -1181,6 +1181,8 @@ ks_status ks_problem_create(const ks_problem_desc *d, ks_problem **out) {
   if ((st = configure_tc_kernels()) != KS_OK) return fail(st);
   if ((st = configure_blas_kernels()) != KS_OK) return fail(st);
   if ((st = configure_sym_kernels()) != KS_OK) return fail(st);
+  if ((st = configure_stencil_kernels(P.p)) != KS_OK) return fail(st);
+  if ((st = configure_oz_kernels()) != KS_OK) return fail(st);
   if ((st = launch_setup(P)) != KS_OK) return fail(st);
   if ((st = launch_sine_setup(P)) != KS_OK) return fail(st);
   if ((st = sync_scalars(P)) != KS_OK) return fail(st);

@@ -245,6 +245,7 @@ int cg_grid_blocks(int sms, int n, int N);
 // blocks of one job in the batched transforms' passes A and B/C (one item each)
 // and in the update (kUpY x kUpZ nodes per thread)
 void cg_batch_blocks(int N, long long *a, long long *bc, long long *update);
+ks_status configure_oz_kernels();
 ks_status launch_gram_oz(Problem &P, const double *A, int pa, const double *B, int qb,
                          int *emax, double *part, int chunks);
 int gram_oz_chunks(const Problem &P, int pa, int qb);
@@ -262,6 +263,7 @@ ks_status launch_reduce(Problem &P, const double *partials, int nchan, int nb, d
 // Blocks of the grid-stride reduction kernels (their partials are nchan x this).
 int reduce_blocks(const Problem &P, long long work);
 // ks_stencil.cu (T = double or float; sums always returned in FP64)
+ks_status configure_stencil_kernels(int p);
 // (EX, MX may be null: not stored)
 template <typename T>
 ks_status launch_hamiltonian(Problem &P, const T *X, const double *veff, T *EX, T *MX,

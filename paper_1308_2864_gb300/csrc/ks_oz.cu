@@ -621,7 +621,13 @@ __global__ void __launch_bounds__(kOzThreads, 1) combine_oz_kernel(
   oz_tmem_free(tmem);
 }
 
-static bool gz_configured = false, cz_configured = false;
+// (on the current device; called when a problem is created)
+ks_status configure_oz_kernels() {
+  const auto at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  KS_CUDA_TRY(cudaFuncSetAttribute(gram_oz_kernel, at, kGzSmem));
+  KS_CUDA_TRY(cudaFuncSetAttribute(combine_oz_kernel, at, kCzSmem));
+  return KS_OK;
+}
 
 size_t oz_image_bytes(int p) { return (size_t)((p + kOzT - 1) / kOzT) * kOzS * kCzCTile; }
 
@@ -633,11 +639,6 @@ bool combine_oz_applies(const Problem &P, int k1, int k2, int q) {
 ks_status launch_combine_oz(Problem &P, const double *A1, int k1, const double *C1,
                             const double *A2, int k2, const double *C2, double alpha, double beta,
                             const double *Bm, double *out, int q) {
-  if (!cz_configured) {
-    KS_CUDA_TRY(cudaFuncSetAttribute(combine_oz_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     kCzSmem));
-    cz_configured = true;
-  }
   if (!A2) k2 = 0;
   const int K = k1 + k2;
   const int kp = (K + kCzKs - 1) / kCzKs * kCzKs;
@@ -664,11 +665,6 @@ ks_status launch_combine_oz(Problem &P, const double *A1, int k1, const double *
 
 ks_status launch_gram_oz(Problem &P, const double *A, int pa, const double *B, int qb,
                          int *emax, double *part, int chunks) {
-  if (!gz_configured) {
-    KS_CUDA_TRY(cudaFuncSetAttribute(gram_oz_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     kGzSmem));
-    gz_configured = true;
-  }
   KS_CUDA_TRY(cudaMemsetAsync(emax, 0, sizeof(int) * (size_t)(pa + qb), P.stream));
   {
     ProfScope ps_(P.stream, KP_GRAM, 0.0, (double)P.n * (pa + qb) * sizeof(double), 2);

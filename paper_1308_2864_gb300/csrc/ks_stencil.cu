@@ -40,8 +40,6 @@
 //     out-of-bounds fill.  V_eff of the output plane is staged in the
 //     working precision once per node.
 //   plain loads (any p): all threads copy the halo box element by element.
-#include <mutex>
-
 #include "ks_async.cuh"
 #include "ks_device.cuh"
 
@@ -987,18 +985,6 @@ static bool stencil_launch_tma(Problem &P, const StArgs &a, int cls, double flop
     if (encode_tensor_map_4d(&ta.aux[i], aux[i], (int)sizeof(T), dims, nbox) != KS_OK)
       return false;
   if constexpr (kF2) {
-    static std::once_flag once;
-    static cudaError_t attr = cudaSuccess;
-    static_assert(st_f2_smem<Kind>() <= 224 * 1024, "the ring fits an SM");
-    std::call_once(once, [] {
-      attr = cudaFuncSetAttribute(stencil_f32x2_kernel<Kind>,
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)st_f2_smem<Kind>());
-    });
-    if (attr != cudaSuccess) {
-      cudaGetLastError();
-      return false;
-    }
     {
       ProfScope ps_(P.stream, cls, flops, bytes);
       stencil_f32x2_kernel<Kind><<<a.nb, kStThreads, st_f2_smem<Kind>(), P.stream>>>(ta);
@@ -1008,22 +994,6 @@ static bool stencil_launch_tma(Problem &P, const StArgs &a, int cls, double flop
     return true;
   } else {
   using Rg = StRing<T, PC, Kind>;
-  // the ring plus the static shared memory (mbarriers, V_eff planes,
-  // reduction scratch: up to ~10 KiB) for two blocks per SM; the kernel
-  // opts in to the ring's size once
-  static_assert(Rg::SMEM + 10 * 1024 <= 113 * 1024, "two blocks of the ring fit an SM");
-  {
-    static std::once_flag once;
-    static cudaError_t attr = cudaSuccess;
-    std::call_once(once, [] {
-      attr = cudaFuncSetAttribute(stencil_tma_kernel<T, PC, Kind>,
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Rg::SMEM);
-    });
-    if (attr != cudaSuccess) {
-      cudaGetLastError();
-      return false;
-    }
-  }
   {
     ProfScope ps_(P.stream, cls, flops, bytes);
     stencil_tma_kernel<T, PC, Kind><<<a.nb, kStThreads, Rg::SMEM, P.stream>>>(ta);
@@ -1032,6 +1002,48 @@ static bool stencil_launch_tma(Problem &P, const StArgs &a, int cls, double flop
   if (e != cudaSuccess) *st = cuda_error(e, "stencil_tma_kernel");
   return true;
   }
+}
+
+// The rings' opt-in to their dynamic shared memory, on the current device: a
+// function's limit belongs to the device, so it is set when a problem is created
+// (like the other kernels') and not once per process.
+template <typename T, int PC, int Kind>
+static ks_status stencil_opt_in() {
+  const auto at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  if constexpr (sizeof(T) == 4 && PC == 32) {
+    static_assert(st_f2_smem<Kind>() <= 224 * 1024, "the ring fits an SM");
+    KS_CUDA_TRY(cudaFuncSetAttribute(stencil_f32x2_kernel<Kind>, at, (int)st_f2_smem<Kind>()));
+  } else {
+    using Rg = StRing<T, PC, Kind>;
+    // the ring plus the static shared memory (mbarriers, V_eff planes,
+    // reduction scratch: up to ~10 KiB) for two blocks per SM
+    static_assert(Rg::SMEM + 10 * 1024 <= 113 * 1024, "two blocks of the ring fit an SM");
+    // (48 KiB, static memory included, need no opt-in)
+    if constexpr (Rg::SMEM + 10 * 1024 > 48 * 1024)
+      KS_CUDA_TRY(cudaFuncSetAttribute(stencil_tma_kernel<T, PC, Kind>, at, (int)Rg::SMEM));
+  }
+  return KS_OK;
+}
+
+template <int PC>
+static ks_status stencil_opt_in_pc() {
+  KS_TRY((stencil_opt_in<double, PC, SK_HAM>()));
+  KS_TRY((stencil_opt_in<double, PC, SK_MASS>()));
+  KS_TRY((stencil_opt_in<double, PC, SK_MASS_DOT>()));
+  KS_TRY((stencil_opt_in<double, PC, SK_MASS_BB>()));
+  KS_TRY((stencil_opt_in<float, PC, SK_HAM>()));
+  KS_TRY((stencil_opt_in<float, PC, SK_MASS>()));
+  KS_TRY((stencil_opt_in<float, PC, SK_MASS_DOT>()));
+  KS_TRY((stencil_opt_in<float, PC, SK_MASS_BB>()));
+  return stencil_opt_in<float, PC, SK_HAM_INC>();
+}
+
+// (of the orbital chunk that stencil_launch takes for p)
+ks_status configure_stencil_kernels(int p) {
+  if (p >= 32) return stencil_opt_in_pc<32>();
+  if (p >= 16) return stencil_opt_in_pc<16>();
+  if (p >= 8) return stencil_opt_in_pc<8>();
+  return p == 1 ? KS_OK : stencil_opt_in_pc<4>();
 }
 
 template <typename T, int PC, int Kind>

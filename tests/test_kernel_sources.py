@@ -21,3 +21,19 @@ def test_wide_update_warps_leave_their_waits_by_vote():
     assert len(waits) == warps.count("role_wait(") == 2
     for name in waits:
         assert re.search(r"__all_sync\(0xffffffffu, %s\)" % name, warps)
+
+
+def test_function_attributes_are_not_set_once_per_process():
+    # a kernel's shared-memory limit belongs to a device: set on the first launch
+    # of a process only, a launch on a second device lacks it.  Every call of
+    # cudaFuncSetAttribute belongs to a function that problem or batch creation runs
+    setters = {"configure_", "stencil_opt_in", "batch_cg_setup", "cg_grid_blocks"}
+    for f in sorted(os.listdir(CSRC)):
+        src = read(f)
+        if "cudaFuncSetAttribute" not in src:
+            continue
+        assert not re.search(r"call_once\([^;]*cudaFuncSetAttribute", src, re.S), f
+        for m in re.finditer(r"cudaFuncSetAttribute\(", src):
+            head = re.findall(r"^(?:static )?(?:inline )?[\w: ]+ \**(\w+)\([^;{]*\) \{", src[:m.start()],
+                              re.M)
+            assert any(head[-1].startswith(s) for s in setters), (f, head[-1])
