@@ -272,10 +272,14 @@ __device__ __forceinline__ void gram_small_body(long long n, int pa, int qb, lon
 // memory at a time.  Threads map onto the outputs with no padding beyond one row
 // and column, so no FMA is spent on entries outside the Gram (the 64-wide tile
 // would spend (64/p)^2 times the work at p = 16).  Up to 256 outputs: one per
-// thread.  Above, a 2 x 2 block per thread: four shared values for four FMAs
-// where one output per thread reads eight, which bound the kernel (two reads
-// per FMA); every output is the same row-ascending chain in both.  Measured, the
-// Grams of 24 batched jobs (N 20 to 38, p 4 to 32): 123 -> 71 us per launch.
+// thread.  Above, in FP32 a 2 x 2 block per thread: four shared values for four
+// FMAs where one output per thread reads eight, which bound the kernel (two reads
+// per FMA).  Measured, the Grams of 24 batched jobs (N 20 to 38, p 4 to 32):
+// 123 -> 71 us per launch.  FP64 keeps single outputs, every 256th to a thread: its
+// pipe is the bound, and 2 x 2 blocks leave warps idle (81 threads at p = 17).  One
+// step_gram call at 48^3, single against 2 x 2: p = 17 95 / 111 us, p = 20 112 / 134,
+// p = 29 199 / 233, p = 32 230 / 232; in FP32 at p = 29 63 / 48, p = 32 71 / 48.
+// Every output is the same row-ascending chain in all.
 constexpr int kMidPQ = 32, kMidRows = 32;
 static_assert(kMidRows * kMidPQ <= 4 * 256, "a stage is 4 values per thread of a 256-thread block");
 
@@ -291,13 +295,20 @@ __device__ __forceinline__ void gram_mid_body(long long n, int pa, int qb, long 
   long long r1 = r0 + rows_per;
   if (r1 > n) r1 = n;
   const int outs = pa * qb;
-  const bool wide = outs > 256;
+  const bool wide = sizeof(T) == 4 && outs > 256;
   const int tb = (qb + 1) / 2, ta = (pa + 1) / 2;
-  const bool work = wide ? (int)threadIdx.x < ta * tb : (int)threadIdx.x < outs;
-  // first output (row, column) of this thread
-  const int oa = !work ? 0 : wide ? 2 * ((int)threadIdx.x / tb) : (int)threadIdx.x / qb;
-  const int ob = !work ? 0 : wide ? 2 * ((int)threadIdx.x % tb) : (int)threadIdx.x % qb;
-  T acc[2][2] = {{0, 0}, {0, 0}};
+  const bool work = (int)threadIdx.x < (wide ? ta * tb : outs);
+  // this thread's outputs (row, column): a 2 x 2 block, or every 256th
+  int oa[4], ob[4];
+  bool own[4];
+  T acc[4] = {0, 0, 0, 0};
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int e = threadIdx.x + u * blockDim.x;
+    oa[u] = !work ? 0 : wide ? 2 * ((int)threadIdx.x / tb) + (u >> 1) : e / qb;
+    ob[u] = !work ? 0 : wide ? 2 * ((int)threadIdx.x % tb) + (u & 1) : e % qb;
+    own[u] = work && oa[u] < pa && ob[u] < qb;
+  }
   // the next stage's values travel in registers while this stage computes
   // (256 threads x 4 cover a stage of kMidRows x kMidPQ)
   T ra[4], rb[4];
@@ -323,31 +334,31 @@ __device__ __forceinline__ void gram_mid_body(long long n, int pa, int qb, long 
     __syncthreads();
     if (r + kMidRows < r1) fetch(r + kMidRows);
     if (!work) continue;
-    const T *as = As + oa, *bs = Bs + ob;
     if (!wide) {
-      T a = acc[0][0];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if (!own[u]) break;
+        T a = acc[u];
 #pragma unroll 8
-      for (int k = 0; k < rows; ++k) a = fma(as[k * pa], bs[k * qb], a);
-      acc[0][0] = a;
+        for (int k = 0; k < rows; ++k) a = fma(As[k * pa + oa[u]], Bs[k * qb + ob[u]], a);
+        acc[u] = a;
+      }
     } else {
+      const T *as = As + oa[0], *bs = Bs + ob[0];
 #pragma unroll 8
       for (int k = 0; k < rows; ++k) {
         const T a0 = as[k * pa], a1 = as[k * pa + 1], b0 = bs[k * qb], b1 = bs[k * qb + 1];
-        acc[0][0] = fma(a0, b0, acc[0][0]);
-        acc[0][1] = fma(a0, b1, acc[0][1]);
-        acc[1][0] = fma(a1, b0, acc[1][0]);
-        acc[1][1] = fma(a1, b1, acc[1][1]);
+        acc[0] = fma(a0, b0, acc[0]);
+        acc[1] = fma(a0, b1, acc[1]);
+        acc[2] = fma(a1, b0, acc[2]);
+        acc[3] = fma(a1, b1, acc[3]);
       }
     }
   }
-  if (!work) return;
   double *dst = part + (long long)chunk * outs;
 #pragma unroll
-  for (int i = 0; i < 2; ++i)
-#pragma unroll
-    for (int j = 0; j < 2; ++j)
-      if ((wide || (i == 0 && j == 0)) && oa + i < pa && ob + j < qb)
-        dst[(oa + i) * qb + ob + j] = (double)acc[i][j];
+  for (int u = 0; u < 4; ++u)
+    if (own[u]) dst[oa[u] * qb + ob[u]] = (double)acc[u];
 }
 
 template <typename T>
