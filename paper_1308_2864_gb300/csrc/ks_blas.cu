@@ -806,8 +806,9 @@ __global__ void __launch_bounds__(256) combine_kernel(long long n, int q, const 
 }
 
 // Narrow updates (q <= kNarrowQ): a thread takes 4 consecutive columns, the small
-// C matrices in shared memory, no padded arithmetic.  FP64, bound by its pipe:
-// one row per thread, A read from L1.  FP32: combine_rows_body.
+// C matrices in shared memory, no padded arithmetic.  One row per thread, A read
+// from L1 (combine_narrow_body): FP64, bound by its pipe, and FP32 launches that do
+// not fill the chip with threads.  The other FP32 ones: combine_rows_body.
 constexpr int kNarrowQ = 32;
 constexpr int kNarrowK = 2 * kNarrowQ;
 constexpr int kNarrowCols = 4;                     // output columns per thread
@@ -947,11 +948,6 @@ __device__ __forceinline__ void combine_narrow_body(
     long long n, int q, const T *__restrict__ A1, int k1, const double *__restrict__ C1,
     const T *__restrict__ A2, int k2, const double *__restrict__ C2, double alpha_d,
     double beta_d, const T *__restrict__ Bm, T *__restrict__ out, int vb, int vnb) {
-  if constexpr (sizeof(T) == 4) {
-    combine_rows_body(n, q, A1, k1, C1, A2, k2, C2, (float)alpha_d, (float)beta_d, Bm, out, vb,
-                      vnb);
-    return;
-  } else {
   __shared__ T Cs[2][kNarrowK * kNarrowQ];
   for (int e = threadIdx.x; e < k1 * q; e += blockDim.x) Cs[0][e] = (T)C1[e];
   if (A2)
@@ -996,16 +992,32 @@ __device__ __forceinline__ void combine_narrow_body(
       out[o] = v;
     }
   }
-  }
 }
 
-template <typename T>
+template <typename T, bool Rows>
 __global__ void __launch_bounds__(256) combine_narrow_kernel(
     long long n, int q, const T *__restrict__ A1, int k1, const double *__restrict__ C1,
     const T *__restrict__ A2, int k2, const double *__restrict__ C2, double alpha_d,
     double beta_d, const T *__restrict__ Bm, T *__restrict__ out) {
-  combine_narrow_body<T>(n, q, A1, k1, C1, A2, k2, C2, alpha_d, beta_d, Bm, out, blockIdx.x,
-                         gridDim.x);
+  if constexpr (Rows)
+    combine_rows_body(n, q, A1, k1, C1, A2, k2, C2, (float)alpha_d, (float)beta_d, Bm, out,
+                      blockIdx.x, gridDim.x);
+  else
+    combine_narrow_body<T>(n, q, A1, k1, C1, A2, k2, C2, alpha_d, beta_d, Bm, out, blockIdx.x,
+                           gridDim.x);
+}
+
+// Staged tiles of rows for an FP32 narrow update of one system (job tables always
+// take them: their jobs fill the chip together): from 16 columns on where the
+// one-row form's threads would fill the chip (2048 per SM), or where its chain over k
+// is longer than a stage.  Below, a tile of up to 1024 rows leaves most SMs without
+// one; on few columns the two are even, or the one-row form is ahead, which skips
+// what a ragged group of four pads.  step_combine_f32 with two blocks and Bm, one-row
+// against staged: 20^3, p = 5 25 / 33 us; 48^3, p = 15 36 / 38; 64^3, p = 9 37 / 46;
+// 80^3, p = 13 62 / 71; 48^3, p = 16 47 / 38; 64^3, p = 16 59 / 48, p = 32 158 / 94.
+static bool narrow_rows_applies(const Problem &P, int K, int q) {
+  const long long threads = (long long)P.n * ((q + kNarrowCols - 1) / kNarrowCols);
+  return (q >= 16 && threads >= 2048LL * P.sms) || K > kNrK;
 }
 
 // Tall-skinny FP32 update, q <= 64 output columns and K = k1 + k2 + k3 <= 192
@@ -1224,8 +1236,16 @@ ks_status launch_combine(Problem &P, const T *A1, int k1, const double *C1, cons
     {
       ProfScope ps_(P.stream, KP_COMBINE, 2.0 * P.n * q * (k1 + (A2 ? k2 : 0)),
                     (double)P.n * ((k1 + (A2 ? k2 : 0)) + q * (Bm ? 2 : 1)) * sizeof(T));
-      combine_narrow_kernel<T><<<(int)nb, 256, 0, P.stream>>>(P.n, q, A1, k1, C1, A2, k2, C2,
-                                                              alpha, beta, Bm, out);
+      bool rows = false;
+      if constexpr (sizeof(T) == 4) {
+        rows = narrow_rows_applies(P, k1 + (A2 ? k2 : 0), q);
+        if (rows)
+          combine_narrow_kernel<T, true><<<(int)nb, 256, 0, P.stream>>>(
+              P.n, q, A1, k1, C1, A2, k2, C2, alpha, beta, Bm, out);
+      }
+      if (!rows)
+        combine_narrow_kernel<T, false><<<(int)nb, 256, 0, P.stream>>>(
+            P.n, q, A1, k1, C1, A2, k2, C2, alpha, beta, Bm, out);
     }
     KS_CUDA_TRY(cudaGetLastError());
     return KS_OK;
@@ -1375,8 +1395,12 @@ __global__ void __launch_bounds__(256) combine_batch_kernel(const BJob *__restri
   const double *C1 = b.pp + (size_t)sl.c1 * len;
   const double *C2 = sl.c2 >= 0 ? b.pp + (size_t)sl.c2 * len : nullptr;
   if constexpr (Narrow) {
-    combine_narrow_body<T>(b.n, p, A1, p, C1, A2, p, C2, sl.alpha, sl.beta, Bm, out, vb,
-                           b.comb_nb);
+    if constexpr (sizeof(T) == 4)
+      combine_rows_body(b.n, p, A1, p, C1, A2, p, C2, (float)sl.alpha, (float)sl.beta, Bm, out,
+                        vb, b.comb_nb);
+    else
+      combine_narrow_body<T>(b.n, p, A1, p, C1, A2, p, C2, sl.alpha, sl.beta, Bm, out, vb,
+                             b.comb_nb);
   } else {
     const int ct = (p + kTile - 1) / kTile;
     if (sizeof(T) == 4)

@@ -53,3 +53,25 @@ def test_increment_form_of_32_orbitals(retraction):
     scale = sum(abs(v) for v in ev.parts.values())
     assert abs(r["E"] - ev.E) <= 1e-6 * scale
     assert ost.ortho_error(model, X.cpu().numpy()) < 1e-6
+
+
+@pytest.mark.parametrize("q", [12, 15, 16, 17, 26, 32])
+def test_narrow_update_forms(q):
+    # 48^3 rows fill the chip: staged tiles from 16 columns on, one row per thread
+    # below; at 12^3 one row per thread up to K = 32.  Both are one chain over k.
+    import paper_1308_2864_gb300 as ks
+    for N, blocks in ((12, 1), (12, 2), (48, 1), (48, 2)):
+        s = ki.small_system(N=N, L=7.0, natoms=2, p=q, Z=4.0, seed=4)
+        P = ks.Problem.from_system(s)
+        g = torch.Generator(device="cuda").manual_seed(q)
+        r = lambda *d: torch.randn(*d, generator=g, device="cuda", dtype=torch.float64)
+        A, Bm = [r(s.n, q).float() for _ in range(blocks)], r(s.n, q).float()
+        C = [r(q, q) for _ in range(blocks)]
+        two = (A[1], C[1]) if blocks == 2 else (None, None)
+        torch.cuda.synchronize()             # the problem has a stream of its own
+        got = P.step_combine_f32(A[0], C[0], *two, alpha=-0.5, beta=2.0, Bm=Bm).double()
+        want, bound = 2.0 * Bm.double(), 2.0 * Bm.double().abs()
+        for a, c in zip(A, C):
+            want = want - 0.5 * (a.double() @ c)
+            bound = bound + 0.5 * (a.double().abs() @ c.abs())
+        assert torch.all((got - want).abs() <= (blocks * q + 4) * 2.0**-23 * bound)
