@@ -417,9 +417,10 @@ __global__ void __launch_bounds__(256) gram_small_kernel(long long n, int pa, in
 // tile and runs alone on stages of kGaRows rows (a ring of kGaStages, cp.async
 // 16 bytes per copy, zero-filled past the last row and past pa, qb); lane
 // (ty, tx) of 8 x 4 owns columns 4 ty + 32 h of A and 4 tx + 16 j of B.  The
-// warps' tiles (chains of about 200 rows at 64^3) are added in pairs in FP32 (in
-// FP64 those 4096 x 8 adds per block took 17 us), the blocks' sums in FP64 in
-// block order.  One Gram at 64^3 x 64: 63 us for 4 x 4 per thread (34 TF/s), 56
+// warps' tiles (chains of about 200 rows at 64^3) are added in pairs in FP32 with
+// the error of every sum kept (two-sum, Knuth), so nothing of a tile is rounded
+// away: a partial is the sum and its error, 48 bits (in FP64 those 4096 x 8 adds
+// per block took 17 us).  The blocks' sums are added in FP64 in block order.  One Gram at 64^3 x 64: 63 us for 4 x 4 per thread (34 TF/s), 56
 // here (38); packed FMAs cost more in duplicating A than they save (65).
 constexpr int kGaStages = 3, kGaRows = 16, kGaWarps = 8;
 
@@ -433,7 +434,7 @@ constexpr size_t gram_wa_smem() {
 template <bool Dual>
 __global__ void __launch_bounds__(32 * kGaWarps, 1) gram2_wa_kernel(
     long long n, int pa, int qb, const float *__restrict__ A1, const float *__restrict__ B1,
-    const float *__restrict__ A2, const float *__restrict__ B2, float *__restrict__ part) {
+    const float *__restrict__ A2, const float *__restrict__ B2, float2 *__restrict__ part) {
   extern __shared__ __align__(16) float ga_smem[];
   constexpr int kStage = 2 * kGaRows * kTile;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, ty = lane >> 2, tx = lane & 3;
@@ -515,34 +516,46 @@ __global__ void __launch_bounds__(32 * kGaWarps, 1) gram2_wa_kernel(
           make_float4(acc[i][4 * j], acc[i][4 * j + 1], acc[i][4 * j + 2], acc[i][4 * j + 3]);
   __syncthreads();
   const int len = pa * qb;
-  float *dst = part + (long long)blockIdx.x * (Dual ? 2 : 1) * len;
+  float2 *dst = part + (long long)blockIdx.x * (Dual ? 2 : 1) * len;
   for (int e = threadIdx.x; e < (Dual ? 2 : 1) * len; e += 32 * kGaWarps) {
     const int which = e >= len ? 1 : 0, f = e - which * len, at = f / qb * kTile + f % qb;
     constexpr int kTiles = Dual ? kGaWarps / 2 : kGaWarps;
-    float v[kTiles];
+    float v[kTiles], lo = 0.f;
 #pragma unroll
     for (int s = 0; s < kTiles; ++s)
       v[s] = ga_smem[(size_t)(s * (Dual ? 2 : 1) + which) * kTile * kTile + at];
 #pragma unroll
     for (int o = kTiles / 2; o > 0; o >>= 1)
 #pragma unroll
-      for (int s = 0; s < o; ++s) v[s] += v[s + o];
-    dst[e] = v[0];
+      for (int s = 0; s < o; ++s) {
+        const float x = v[s], y = v[s + o], sum = __fadd_rn(x, y);
+        const float yy = __fsub_rn(sum, x);
+        lo += __fadd_rn(__fsub_rn(x, __fsub_rn(sum, yy)), __fsub_rn(y, yy));
+        v[s] = sum;
+      }
+    dst[e] = make_float2(v[0], isfinite(v[0]) ? lo : 0.f);
   }
 }
 
-// FP64 sums of the blocks' partials in block order: element e < len1 of each
-// goes to out1[e], the rest to out2[e - len1]; out32 (optional) gets every sum
-// rounded to FP32 at index e.
+// FP64 sums of the blocks' partials (sum and error) in block order: element e <
+// len1 of each goes to out1[e], the rest to out2[e - len1]; out32 (optional) gets
+// every sum rounded to FP32 at index e.  The errors, 2^-24 of the sums, are added in
+// FP32 first.
 __global__ void gram_reduce2_kernel(int chunks, long long len, long long len1,
-                                    const float *__restrict__ part, double *__restrict__ out1,
+                                    const float2 *__restrict__ part, double *__restrict__ out1,
                                     double *__restrict__ out2, float *__restrict__ out32) {
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long e = t >> 3;
   const int sub = (int)(t & 7);
   double acc = 0.0;
+  float lo = 0.f;
   if (e < len)
-    for (int c = sub; c < chunks; c += 8) acc += (double)part[(long long)c * len + e];
+    for (int c = sub; c < chunks; c += 8) {
+      const float2 v = part[(long long)c * len + e];
+      acc += (double)v.x;
+      lo += v.y;
+    }
+  acc += (double)lo;
   acc += __shfl_xor_sync(0xffffffffu, acc, 1);
   acc += __shfl_xor_sync(0xffffffffu, acc, 2);
   acc += __shfl_xor_sync(0xffffffffu, acc, 4);
@@ -571,10 +584,9 @@ static ks_status launch_gram2_wa(Problem &P, int pa, int qb, const float *A1, co
   long long blocks = P.sms;
   if (blocks > nst) blocks = nst;
   const long long len = (long long)pa * qb * (Dual ? 2 : 1);
-  // FP32 partials in the FP64 partial buffer
-  if ((size_t)blocks * len > 2 * P.partials_len)
+  if ((size_t)blocks * len > P.partials_len)
     return set_error(KS_EINVAL, "gram: partial buffer too small");
-  float *part = reinterpret_cast<float *>(P.partials);
+  float2 *part = reinterpret_cast<float2 *>(P.partials);
   {
     ProfScope ps_(P.stream, KP_GRAM, 2.0 * nv * pa * qb * (Dual ? 2 : 1),
                   (double)nv * (pa + qb + (Dual ? pa : 0)) * sizeof(float));
