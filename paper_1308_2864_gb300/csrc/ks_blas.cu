@@ -240,7 +240,14 @@ __device__ __forceinline__ void gram_small_body(long long n, int pa, int qb, lon
     }
   }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (pa <= 4 && qb <= 4) {
+  if (pa * qb == 1) {
+    // one value (the orbital-free model): five adds, not the 16 of the spread sum.  An
+    // FP64 add holds the SM's pipe for 16 clocks per warp, 32 of them share it
+    double v = (double)acc[0][0];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0) red[warp][0] = v;
+  } else if (pa <= 4 && qb <= 4) {
     double v[16];
 #pragma unroll
     for (int a = 0; a < 4; ++a)
