@@ -654,9 +654,12 @@ ks_status launch_gram(Problem &P, const T *A, int pa, const T *B, int qb, double
   const size_t need = (size_t)chunks * pa * qb;
   if (need > P.partials_len)
     return set_error(KS_EINVAL, "gram: partial buffer too small (%zu > %zu)", need, P.partials_len);
-  // few chunks of a small Gram are summed by the last block (a launch less);
-  // many take too long in one block
-  const bool tail = pa <= kSmallPQ && qb <= kSmallPQ && chunks <= 128;
+  // few chunks of a small Gram are summed by the last block (a launch less); many
+  // take too long in one block.  step_gram by a reduction launch against the last
+  // block: 20^3 (32 chunks) p = 2 33.5 / 32.8 us, p = 8 36.5 / 35.4; 28^3 (86) p = 4
+  // 34.2 / 33.4, p = 8 37.5 / 37.6; 32^3 (128) p = 1 30.0 / 33.6, p = 8 37.5 / 42.6;
+  // 48^3 (432) p = 1 34.6 / 46.6
+  const bool tail = pa <= kSmallPQ && qb <= kSmallPQ && chunks <= 96;
   {
     ProfScope ps_(P.stream, KP_GRAM, 2.0 * P.n * pa * qb, (double)P.n * (pa + qb) * sizeof(T));
     if (pa <= kSmallPQ && qb <= kSmallPQ)
