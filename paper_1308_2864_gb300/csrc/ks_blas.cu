@@ -28,8 +28,12 @@ __device__ __forceinline__ void cp_async_commit() {
 
 // Tensor cores for the FP32 phase when the products are wide enough for the
 // SIMT FP32 pipes to be the bound (use_tc = 1: from 256 columns; 2: always;
-// 0: never).  At p = 64 the SIMT kernels are as fast as the register-staged
-// tensor-core kernels, which do not yet overlap their loads deeply enough.
+// 0: never).  Below, the line is one of accuracy: three TF32 products leave an error
+// of 2e-7 of sum |a||c| (rms; SIMT 2.8e-8) in an update and 4e-8 (2e-9) in a Gram,
+// although they are the faster ones from 96 columns on.  64^3, update of two blocks /
+// Gram, SIMT against tensor cores: p = 64 138 / 86 against 251 / 186 us, p = 96
+// 460 / 267 against 310 / 188, p = 128 601 / 273 against 373 / 201, p = 256
+// 2234 / 942 against 835 / 385.
 static bool use_tensor_cores(const Problem &P, int a, int b) {
   if (P.use_tc == 0 || a <= 8 || b <= 8) return false;
   return P.use_tc == 2 || (a >= 256 && b >= 256);
@@ -473,7 +477,8 @@ __global__ void __launch_bounds__(32 * kGaWarps, 1) gram2_wa_kernel(
         src = M + row * w_ + c4;
         bytes = 16;
       }
-      cp_async16(smem_addr(dst + op * kGaRows * kTile + rr * kTile + c4), src, bytes);
+      const int di = op * kGaRows * kTile + rr * kTile + c4;
+      if (KS_IN(di + 3, kStage)) cp_async16(smem_addr(dst + di), src, bytes);
     }
   };
   float acc[8][16];
@@ -540,7 +545,9 @@ __global__ void __launch_bounds__(32 * kGaWarps, 1) gram2_wa_kernel(
         lo += __fadd_rn(__fsub_rn(x, __fsub_rn(sum, yy)), __fsub_rn(y, yy));
         v[s] = sum;
       }
-    dst[e] = make_float2(v[0], isfinite(v[0]) ? lo : 0.f);
+    if (KS_IN((long long)blockIdx.x * (Dual ? 2 : 1) * len + e,
+              (long long)gridDim.x * (Dual ? 2 : 1) * len))
+      dst[e] = make_float2(v[0], isfinite(v[0]) ? lo : 0.f);
   }
 }
 
@@ -1647,7 +1654,10 @@ __global__ void __launch_bounds__(32 * kWaWarps, 1) combine_wa_kernel(
   int istage = 0;                                       // K stage and tile of the next issue
   long long itile = first;
   int ibuf = 0;
-  // widths that are multiples of kWaK (q = 32 or 64): a stage lies in one operand
+  // widths that are multiples of kWaK (q = 32 or 64): a stage lies in one operand, so
+  // its copies share one base and one bound.  step_combine_f32 with Bm at 64^3, each copy
+  // looking for its operand against this: k = 64, q = 64 97 / 88 us, 64 + 64, 64 142 /
+  // 138, 96, 32 112 / 105; at 32^3 even
   const bool whole = k1 % kWaK == 0 && k12 % kWaK == 0 && K % kWaK == 0 && q % kWaK == 0;
   auto issue = [&]() {
     const int k0 = istage * kWaK;
@@ -1686,7 +1696,8 @@ __global__ void __launch_bounds__(32 * kWaWarps, 1) combine_wa_kernel(
           if (KS_IN(row * k3 + (k - k12) + 3, n * k3)) { src = A3 + row * k3 + (k - k12); bytes = 16; }
         }
       }
-      cp_async16(smem_addr(dst + rr * kWaLd + kq), src, bytes);
+      const int di = rr * kWaLd + kq;
+      if (KS_IN(di + 3, kWaRows * kWaLd)) cp_async16(smem_addr(dst + di), src, bytes);
     }
     if (++istage == ntot) {
       istage = 0;

@@ -23,8 +23,16 @@
 // passes.  What bounds a solve is the chain of phases: a barrier costs 2.5 to
 // 4 us, a transform phase its loads' latency, the update the FP64 pipe.
 // Measured, PCG with full transforms -> this form: warm solve at 64^3 172 ->
-// 104 us, at 105^3 519 -> 293 us; cold at 81^3 463 -> 177 us; 24^3 80 -> 63 us
-// (of which packed FMAs in the transforms' tiles 2 to 6 us).
+// 104 us, at 105^3 519 -> 293 us; cold at 24^3 80 -> 63 us (of which packed FMAs in
+// the transforms' tiles 2 to 6 us).  Cold at 81^3 463 -> 177 us, with a step fewer
+// by the same stopping rule: the second residual is below 1e-10 of ||b|| here (4e-11
+// to 7e-11) and was 1.04e-10 there, and the potential's error, which stops where the
+// residual does, goes from 3e-14 to 3e-13 .. 8e-13 with it.  Over 44 grids of 20^3 to
+// 161^3 and three densities each (relative error of the potential in the 2-norm) it
+// is 0.15 times PCG's in the geometric mean, at most 1.6e-11 against 7.4e-11, and
+// larger for 26 of 132, those that PCG gave a third step.
+// Tiled passes, cold: 129^3 1.99 -> 1.72 ms, 161^3 3.16 -> 2.70 ms, 200^3 6.16 ->
+// 5.22 ms.
 //
 // Each step's reductions are partial sums written per block and summed by
 // every block in the same order, so all blocks take identical branch

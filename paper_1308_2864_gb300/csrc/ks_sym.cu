@@ -16,8 +16,6 @@
 // 5.9 ms (one Gram of it left out, the other halved).  Below 9 columns the
 // one-thread-per-row kernels have no padding to save; above 128 the packed U
 // and a row tile no longer fit shared memory, and the full tiles stay.
-#include <mutex>
-
 #include "ks_device.cuh"
 
 namespace ks {
@@ -49,7 +47,7 @@ static SymPlan sym_plan(const Problem &P) {
   s.nsets = kSymThreads / s.tri;
   s.threads = (s.nsets * s.tri + 31) / 32 * 32;
   // about 2048 entries per operand and stage, a multiple of the sets (equal
-  // work) and even (16-byte copies at odd p too)
+  // work) rounded up to even (copies are of 16 bytes at even p, of 8 at odd p)
   int m = 2048 / (p * s.nsets);
   if (m < 1) m = 1;
   s.sk = s.nsets * m;

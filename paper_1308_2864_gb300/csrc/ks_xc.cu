@@ -49,7 +49,10 @@ __device__ __forceinline__ double inv_of(double x) {
 
 // ln x: x = 2^k m with m in [sqrt(1/2), sqrt(2)), and the area-tangent series
 // ln m = 2 (s + s^3/3 + s^5/5 + ...), s = (m - 1)/(m + 1), |s| <= 0.1716: the
-// terms through s^21 leave 2 s^23/23 < 3e-19.  -inf at 0: r_s of a density beyond
+// terms through s^21 leave 2 s^23/23 < 3e-19.  Its roundings leave 3.5 unit
+// roundoffs (the library's log about two); in v_xc, where the exchange term is tens
+// of times larger, nothing of it is left: within 5.0 unit roundoffs of 128-bit values
+// over rho = 1e-30 .. 1e12, against 7.7 with the library functions.  -inf at 0: r_s of a density beyond
 // the FP32 range, whose start of rho^(-1/3) is 0, must not pass for a number.
 __device__ __forceinline__ double ln_series(double x) {
   const long long bits = __double_as_longlong(x);
@@ -258,7 +261,9 @@ ks_status launch_potential(Problem &P, const double *rho, const double *vH, cons
                            double *veff, bool with_hartree, bool fp32_xc) {
   // at most two blocks per SM: a block ends in four FP64 sums, as much work for
   // the FP64 pipe as a third of a node per thread, and the last one sums all
-  // blocks' partials (1024 blocks of one node per thread took 53 us at 64^3)
+  // blocks' partials.  Up to eight blocks per SM against two: FP64 step_potential
+  // at 64^3 93 / 85 us, at 128^3 400 / 387, at 200^3 1388 / 1376, even below 48^3;
+  // the FP32 form in a minimisation, 64^3 53 / 43 us per launch, 96^3 121 / 108
   const int nb = std::min(reduce_blocks(P, P.n), 2 * P.sms);
   const double h3 = P.h * P.h * P.h;
   {
