@@ -1022,12 +1022,19 @@ ks_status launch_combine_tc(Problem &P, const float *A1, int k1, const double *C
                             const float *A2, int k2, const double *C2, double alpha, double beta,
                             const float *Bm, float *out, int q) {
   const int K = k1 + (A2 ? k2 : 0);
-  // 16-byte loads of A: every width a multiple of 4, aligned bases
-  const bool wide = k1 % 4 == 0 && (!A2 || k2 % 4 == 0) &&
+  const int ncol = (q + kTcN - 1) / kTcN;
+  // 16-byte loads of A: every width a multiple of 4, aligned bases.  Not where the
+  // 128-row tiles of the other kernel all run at once and K is short: with half as
+  // many tiles, each of twice the rows, the chip has less to do at a time.  One call
+  // of step_combine_f32 with two blocks and Bm, 128-row tiles against 256: 24^3 x 256
+  // (K = 512) 94 / 112 us, 20^3 x 320 105 / 121, 16^3 x 512 138 / 148, even from
+  // K = 1280 on; in two waves and more 28^3 x 256 151 / 112, 24^3 x 320 164 / 124
+  const bool one_wave = (P.n + kTcM - 1) / kTcM * (long long)ncol <= P.sms && K <= 1024;
+  const bool wide = !one_wave && k1 % 4 == 0 && (!A2 || k2 % 4 == 0) &&
                     reinterpret_cast<uintptr_t>(A1) % 16 == 0 &&
                     reinterpret_cast<uintptr_t>(A2) % 16 == 0;
   const int ks = wide ? kWK : kTcK;
-  const int stages = (K + ks - 1) / ks, ncol = (q + kTcN - 1) / kTcN;
+  const int stages = (K + ks - 1) / ks;
   const long long img_len = (long long)ncol * stages * 2 * kTcN * ks;
   if ((size_t)img_len > P.tc_img_len) return set_error(KS_EINVAL, "combine_tc: image too large");
   {

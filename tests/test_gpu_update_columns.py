@@ -75,3 +75,26 @@ def test_narrow_update_forms(q):
             want = want - 0.5 * (a.double() @ c)
             bound = bound + 0.5 * (a.double().abs() @ c.abs())
         assert torch.all((got - want).abs() <= (blocks * q + 4) * 2.0**-23 * bound)
+
+
+@pytest.mark.parametrize("N,k1,k2,q", [(28, 36, 36, 36), (28, 72, 4, 257), (29, 256, 256, 256),
+                                       (28, 300, 260, 300), (24, 256, 256, 256),
+                                       (10, 640, 640, 640), (9, 644, 640, 300)])
+def test_wide_update_tiles(N, k1, k2, q):
+    # 256-row tiles: grids of more than one wave of 128-row tiles, or K above 1024;
+    # 128-row tiles otherwise (24^3 x 256).  The bound of the general tensor-core test
+    import paper_1308_2864_gb300 as ks
+    s = ki.small_system(N=N, L=7.0, natoms=2, p=max(k1, k2, q), Z=4.0, seed=4)
+    P = ks.Problem.from_system(s)
+    P.set_tensor_cores(2)
+    g = torch.Generator(device="cuda").manual_seed(29)
+    r = lambda *d: torch.randn(*d, generator=g, device="cuda", dtype=torch.float64)
+    A1, A2, Bm, C1, C2 = (r(s.n, k1).float(), r(s.n, k2).float(), r(s.n, q).float(), r(k1, q),
+                          r(k2, q))
+    torch.cuda.synchronize()                 # the problem has a stream of its own
+    for bm, beta in ((None, 0.0), (Bm, 2.0)):
+        got = P.step_combine_f32(A1, C1, A2, C2, alpha=-0.5, beta=beta, Bm=bm).double()
+        want = -0.5 * (A1.double() @ C1 + A2.double() @ C2) + beta * Bm.double()
+        bound = (0.5 * (A1.double().abs() @ C1.abs() + A2.double().abs() @ C2.abs())
+                 + beta * Bm.double().abs())
+        assert torch.all((got - want).abs() <= 4e-6 * bound + 1e-12)
