@@ -466,8 +466,8 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
 // x 512, K = 1024, against 0.48 ms here, 240 TF/s of useful products: tensor pipe
 // active 63 %, shared-memory data pipe 75 %, issue slots 22 %.)  The MMA order per
 // accumulator is that kernel's, so the results are too.  It stays for operands
-// without 16-byte rows.  Every wait is bounded; a role that gives up sets the block's
-// abort flag, the others stop at their next poll (a warp by vote: its lanes may see
+// without 16-byte rows and for few rows (launch_combine_tc).  Every wait is bounded;
+// a role that gives up sets the block's abort flag, the others stop at their next poll (a warp by vote: its lanes may see
 // the flag at different polls, and what follows a wait is for whole warps), copies and
 // MMAs in flight get a bounded wait, and the block records KS_ETIMEOUT.
 constexpr int kWM = 256, kWK = 16, kWSlots = 3;
