@@ -346,9 +346,10 @@ __device__ __forceinline__ void gram_mid_body(long long n, int pa, int qb, long 
     if (r + kMidRows < r1) fetch(r + kMidRows);
     if (!work) continue;
     if (!wide) {
+      // (up to 256 outputs: the first only)
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        if (!own[u]) break;
+      for (int u = 0; u < (sizeof(T) == 8 ? 4 : 1); ++u) {
+        if (u > 0 && !own[u]) break;
         T a = acc[u];
 #pragma unroll 8
         for (int k = 0; k < rows; ++k) a = fma(As[k * pa + oa[u]], Bs[k * qb + ob[u]], a);
