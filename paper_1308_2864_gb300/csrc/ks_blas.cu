@@ -432,8 +432,9 @@ __global__ void __launch_bounds__(256) gram_small_kernel(long long n, int pa, in
 // warps' tiles (chains of about 200 rows at 64^3) are added in pairs in FP32 with
 // the error of every sum kept (two-sum, Knuth), so nothing of a tile is rounded
 // away: a partial is the sum and its error, 48 bits (in FP64 those 4096 x 8 adds
-// per block took 17 us).  The blocks' sums are added in FP64 in block order.  One Gram at 64^3 x 64: 63 us for 4 x 4 per thread (34 TF/s), 56
-// here (38); packed FMAs cost more in duplicating A than they save (65).
+// per block took 17 us).  The blocks' sums are added in FP64 in block order.  One
+// Gram at 64^3 x 64: 63 us for 4 x 4 per thread (34 TF/s), 56 here (38); packed FMAs
+// cost more in duplicating A than they save (65).
 constexpr int kGaStages = 3, kGaRows = 16, kGaWarps = 8;
 
 constexpr size_t gram_wa_smem() {
@@ -1602,9 +1603,10 @@ __device__ __forceinline__ void wa_half(long long n, int q, long long row0, int 
 // epilogue overlaps the others' products.  The epilogue's operand (Bm or
 // add2) follows the K stages through the ring as two more stages: read from
 // global memory in the epilogue, its 16 loads per lane waited one by one (one
-// stage where q <= kWaK).  A lane owns rows ty + 4 i (i < 8) and columns 4 tx .. + 3 and 32 + 4 tx .. + 3
-// (ty = lane / 8, tx = lane % 8).  The coefficient image (K x 64, zero padded)
-// is shared by the block's warps, and the FMAs are packed pairs of columns
+// stage where q <= kWaK).  A lane owns rows ty + 4 i (i < 8) and columns 4 tx .. + 3
+// and 32 + 4 tx .. + 3 (ty = lane / 8, tx = lane % 8).  The coefficient image (K x
+// 64, zero padded) is shared by the block's warps, and the FMAs are packed pairs of
+// columns
 // (f2_fma: the scalar outer product stops at 49 of 76 TF/s).  Update with Bm at
 // 64^3, K = 128: 134 us for the block-synchronous 8 x 4 form (32 TF/s), 107 us
 // here (40 TF/s); 16 x 8 per lane (8 warps) took 168 us.

@@ -1056,8 +1056,9 @@ __global__ void __launch_bounds__(kCgThreads) cg_b_it1(CgBatchView v) {
        k += (long long)nb * blockDim.x) {
     const int ix = (int)(k % N), iy = (int)((k / N) % N), iz = (int)(k / NN);
     double pk;
-    const double qk = t.cg_it == 0 ? stiff_apply<false>(s_vec, nullptr, 0.0, N, ix, iy, iz, a.c, &pk)
-                                   : stiff_apply<true>(s_vec, pold, t.beta, N, ix, iy, iz, a.c, &pk);
+    const double qk =
+        t.cg_it == 0 ? stiff_apply<false>(s_vec, nullptr, 0.0, N, ix, iy, iz, a.c, &pk)
+                     : stiff_apply<true>(s_vec, pold, t.beta, N, ix, iy, iz, a.c, &pk);
     pnew[k] = pk;
     a.q[k] = qk;
     pq_l = fma(pk, qk, pq_l);

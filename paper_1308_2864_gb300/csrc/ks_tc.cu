@@ -452,9 +452,10 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
 // whose rows allow 16-byte loads.  The MMAs bound it when nothing waits (three
 // TF32 products: 116 GFLOP of 48^3 x 512 are 0.36 ms at half the measured BF16
 // rate); next to them shared memory, which takes A's hi and lo parts and feeds the
-// MMAs, and L2, which delivers the coefficient image to every row tile.  So a block owns 256 rows x 256 columns, two 128-row accumulators that
-// share each coefficient stage (half the image traffic of 128-row tiles), and
-// K advances in stages of 16 through a ring of kWSlots slots:
+// MMAs, and L2, which delivers the coefficient image to every row tile.  So a block
+// owns 256 rows x 256 columns, two 128-row accumulators that share each coefficient
+// stage (half the image traffic of 128-row tiles), and K advances in stages of 16
+// through a ring of kWSlots slots:
 //   warps 0-7  load A two stages ahead in registers, split it into TF32 hi and
 //              lo (kmajor_offset_of<16>), then read the accumulators out;
 //   warp 8     (one thread) issues 2 K-steps x 2 row halves x (hi.hi + hi.lo +
@@ -467,9 +468,10 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
 // active 63 %, shared-memory data pipe 75 %, issue slots 22 %.)  The MMA order per
 // accumulator is that kernel's, so the results are too.  It stays for operands
 // without 16-byte rows and for few rows (launch_combine_tc).  Every wait is bounded;
-// a role that gives up sets the block's abort flag, the others stop at their next poll (a warp by vote: its lanes may see
-// the flag at different polls, and what follows a wait is for whole warps), copies and
-// MMAs in flight get a bounded wait, and the block records KS_ETIMEOUT.
+// a role that gives up sets the block's abort flag, the others stop at their next
+// poll (a warp by vote: its lanes may see the flag at different polls, and what
+// follows a wait is for whole warps), copies and MMAs in flight get a bounded wait,
+// and the block records KS_ETIMEOUT.
 constexpr int kWM = 256, kWK = 16, kWSlots = 3;
 constexpr int kWTile = 256 * kWK * 4;                       // 16 KiB: hi or lo of A or B
 constexpr int kWStage = 4 * kWTile;                         // A hi, A lo, B hi, B lo

@@ -52,8 +52,9 @@ __device__ __forceinline__ double inv_of(double x) {
 // terms through s^21 leave 2 s^23/23 < 3e-19.  Its roundings leave 3.5 unit
 // roundoffs (the library's log about two); in v_xc, where the exchange term is tens
 // of times larger, nothing of it is left: within 5.0 unit roundoffs of 128-bit values
-// over rho = 1e-30 .. 1e12, against 7.7 with the library functions.  -inf at 0: r_s of a density beyond
-// the FP32 range, whose start of rho^(-1/3) is 0, must not pass for a number.
+// over rho = 1e-30 .. 1e12, against 7.7 with the library functions.  -inf at 0: r_s
+// of a density beyond the FP32 range, whose start of rho^(-1/3) is 0, must not pass
+// for a number.
 __device__ __forceinline__ double ln_series(double x) {
   const long long bits = __double_as_longlong(x);
   // exponent of x / sqrt(1/2), by its high word (sqrt(1/2) = 0x3fe6a09e...)
